@@ -183,8 +183,9 @@ ssa_status ssa_set_lane_tier(const ssa_graph* g, int32_t on);
 /* Process-wide choice of the greedy kernel's launch shape (results never
  * depend on it): 0 (default) uses one thread-block cluster of 16 (or 8) blocks,
  * synchronised by the hardware cluster barrier, for solvers marked shared
- * (ssa_solver_set_shared) on pools of at most 2^26 entries, and a cooperative
- * grid of one block per SM otherwise; 1 always uses the cooperative grid; 2
+ * (ssa_solver_set_shared) on pools of at most 2^26 entries, a single block on
+ * pools of a few thousand entries and nodes, and a cooperative grid of one
+ * block per SM otherwise; 1 always uses the cooperative grid; 2
  * always a cluster.  Applies to launches after the call.  SSA_E_ARG for other
  * values. */
 ssa_status ssa_set_greedy_mode(int32_t mode);
@@ -231,7 +232,7 @@ typedef struct {
 enum {
   SSA_K_SAMPLE_WARP = 0,     /* RR sampler, warp-per-sample tier */
   SSA_K_SAMPLE_CTA = 1,      /* RR sampler, CTA-per-sample tier (large sets) */
-  SSA_K_INDEX = 2,           /* node -> set index build (count, scan, scatter) */
+  SSA_K_INDEX = 2,           /* counts per node of the pool's sets */
   SSA_K_GREEDY = 3,          /* Max-Coverage argmax + cover steps */
   SSA_K_STARE = 4,           /* Cov over R^c_t, Estimate-Inf first-T search */
   SSA_K_COUNT = 5
@@ -280,7 +281,7 @@ ssa_status ssa_solve(const ssa_graph* g, const ssa_params* p, ssa_result* out);
  * device memory free at creation). */
 ssa_status ssa_solver_create(const ssa_graph* g, void* stream, int64_t pool_bytes_cap, ssa_solver** out);
 ssa_status ssa_solver_solve(ssa_solver* s, const ssa_params* p, ssa_result* out);
-/* Run each round's device work after sampling -- the index of the new sets,
+/* Run each round's device work after sampling -- the counts of the new sets,
  * Max-Coverage and, for D-SSA, the hit-tested stare count over R^c_t
  * (Algorithms 2 and 4) -- as one CUDA graph instead of separate launches and
  * host waits (on = 1; 0 = separate launches, the default).  The graph of
@@ -316,13 +317,13 @@ ssa_status ssa_pool_info(const ssa_pool* p, int64_t* count, int64_t* entries, in
  * SSA_E_ARG if cap is too small (off is still filled). */
 ssa_status ssa_pool_export(const ssa_pool* p, int64_t first, int64_t count, int64_t* off,
                            int32_t* nodes, int64_t cap);
-/* Node -> set index over sets [0, N): cnt int32[n] (host) = #sets holding v. */
+/* Counts over sets [0, N): cnt int32[n] (host) = #sets holding v. */
 ssa_status ssa_pool_counts(ssa_pool* p, int64_t N, int32_t* cnt);
 /* Max-Coverage (Algorithm 2) over sets [0, N): k picks of largest marginal
  * gain, ties to the smallest id, seeds never re-picked.  seeds int32[k],
  * gains int64[k] (host); *cov = Cov_R(S).  1 <= k <= n; N <= 2^31 - 2
- * (SSA_E_ARG beyond).  All k picks run in one cooperative kernel; a wait at
- * its grid barriers gives up after a bounded number of polls (about a second
+ * (SSA_E_ARG beyond).  All k picks run in one kernel; a wait at its grid
+ * barriers gives up after a bounded number of polls (about a second
  * by default, see ssa_set_wait_polls): every block then returns and the call
  * reports SSA_E_TIMEOUT, leaving the CUDA context usable. */
 ssa_status ssa_max_coverage(ssa_pool* p, int64_t N, int32_t k, int32_t* seeds, int64_t* gains,

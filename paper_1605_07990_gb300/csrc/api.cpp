@@ -227,17 +227,23 @@ struct DevPool {
   int64_t byte_cap = 0;
 
   int64_t bytes_for(int64_t ents, int64_t sets) const { return ents * 12 + sets * 14; }
-  // entries range covering samples [a, b)
-  void entry_range(int64_t a, int64_t b, int64_t* e0, int64_t* e1) const {
+  // entries range covering samples [a, b); *whole: it holds no other samples
+  void entry_range(int64_t a, int64_t b, int64_t* e0, int64_t* e1, bool* whole) const {
     *e0 = 0;
     *e1 = entries;
+    int64_t from = 0, to = count;
     for (auto& p : bounds) {
-      if (p.first <= a) *e0 = p.second;
+      if (p.first <= a) {
+        *e0 = p.second;
+        from = p.first;
+      }
       if (p.first >= b) {
         *e1 = p.second;
+        to = p.first;
         break;
       }
     }
+    if (whole) *whole = from == a && to == b;
   }
   void release(cudaStream_t st) {
     dev_free(nodes, st);
@@ -626,37 +632,26 @@ std::mutex& coop_mutex() {
   return mu;
 }
 
-// Node -> set index and greedy buffers.  The pool only ever appends whole
-// batches, so the index is kept per batch: each batch is counted, scanned and
-// scattered once, its counts are added to a running total, and Max-Coverage
-// walks v*'s list in every batch.  A cut N inside a batch gets a temporary
-// filtered index for the partial batch.
+// Counts per node and greedy buffers.  The pool only ever appends, so counts are
+// kept as a running total over the sets [0, counted): later sets are counted
+// on top.
 struct Cover {
-  struct Batch {
-    int64_t j0, j1;          // sample ids [j0, j1)
-    int64_t* off = nullptr;  // n+1
-    int32_t* samp = nullptr; // entries of the batch
-    int64_t e0 = 0, e1 = 0;  // its pool entries
-    bool ready = false;      // kernels queued
-  };
   int64_t n = 0;
   int64_t n_pad = 0;
-  std::vector<Batch> batches;
-  Batch partial_batch;       // temporary, for a cut inside a batch
-  int32_t* cnt_total = nullptr;  // counts of the cached batches
-  int32_t* cnt_tmp = nullptr;    // one batch's counts
+  int64_t counted = 0;           // sets in cnt_total
+  int32_t* cnt_total = nullptr;  // counts of the sets [0, counted); padding 0
   int32_t* cnt = nullptr;        // working gains of the current Max-Coverage
-  unsigned long long* cur = nullptr;
-  void* scan_tmp = nullptr;
+  uint16_t* lid = nullptr;       // greedy: local ids of the candidates, then their mark bits; zero between launches
+  bool lid_dirty = true;
   uint8_t* covered = nullptr;
   int64_t covered_cap = 0;
   uint8_t* in_seed = nullptr;
-  unsigned long long* argmax = nullptr;  // greedy argmax slots (3, one 128-byte line apart)
-  unsigned int* sync = nullptr;
-  unsigned long long* chunk_q = nullptr;
+  unsigned char* ctl = nullptr;  // greedy control block
+  int32_t* cand = nullptr;       // 3 x GREEDY_CANDS: ids, list lengths, list offsets
+  unsigned int* ents = nullptr;  // greedy candidate lists
+  int64_t ents_cap = 0;
+  uint4* chunks = nullptr;
   int64_t chunk_cap = 0;
-  unsigned int* hist = nullptr;   // greedy gain histograms (2 x 4096) and cache counts (2), one buffer
-  int32_t* cache = nullptr;       // greedy candidate caches (2 x 8192)
   int32_t* d_seeds = nullptr;
   int32_t* d_gains = nullptr;
   int k_cap = 0;
@@ -673,61 +668,44 @@ struct Cover {
   int h_cap = 0;
   unsigned int* h_sync = nullptr;        // 128 words
   unsigned long long* h_count = nullptr;
-  int64_t total_e = 0;                   // entries of the sets the next greedy covers (greedy_prepare)
+  int64_t total_e = 0;                   // entries that hold the sets the next greedy covers (greedy_prepare)
   bool shared_gpu = false;               // the solve shares the GPU with others (greedy launch shape)
 
+  // 16-bit words of lid: n_pad ids (a multiple of 4: the 32-bit words behind stay aligned) and n_pad bits
+  size_t lid_words() const { return (size_t)n_pad + 2 * (size_t)((n_pad + 31) / 32); }
   ssa_status init(int64_t nn, Exec& X) {
     n = nn;
     n_pad = (n + 3) & ~int64_t(3);
     TRY(dev_alloc(&cnt_total, (size_t)n_pad, X.st));
-    TRY(dev_alloc(&cnt_tmp, (size_t)n_pad, X.st));
     TRY(dev_alloc(&cnt, (size_t)n_pad, X.st));
-    CU(cudaMemsetAsync(cnt_total, 0, sizeof(int32_t) * (size_t)n_pad, X.st));
-    TRY(dev_alloc(&cur, (size_t)n + 1, X.st));
+    TRY(dev_alloc(&lid, lid_words(), X.st));
+    lid_dirty = true;
+    TRY(reset(X));
     TRY(dev_alloc(&in_seed, (size_t)n_pad, X.st));
-    CU(cudaMallocAsync(&scan_tmp, scan_tmp_bytes(n), X.st));
-    TRY(dev_alloc(&argmax, 64 + 2 * 1024, X.st));
-    TRY(dev_alloc(&sync, 128, X.st));
-    TRY(dev_alloc(&hist, 2 * 4096 + 2, X.st));
-    TRY(dev_alloc(&cache, 2 * 8192, X.st));
+    TRY(dev_alloc(&ctl, GREEDY_CTL_BYTES, X.st));
+    TRY(dev_alloc(&cand, 3 * (size_t)GREEDY_CANDS, X.st));
     TRY(dev_alloc(&d_count, 1, X.st));
     TRY(dev_alloc(&d_first, 2, X.st));
     CU(cudaMallocHost(reinterpret_cast<void**>(&h_sync), sizeof(unsigned int) * 128));
     CU(cudaMallocHost(reinterpret_cast<void**>(&h_count), sizeof(unsigned long long)));
     return SSA_OK;
   }
-  // a new solve on kept workspaces: drop the previous solve's index
+  // a new solve on kept workspaces: drop the previous solve's counts
   ssa_status reset(Exec& X) {
-    drop_index(X.st);
+    counted = 0;
     CU(cudaMemsetAsync(cnt_total, 0, sizeof(int32_t) * (size_t)n_pad, X.st));
     return SSA_OK;
   }
-  void drop_index(cudaStream_t st) {
-    for (auto& b : batches) free_batch(b, st);
-    batches.clear();
-    free_batch(partial_batch, st);
-  }
-  void free_batch(Batch& b, cudaStream_t st) {
-    dev_free(b.off, st);
-    dev_free(b.samp, st);
-  }
   void release(cudaStream_t st) {
-    for (auto& b : batches) free_batch(b, st);
-    batches.clear();
-    free_batch(partial_batch, st);
     dev_free(cnt_total, st);
-    dev_free(cnt_tmp, st);
     dev_free(cnt, st);
-    dev_free(cur, st);
-    if (scan_tmp) cudaFreeAsync(scan_tmp, st);
-    scan_tmp = nullptr;
+    dev_free(lid, st);
     dev_free(covered, st);
     dev_free(in_seed, st);
-    dev_free(argmax, st);
-    dev_free(sync, st);
-    dev_free(chunk_q, st);
-    dev_free(hist, st);
-    dev_free(cache, st);
+    dev_free(ctl, st);
+    dev_free(cand, st);
+    dev_free(ents, st);
+    dev_free(chunks, st);
     dev_free(d_seeds, st);
     dev_free(d_gains, st);
     dev_free(d_count, st);
@@ -746,85 +724,21 @@ struct Cover {
     h_cap = 0;
   }
 
-  ssa_status index_alloc(Batch& B, Exec& X) {
-    TRY(dev_alloc(&B.off, (size_t)n + 1, X.st));
-    TRY(dev_alloc(&B.samp, (size_t)std::max<int64_t>(B.e1 - B.e0, 1), X.st));
-    return SSA_OK;
-  }
-  // index of the samples [B.j0, B.j1) whose entries lie in [B.e0, B.e1); counts land in cnt_tmp
-  ssa_status index_kernels(const DevPool& P, const Batch& B, bool filter, Exec& X) {
-    CU(cudaMemsetAsync(cnt_tmp, 0, sizeof(int32_t) * (size_t)n_pad, X.st));
-    CU(launch_count_nodes(P.nodes, filter ? P.samp : nullptr, B.e0, B.e1, B.j0, B.j1, cnt_tmp, X.st, X.num_sms));
-    int l = 0;
-    CU(launch_exclusive_scan(cnt_tmp, n, B.off, scan_tmp, X.st, &l));
-    // positions inside the batch's own sample array: offsets start at 0
-    CU(cudaMemcpyAsync(cur, B.off, sizeof(int64_t) * (size_t)(n + 1), cudaMemcpyDeviceToDevice, X.st));
-    CU(launch_scatter_index(P.nodes, P.samp, B.e0, B.e1, B.j0, B.j1, cur, B.samp, X.st, X.num_sms));
-    X.launches += 2 + l;
-    return SSA_OK;
-  }
-
-  // Buffers for the index of every whole pool batch below N not indexed yet.
-  // *whole: N lies on a batch boundary, so index_issue needs no temporary
-  // partial batch (and allocates nothing).
-  ssa_status index_prepare(const DevPool& P, int64_t N, bool* whole, Exec& X) {
-    free_batch(partial_batch, X.st);
-    if (!batches.empty() && batches.back().j1 > N) {
-      // a smaller cut than before (direct callers): start the cache over
-      for (auto& b : batches) free_batch(b, X.st);
-      batches.clear();
-      CU(cudaMemsetAsync(cnt_total, 0, sizeof(int32_t) * (size_t)n_pad, X.st));
-    }
-    for (size_t i = 1; i < P.bounds.size(); ++i) {
-      const int64_t j0 = P.bounds[i - 1].first, j1 = P.bounds[i].first;
-      if (j1 > N) break;
-      if (!batches.empty() && batches.back().j1 >= j1) continue;
-      if (batches.size() >= (size_t)GREEDY_MAX_LISTS - 1)
-        return fail(SSA_E_INTERNAL, "more than %d index batches", GREEDY_MAX_LISTS - 1);
-      Batch B;
-      B.j0 = j0;
-      B.j1 = j1;
-      B.e0 = P.bounds[i - 1].second;
-      B.e1 = P.bounds[i].second;
-      TRY(index_alloc(B, X));
-      batches.push_back(B);
-    }
-    *whole = (batches.empty() ? 0 : batches.back().j1) >= N;
-    return SSA_OK;
-  }
-
-  // Queue the index kernels of the batches index_prepare added (each batch is
-  // counted, scanned and scattered once) and, for a cut inside a batch, of a
-  // temporary partial one.  Leaves the counts of [0, N) in `cnt`.
-  ssa_status index_issue(const DevPool& P, int64_t N, Exec& X) {
+  // Queue the counts of the sets [counted, N); cnt_total then holds those of
+  // [0, N).  Device work only.
+  ssa_status count_issue(const DevPool& P, int64_t N, Exec& X) {
     int h = X.begin(SSA_K_INDEX);
-    for (auto& B : batches) {
-      if (B.ready) continue;
-      TRY(index_kernels(P, B, false, X));
-      CU(launch_add_counts(cnt_total, cnt_tmp, n, X.st, X.num_sms));
+    if (counted > N) TRY(reset(X));  // a smaller cut than before (direct callers): start over
+    if (counted < N) {
+      int64_t e0 = 0, e1 = 0;
+      bool whole = false;
+      P.entry_range(counted, N, &e0, &e1, &whole);
+      CU(launch_count_nodes(P.nodes, whole ? nullptr : P.samp, e0, e1, counted, N, cnt_total, X.st, X.num_sms));
       X.launches += 1;
-      B.ready = true;
-    }
-    CU(cudaMemcpyAsync(cnt, cnt_total, sizeof(int32_t) * (size_t)n_pad, cudaMemcpyDeviceToDevice, X.st));
-    const int64_t covered_to = batches.empty() ? 0 : batches.back().j1;
-    if (covered_to < N) {
-      partial_batch.j0 = covered_to;
-      partial_batch.j1 = N;
-      P.entry_range(covered_to, N, &partial_batch.e0, &partial_batch.e1);
-      TRY(index_alloc(partial_batch, X));
-      TRY(index_kernels(P, partial_batch, true, X));
-      CU(launch_add_counts(cnt, cnt_tmp, n, X.st, X.num_sms));
-      X.launches += 1;
+      counted = N;
     }
     X.end(h);
     return SSA_OK;
-  }
-
-  // Make the index cover the sets [0, N).
-  ssa_status build_index(const DevPool& P, int64_t N, Exec& X) {
-    bool whole = false;
-    TRY(index_prepare(P, N, &whole, X));
-    return index_issue(P, N, X);
   }
 
   // Max-Coverage (Algorithm 2) over sets [0, N) in three parts, so that the
@@ -852,58 +766,78 @@ struct Cover {
       h_cap = k;
     }
     TRY(dev_grow(&covered, &covered_cap, std::max<int64_t>(N, 1), 0, X.st));
-    // entries of sets [0, N), an upper bound when N cuts a batch; queued
-    // decrement chunks of one pick: a set longer than 2048 entries queues
-    // ceil(len / 2048) < len / 1024 chunks
+    // the entries up to the end of the batch that holds set N - 1
     int64_t e0 = 0, e1 = 0;
-    P.entry_range(0, N, &e0, &e1);
-    total_e = e1 - e0;
-    TRY(dev_grow(&chunk_q, &chunk_cap, e1 / 1024 + 1, 0, X.st));
+    P.entry_range(0, N, &e0, &e1, nullptr);
+    total_e = e1;
+    // Candidate lists: entries for every member while that is little, else for
+    // the most frequent nodes (a candidate has at most N); 16-byte chunks for
+    // every member of the sets left after the first pick, at most 512 MB (more
+    // than fits makes the kernel cover the best node's sets first).
+    ents_now = std::min<int64_t>(std::min<int64_t>(total_e, std::max<int64_t>(2 * N, int64_t(1) << 25)),
+                                 INT32_MAX - 4096);
+    TRY(dev_grow(&ents, &ents_cap, ents_now + GREEDY_ENTS_SPARE, 0, X.st));
+    chunks_now = std::min<int64_t>((total_e + 19 * N) / 8 + 1, int64_t(1) << 25);
+    // behind the chunks: a 16-byte record per 256 members of a long set (more
+    // than 256 members, so at least 16 chunks a record)
+    TRY(dev_grow(&chunks, &chunk_cap, chunks_now + GREEDY_CHUNKS_SPARE + chunks_now / 16 + 1, 0, X.st));
+    if (lid_dirty) {
+      CU(cudaMemsetAsync(lid, 0, sizeof(uint16_t) * lid_words(), X.st));
+      lid_dirty = false;
+    }
     return SSA_OK;
   }
+  int64_t ents_now = 0, chunks_now = 0;  // what the next greedy may use of them
   ssa_status greedy_issue(const DevPool& P, int64_t N, int k, Exec& X) {
     int h = X.begin(SSA_K_GREEDY);
     CU(cudaMemsetAsync(covered, 0, (size_t)std::max<int64_t>(N, 1), X.st));
-    CU(cudaMemsetAsync(sync, 0, sizeof(unsigned int) * 128, X.st));
-    CU(cudaMemsetAsync(hist, 0, sizeof(unsigned int) * (2 * 4096 + 2), X.st));
-    CU(cudaMemsetAsync(argmax, 0, sizeof(unsigned long long) * (64 + 2 * 1024), X.st));
-    // padding nodes can never be picked
-    if (n_pad > n) CU(cudaMemsetAsync(cnt + n, 0xC0, sizeof(int32_t) * (size_t)(n_pad - n), X.st));
+    CU(cudaMemsetAsync(ctl, 0, GREEDY_CTL_BYTES, X.st));
     GreedyJob J{};
+    J.cnt0 = cnt_total;
     J.cnt = cnt;
+    J.n = n;
     J.n_pad = n_pad;
-    J.nlists = 0;
-    for (auto& b : batches) J.lists[J.nlists++] = InvList{b.off, b.samp};
-    if (partial_batch.off) J.lists[J.nlists++] = InvList{partial_batch.off, partial_batch.samp};
     J.pool_nodes = P.nodes;
+    J.pool_samp = P.samp;
     J.set_start = P.set_start;
     J.set_len = P.set_len;
+    J.total_entries = (unsigned long long)total_e;
+    J.n_sets = N;
+    J.bulk_first = J.total_entries > GREEDY_BULK_ENTRIES ? 1 : 0;
     J.covered = covered;
     J.seeds = d_seeds;
     J.gains = d_gains;
     J.k = k;
-    J.argmax = argmax;
-    J.n_sets = N;
-    J.total_entries = (unsigned long long)total_e;
-    J.sync = sync;
-    J.chunk_q = chunk_q;
-    J.chunk_cap = chunk_cap;
-    J.hist = hist;
-    J.cache = cache;
-    J.cache_n = hist + 2 * 4096;
+    J.sync = reinterpret_cast<unsigned int*>(ctl);
+    J.argmax = reinterpret_cast<unsigned long long*>(ctl + GREEDY_CTL_ARGMAX);
+    J.nchunk = reinterpret_cast<unsigned long long*>(ctl + GREEDY_CTL_NCHUNK);
+    J.ncand = reinterpret_cast<unsigned int*>(ctl + GREEDY_CTL_NCAND);
+    J.hist = reinterpret_cast<unsigned int*>(ctl + GREEDY_CTL_HIST);
+    J.blk = reinterpret_cast<unsigned int*>(ctl + GREEDY_CTL_BLK);
+    J.lid = lid;
+    J.mark = reinterpret_cast<unsigned int*>(lid + n_pad);
+    J.cand_id = cand;
+    J.cand_len = cand + GREEDY_CANDS;
+    J.cand_off = reinterpret_cast<unsigned int*>(cand + 2 * GREEDY_CANDS);
+    J.ents = ents;
+    J.ents_cap = ents_now;
+    J.chunks = chunks;
+    J.chunk_cap = (unsigned long long)chunks_now;
+    J.tasks = chunks + chunks_now + GREEDY_CHUNKS_SPARE;
     J.wait_polls = greedy_wait_polls();
-    int blocks = 0;
-    CU(launch_greedy(J, X.st, X.num_sms, &blocks, shared_gpu));
+    CU(launch_greedy(J, X.st, X.num_sms, shared_gpu));
     X.end(h);
     X.launches += 1;
     CU(cudaMemcpyAsync(h_seeds, d_seeds, sizeof(int32_t) * (size_t)k, cudaMemcpyDeviceToHost, X.st));
     CU(cudaMemcpyAsync(h_gains, d_gains, sizeof(int32_t) * (size_t)k, cudaMemcpyDeviceToHost, X.st));
-    CU(cudaMemcpyAsync(h_sync, sync, sizeof(unsigned int) * 128, cudaMemcpyDeviceToHost, X.st));
+    CU(cudaMemcpyAsync(h_sync, ctl, sizeof(unsigned int) * 128, cudaMemcpyDeviceToHost, X.st));
     return SSA_OK;
   }
   ssa_status greedy_finish(int k, int32_t* seeds, int64_t* gains, int64_t* cov) {
-    if (h_sync[64] == 2u) return fail(SSA_E_INTERNAL, "greedy decrement queue overflow");
-    if (h_sync[64]) return fail(SSA_E_TIMEOUT, "greedy grid barrier timed out");
+    if (h_sync[64]) {
+      lid_dirty = true;  // the kernel left in the middle of a session
+      return fail(SSA_E_TIMEOUT, "greedy grid barrier timed out");
+    }
     int64_t c = 0;
     for (int i = 0; i < k; ++i) {
       seeds[i] = h_seeds[i];
@@ -916,7 +850,7 @@ struct Cover {
   // Max-Coverage (Algorithm 2) over sets [0, N): seeds/gains to host.
   ssa_status greedy(const DevPool& P, int64_t N, int k, int32_t* seeds, int64_t* gains, int64_t* cov, Exec& X) {
     TRY(greedy_prepare(P, N, k, X));
-    TRY(build_index(P, N, X));
+    TRY(count_issue(P, N, X));
     {
       std::lock_guard<std::mutex> coop_lock(coop_mutex());
       TRY(greedy_issue(P, N, k, X));
@@ -933,7 +867,7 @@ struct Cover {
       return SSA_OK;
     }
     int64_t e0, e1;
-    P.entry_range(a, b, &e0, &e1);
+    P.entry_range(a, b, &e0, &e1, nullptr);
     TRY(dev_grow(&hitc, &hitc_cap, cnt_sets, 0, X.st));
     int h = X.begin(SSA_K_STARE);
     CU(cudaMemsetAsync(hitc, 0, (size_t)cnt_sets, X.st));
@@ -1262,21 +1196,19 @@ ssa_status solve_impl(ssa_solver* sv, const ssa_params* p, ssa_result* out) {
   int64_t used = 0;  // SSA: sets of the last round (the pool may hold more, sampled ahead)
   double influence = 0.0;
   const bool graphs = sv->use_graphs && !X.timing;
-  // Max-Coverage over the whole batches [0, N), and for D-SSA the stare count
+  // Max-Coverage over the sets [0, N), and for D-SSA the stare count
   // over the hit-tested check half [N, 2N): as one CUDA graph when enabled
   auto greedy_round = [&](int64_t N, int64_t* cov, int64_t* c) -> ssa_status {
-    bool whole = false;
     TRY(C.greedy_prepare(pool, N, k, X));
-    TRY(C.index_prepare(pool, N, &whole, X));
     if (c) TRY(S.hits_prepare(N, X));
-    if (graphs && whole) {
+    if (graphs) {
       TRY(run_graph(sv, (size_t)(dssa ? 64 : 0) + (size_t)t, [&]() -> ssa_status {
-        TRY(C.index_issue(pool, N, X));
+        TRY(C.count_issue(pool, N, X));
         TRY(C.greedy_issue(pool, N, k, X));
         return c ? stare_issue(S, C, p->seed, 0, N, N, C.d_seeds, k, X) : SSA_OK;
       }));
     } else {
-      TRY(C.index_issue(pool, N, X));
+      TRY(C.count_issue(pool, N, X));
       {
         std::lock_guard<std::mutex> lock(coop_mutex());
         TRY(C.greedy_issue(pool, N, k, X));
@@ -1427,10 +1359,8 @@ ssa_status solve_impl(ssa_solver* sv, const ssa_params* p, ssa_result* out) {
   } else {
     X.collect(nullptr);
   }
-  // the RR pool and this solve's index go back to the device's memory pool;
-  // the fixed-size scratch stays with the solver
+  // the RR pool goes back to the device's memory pool; the scratch stays with the solver
   pool.release(X.st);
-  if (sv->c_ready) C.drop_index(X.st);
   if (sv->s_ready[p->model]) dev_free(S.bprefix, X.st);
   cudaStreamSynchronize(X.st);
   out->seconds = now_s() - t0;
@@ -1871,8 +1801,8 @@ ssa_status ssa_pool_export(const ssa_pool* pc, int64_t first, int64_t count, int
 ssa_status ssa_pool_counts(ssa_pool* p, int64_t N, int32_t* cnt) {
   if (!p || !cnt) return fail(SSA_E_ARG, "null pool or output");
   if (N < 0 || N > p->P.count) return fail(SSA_E_ARG, "N outside the pool");
-  TRY(p->C.build_index(p->P, N, p->X));
-  CU(cudaMemcpyAsync(cnt, p->C.cnt, sizeof(int32_t) * (size_t)p->g->n, cudaMemcpyDeviceToHost, p->X.st));
+  TRY(p->C.count_issue(p->P, N, p->X));
+  CU(cudaMemcpyAsync(cnt, p->C.cnt_total, sizeof(int32_t) * (size_t)p->g->n, cudaMemcpyDeviceToHost, p->X.st));
   CU(cudaStreamSynchronize(p->X.st));
   return SSA_OK;
 }

@@ -1,14 +1,12 @@
-// RR pool index, greedy Max-Coverage (Algorithm 2), coverage checks (Eq. 1)
+// RR pool counts, greedy Max-Coverage (Algorithm 2), coverage checks (Eq. 1)
 // and the Estimate-Inf first-T search (Algorithm 3) on sm_103a.
 //
-// Index: cnt[v] = number of sets holding v by a counting pass over the flat
-// (node, sample) entries, exclusive scan into inv_off, scatter of sample ids
-// into inv_samp (order inside a list is irrelevant: each step only needs the
-// set of samples holding the picked node).
-// Greedy: one persistent cooperative kernel for all k picks; a pick is the
-// maximum packed key (gain+1)<<32 | ~v (largest gain, then smallest id; picked
-// nodes keyed to 0), then warps decrement the gains of the members of each
-// newly covered set.
+// Counts: cnt[v] = number of sets holding v, one pass over the flat (node,
+// sample) entries; sets added later are counted on top.
+// Greedy: one persistent kernel for all k picks.  Gains only fall, so the
+// nodes of the largest counts hold the next picks; their sets alone are laid
+// out per pick (candidate lists) and one block then picks out of its own
+// shared memory (see k_greedy).
 #include <atomic>
 #include <mutex>
 
@@ -23,7 +21,7 @@ namespace {
 constexpr int TPB = 256;
 
 // samp == nullptr: every entry in [e0, e1) counts; else only samples in [jlo, jhi)
-// Index build.  Hubs appear in a large share of the sets, so the lanes of a
+// Hubs appear in a large share of the sets, so the lanes of a
 // warp that hold the same node are grouped (labeled_partition) and one of
 // them issues the group's atomic: one atomic per distinct node per warp
 // instead of one per entry on the hub's counter.
@@ -38,22 +36,6 @@ __global__ void k_count_nodes(const int32_t* __restrict__ nodes, const int32_t* 
     const int32_t v = nodes[q];
     const cg::coalesced_group same = cg::labeled_partition(cg::coalesced_threads(), v);
     if (same.thread_rank() == 0) atomicAdd(cnt + v, (int)same.size());
-  }
-}
-
-__global__ void k_scatter_index(const int32_t* __restrict__ nodes, const int32_t* __restrict__ samp, int64_t e0,
-                                int64_t e1, int64_t jlo, int64_t jhi, unsigned long long* cur, int32_t* inv_samp) {
-  namespace cg = cooperative_groups;
-  for (int64_t q = e0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < e1;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t s = samp[q];
-    if (s < jlo || s >= jhi) continue;
-    const int32_t v = nodes[q];
-    const cg::coalesced_group same = cg::labeled_partition(cg::coalesced_threads(), v);
-    unsigned long long pos = 0;
-    if (same.thread_rank() == 0) pos = atomicAdd(cur + v, (unsigned long long)same.size());
-    pos = same.shfl(pos, 0) + same.thread_rank();
-    inv_samp[pos] = s;
   }
 }
 
@@ -86,63 +68,15 @@ __device__ __forceinline__ T block_exclusive_scan(T x, T* s_warp, T* total) {
   return r;
 }
 
-constexpr int SCAN_TILE = 4096;  // 1024 threads x 4
-
-__global__ void __launch_bounds__(1024) k_tile_sums(const int32_t* in, int64_t n, long long* part) {
-  __shared__ long long s_w[32];
-  __shared__ long long s_tot;
-  const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
-  long long sum = 0;
-  for (int i = threadIdx.x; i < SCAN_TILE; i += blockDim.x)
-    if (base + i < n) sum += in[base + i];
-  block_exclusive_scan<long long>(sum, s_w, &s_tot);
-  if (threadIdx.x == 0) part[blockIdx.x] = s_tot;
-}
-
-__global__ void __launch_bounds__(1024) k_scan_parts(long long* part, int64_t tiles) {
-  __shared__ long long s_w[32];
-  __shared__ long long s_tot;
-  long long carry = 0;
-  for (int64_t b = 0; b < tiles; b += blockDim.x) {
-    const int64_t i = b + threadIdx.x;
-    const long long x = i < tiles ? part[i] : 0;
-    const long long ex = block_exclusive_scan<long long>(x, s_w, &s_tot);
-    if (i < tiles) part[i] = carry + ex;
-    carry += s_tot;
-    __syncthreads();
-  }
-}
-
-__global__ void __launch_bounds__(1024) k_tile_scan(const int32_t* in, int64_t n, const long long* part,
-                                                    int64_t* out) {
-  __shared__ long long s_w[32];
-  __shared__ long long s_tot;
-  const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * 4;
-  long long v[4], loc = 0;
-#pragma unroll
-  for (int t = 0; t < 4; ++t) {
-    v[t] = (base + t < n) ? in[base + t] : 0;
-    loc += v[t];
-  }
-  long long ex = block_exclusive_scan<long long>(loc, s_w, &s_tot) + part[blockIdx.x];
-#pragma unroll
-  for (int t = 0; t < 4; ++t) {
-    if (base + t < n) out[base + t] = ex;
-    ex += v[t];
-  }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = part[blockIdx.x] + s_tot;
-}
-
 // ---- greedy ----
 
-// maximum (or sum) over the block of x, in every thread
-template <bool SUM>
-__device__ __forceinline__ unsigned long long block_reduce(unsigned long long x, unsigned long long* s) {
+// maximum over the block of x, in every thread
+__device__ __forceinline__ unsigned long long block_max(unsigned long long x, unsigned long long* s) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
   for (int d = 16; d; d >>= 1) {
     const unsigned long long t = __shfl_xor_sync(FULL_MASK, x, d);
-    x = SUM ? x + t : (t > x ? t : x);
+    x = t > x ? t : x;
   }
   if (lane == 0) s[wid] = x;
   __syncthreads();
@@ -151,7 +85,7 @@ __device__ __forceinline__ unsigned long long block_reduce(unsigned long long x,
 #pragma unroll
     for (int d = 16; d; d >>= 1) {
       const unsigned long long t = __shfl_xor_sync(FULL_MASK, x, d);
-      x = SUM ? x + t : (t > x ? t : x);
+      x = t > x ? t : x;
     }
     if (lane == 0) s[0] = x;
   }
@@ -160,23 +94,17 @@ __device__ __forceinline__ unsigned long long block_reduce(unsigned long long x,
   __syncthreads();
   return x;
 }
-__device__ __forceinline__ unsigned long long block_max(unsigned long long x, unsigned long long* s) {
-  return block_reduce<false>(x, s);
-}
 
-// sync layout: arrival count, release word and timeout flag on separate
+// sync layout: arrival count, release word and error flag on separate
 // 128-byte lines so that polling does not contend with the arrivals.
-constexpr int SYNC_COUNT = 0, SYNC_GEN = 32, SYNC_ERR = 64, SYNC_CHUNKS = 96;
-constexpr int DEC_CHUNK = 2048;    // covered sets longer than this are decremented in chunks by all warps
-constexpr int CACHE_MAX = 8192;    // greedy candidate cache entries
-constexpr int ARGMAX_STRIDE = 16;  // argmax slots one 128-byte line apart
-constexpr int HBINS = 4096;        // gain histogram: gain g >= floor counts in bin min(g - floor, HBINS - 1)
-constexpr unsigned long long PENDING = 1ull << 62;  // barrier payload flag: decrement chunks are queued
-constexpr unsigned long long RECOUNT = 1ull << 61;  // with PENDING: recount the gains instead of draining
-// per-block entry tallies (64-bit slots after the argmax slots): entries of
-// all sets the block covered so far, and entries it queued in the last pick
-// that queued any
-constexpr int ACC_DONE = 64, ACC_QUEUED = 64 + 1024;
+constexpr int SYNC_COUNT = 0, SYNC_GEN = 32, SYNC_ERR = 64;
+constexpr int ARGMAX_STRIDE = 16;  // 64-bit words: argmax slots one 128-byte line apart
+constexpr int GCANDS = GREEDY_CANDS;  // candidates of one session: their gains, ids and list offsets fill 192 KB
+constexpr int GBITS = 14;          // a candidate's key: gain above, GCANDS - 1 - local id in the low GBITS
+constexpr int GMAX = 1 << (32 - GBITS);
+constexpr int GBINS = 1024;        // histogram bins
+constexpr int GHISTS = 4;          // histograms in turn, so that one is cleared while another fills
+constexpr int GLONG = 256;         // members of a set beyond which its list is made by several warps
 
 // Grid barrier for a cooperative launch.  The last block to arrive runs f()
 // (all its threads; f sees every block's writes from before the barrier) and
@@ -244,6 +172,12 @@ template <bool CLUSTER, class F>
 __device__ __forceinline__ bool greedy_barrier(const GreedyJob& J, unsigned int* phase, F&& f,
                                                unsigned long long& info) {
   if constexpr (!CLUSTER) {
+    if (gridDim.x == 1) {  // a single block needs no waits
+      __syncthreads();
+      info = f();
+      __syncthreads();
+      return true;
+    }
     return grid_barrier(J.sync, phase, J.wait_polls, f, info);
   } else {
     namespace cg = cooperative_groups;
@@ -261,9 +195,8 @@ __device__ __forceinline__ bool greedy_barrier(const GreedyJob& J, unsigned int*
   }
 }
 
-// Packed argmax key: larger gain first, then smaller id; picked nodes (negative
-// gain) key to 0.  With gains below 2^31 - 1 and ids below 2^31, keys stay
-// below 2^62, under the barrier payload's PENDING flag.
+// Packed key: larger gain first, then smaller id; picked nodes (negative gain)
+// key to 0.  With gains below 2^31 - 1 and ids below 2^31, keys stay below 2^62.
 __device__ __forceinline__ unsigned long long gain_key(int32_t c, uint32_t v) {
   return c < 0 ? 0ull : (((unsigned long long)(uint32_t)(c + 1)) << 31) | (unsigned long long)(0x7FFFFFFFu - v);
 }
@@ -271,377 +204,630 @@ __device__ __forceinline__ int32_t key_node(unsigned long long key) {
   return (int32_t)(0x7FFFFFFFu - (uint32_t)(key & 0x7FFFFFFFull));
 }
 __device__ __forceinline__ int32_t key_gain(unsigned long long key) { return (int32_t)(key >> 31) - 1; }
+// the smallest key of gain g (any id)
+__device__ __forceinline__ unsigned long long gain_floor_key(int32_t g) {
+  return ((unsigned long long)(uint32_t)(g + 1)) << 31;
+}
 
-// gains of the `len` members at mem lose one each (a warp, lanes striped)
-__device__ __forceinline__ void decrement_members(int32_t* cnt, const int32_t* mem, int32_t len, int lane) {
-  int t = lane;
-  for (; t + 96 < len; t += 128) {  // four independent loads in flight per lane
-    const int32_t a = __ldg(mem + t), b = __ldg(mem + t + 32), c = __ldg(mem + t + 64), d = __ldg(mem + t + 96);
-    atomicSub(cnt + a, 1);
-    atomicSub(cnt + b, 1);
-    atomicSub(cnt + c, 1);
-    atomicSub(cnt + d, 1);
+// Histogram bin of a gain: exact below 64, then 32 bins per octave.
+__device__ __forceinline__ int gain_bin(int32_t g) {
+  if (g < 64) return g;
+  const int e = 31 - __clz(g);
+  return 64 + (e - 6) * 32 + ((g >> (e - 5)) & 31);
+}
+// smallest gain of a bin (2^31 - 1 past the last gain)
+__device__ __forceinline__ int32_t bin_gain(int b) {
+  if (b < 64) return b;
+  const int e = 6 + (b - 64) / 32;
+  if (e > 30) return 0x7FFFFFFF;
+  return (int32_t)((32u + (uint32_t)(b & 31)) << (e - 5));
+}
+
+// Sets [0, n_sets) not covered yet, cut into runs of `bs` per warp; each warp
+// deals the members of its run's sets to its lanes 32 at a time whatever the
+// sets' sizes (median 1, largest 10^4), four rounds in flight.
+//   begin(j, start, len): the lane holds set j (len 0: none; it may be set to
+//     0 to leave the set out); once per run
+//   item(node, owner, base, excl, incl): in round t of four the lane holds
+//     member node[t] (-1: none) of the set of lane owner[t]; the run's members
+//     count from 0, the round's first is base + 32 t, and the lane's own set
+//     holds [excl, incl)
+//   finish(j, len)
+template <class Begin, class Item, class Finish>
+__device__ __forceinline__ void for_live_members(const GreedyJob& J, int64_t warp, int64_t nwarps, int lane,
+                                                 Begin&& begin, Item&& item, Finish&& finish) {
+  int bs = 32;
+  while (bs > 1 && (int64_t)bs * nwarps > J.n_sets) bs >>= 1;
+  for (int64_t j0 = warp * bs; j0 < J.n_sets; j0 += nwarps * bs) {
+    const int64_t j = j0 + lane;
+    int len = 0;
+    int64_t start = 0;
+    if (lane < bs && j < J.n_sets) {
+      const uint8_t was = J.covered[j];
+      len = J.set_len[j];
+      start = J.set_start[j];
+      if (was) len = 0;
+    }
+    if (!__any_sync(FULL_MASK, len > 0)) continue;
+    begin(j, start, len);
+    const int incl = warp_inclusive_scan(len, lane);
+    const int excl = incl - len;
+    const int total = __shfl_sync(FULL_MASK, incl, 31);
+    for (int b = 0; b < total; b += 128) {
+      int32_t node[4];
+      int own[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int q = b + 32 * t + lane;
+        int o = 0;
+#pragma unroll
+        for (int s = 16; s; s >>= 1) {
+          const int x = __shfl_sync(FULL_MASK, incl, o + s - 1);
+          if (x <= q) o += s;
+        }
+        o = o > 31 ? 31 : o;
+        own[t] = o;
+        const int64_t at = __shfl_sync(FULL_MASK, start, o) + (q - __shfl_sync(FULL_MASK, excl, o));
+        node[t] = q < total ? __ldg(J.pool_nodes + at) : -1;
+      }
+      item(node, own, b, excl, incl);
+    }
+    finish(j, len);
   }
-  for (; t < len; t += 32) atomicSub(cnt + __ldg(mem + t), 1);
 }
 
-// Grid-wide maximum of the threads' keys, in every thread: each block folds
-// its own into one of three slots by atomicMax, and the barrier publishes the
-// slot.  Argmax number a uses slot a % 3; block 0 clears slot (a + 2) % 3 after
-// the barrier, which no block writes before the next barrier has completed.
-template <bool CLUSTER>
-__device__ __forceinline__ bool grid_argmax(const GreedyJob& J, unsigned long long& best, unsigned long long* s_red,
-                                            int& n_argmax, unsigned int* phase) {
-  best = block_max(best, s_red);
-  const int slot = n_argmax % 3;
-  n_argmax += 1;
-  unsigned long long* at = J.argmax + slot * ARGMAX_STRIDE;
-  if (threadIdx.x == 0 && best != 0ull) atomicMax(at, best);
-  if (!greedy_barrier<CLUSTER>(J, phase, [&] { return __ldcg(at); }, best)) return false;
-  if (blockIdx.x == 0 && threadIdx.x == 0) J.argmax[((slot + 2) % 3) * ARGMAX_STRIDE] = 0ull;
-  return true;
-}
-
-// Persistent greedy: all k picks of Algorithm 2 in one cooperative launch.
+// Persistent greedy: all k picks of Algorithm 2 in one launch (a cooperative
+// grid, one cluster, or a single block for small pools).
 //
-// Argmax.  A pick needs the node of largest gain, then smallest id.  Gains only
-// fall, so after a scan of all n nodes that finds the threshold g* with at
-// most CACHE_MAX nodes of gain >= g*, those nodes form a candidate cache: while
-// the best cached gain is still >= g*, it beats every node outside (all
-// <= g* - 1, ties included).  Every block holds the whole cache in shared
-// memory, and the last block to reach the barrier that ends a pick computes
-// the next pick's argmax over it, published with the release: a cached pick
-// costs one grid barrier.  When the best cached gain falls below g*, the pick
-// scans all n nodes (a second barrier publishes the maximum of the blocks'
-// keys) and builds a new cache from a gain histogram taken in the same pass.
+// Sessions.  Gains only fall.  A session takes the nodes of key (gain, ~id)
+// >= key* -- up to GCANDS of them, key* from a histogram over all n counts --
+// as candidates: while the best candidate's key is >= key*, it beats every
+// node outside, ties included, so the picks never look outside.  The sets not
+// covered yet are read once and written as candidate lists: per set the local
+// ids of its candidates, in 16-byte chunks (first {count:16, set:32} and four
+// 16-bit ids, then eight per chunk), and per candidate the list of its sets'
+// chunks.  This also gives every candidate's exact gain, whatever the counts
+// that chose it.  Then block 0 alone makes the picks: gains in its shared
+// memory, each thread keeping the best of its candidates, a pick's argmax two
+// warp reductions and a block barrier; the pick's sets are read eight lanes to
+// a set, their count set to 0 (covered) and their candidates' gains lowered by
+// shared-memory atomics.  A pick costs two dependent L2 round trips and two
+// block barriers, no grid barrier and no atomic in global memory.  When the
+// best candidate falls below key*, the counts of all nodes are taken again
+// over the sets left and the next session starts.
 //
-// Cover.  Warps walk v*'s inverted lists of all index batches and, for each
-// newly covered set, decrement the gains of its members.  Sets longer than
-// DEC_CHUNK go whole, as chunks, to a queue that every warp drains after the
-// barrier that closes the pick.  When the queued entries outnumber the
-// entries of the sets still uncovered (one pick can cover a bulk of huge sets
-// that share one core of nodes), the last block at that barrier calls for a
-// recount instead: gains are rebuilt from the uncovered sets, which costs
-// fewer atomics than the decrements would.  Barrier waits are bounded
-// (sync[SYNC_ERR] on timeout).
+// The first pick of a large pool goes by a pass over the flat entries instead
+// (`bulk`): it covers by far the most members (59% of the entries of 1.15M
+// weighted-cascade sets on the 2^25-node R-MAT graph, nearly all of a
+// trivalency pool's), which then need no list.  The first session after it
+// still chooses candidates by the counts before it: any upper bound on the
+// gains outside is a valid key*, and a recount is saved.
+//
+// Bound: the chain of a pick (two L2 round trips of ~600 clocks, two block
+// barriers, the argmax over shared memory), 1.5 us while a pick covers tens of
+// sets; picks that cover thousands are bound by the shared-memory atomics of
+// one SM.  Measured on GB300 against the former design (an inverted index of
+// all entries, a grid barrier of ~6 us per pick): 1000 picks over 134,016 sets
+// of the 2^23-node R-MAT graph 8.7 -> 2.3 ms, 500 over 131,832 LT sets there
+// 6.0 -> 2.1 ms, 100 over 1,149,440 sets of the 2^25-node one 3.5 -> 2.0 ms,
+// each with its index (0.2, 0.3 and 1.6 ms) gone.
+//
+// Gains of 0 go by smallest id.  Barrier waits are bounded (sync[SYNC_ERR] on
+// timeout); a session makes at most GCANDS picks, milliseconds, between two
+// barriers.
 template <bool CLUSTER>
 __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
+  extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ unsigned long long s_red[32];
-  __shared__ int64_t s_lo[GREEDY_MAX_LISTS], s_hi[GREEDY_MAX_LISTS];
-  // the gain histogram (HBINS) and the staged cache (CACHE_MAX ids) share
-  // space: a histogram is only taken after the cache has been dropped
-  __shared__ unsigned int s_buf[CACHE_MAX > HBINS ? CACHE_MAX : HBINS];
   __shared__ long long s_scan[32], s_scan_tot;
-  __shared__ unsigned long long s_cov_e, s_queued_e;  // entries of the sets this block covered / queued
-  __shared__ unsigned int s_phase;                     // sense of the next grid barrier
-  unsigned long long my_done = 0, my_queued = 0;      // thread 0: this block's slot values
-  unsigned int* s_hist = s_buf;
-  int32_t* s_cache = reinterpret_cast<int32_t*>(s_buf);
-  const int lane = threadIdx.x & 31;
-  const int64_t gtid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  __shared__ unsigned int s_phase;  // sense of the next grid barrier
+  __shared__ unsigned int s_w[2][32];
+  unsigned int* s_key = reinterpret_cast<unsigned int*>(s_dyn);  // block 0 in a session: keys (gain, ~local id),
+  unsigned int* s_id = s_key + GCANDS;                           // node ids
+  unsigned int* s_off = s_id + GCANDS;                           // and list offsets of the candidates
+  unsigned int* s_hist = reinterpret_cast<unsigned int*>(s_dyn);     // otherwise: the histogram
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int64_t gtid = blockIdx.x * (int64_t)blockDim.x + tid;
   const int64_t gthreads = (int64_t)gridDim.x * blockDim.x;
   const int64_t warp = gtid >> 5, nwarps = gthreads >> 5;
   const int64_t n4 = J.n_pad >> 2;
-  const int4* c4 = reinterpret_cast<const int4*>(J.cnt);
-  int n_argmax = 0;
-  if (threadIdx.x == 0) s_phase = 0u;  // the host zeroed the release word (sense 0)
-  // Rebuild policy (every block tracks the same values): the first pick only
-  // scans; a rebuild needs at least REBUILD_MIN picks left; a cache that served
-  // fewer than REBUILD_MIN picks, or a rebuild that found no threshold,
-  // postpones the next rebuild by a doubling back-off.
-  constexpr int REBUILD_MIN = 8;
-  int rebuilds = 0, next_try = 1, backoff = REBUILD_MIN, built_at = 0, gstar = 0, g_prev = 0;
-  bool cached = false, stage = false, fused_ok = false;
-  int nc = 0;                          // staged cache entries
-  unsigned long long fused_key = 0;    // this pick's argmax, from the previous pick's last barrier
-  // block-wide argmax over the staged cache, for the last block at a barrier
-  auto cache_argmax = [&]() -> unsigned long long {
-    unsigned long long b = 0;
-    for (int t = threadIdx.x; t < nc; t += blockDim.x) {
-      const int32_t v = s_cache[t];
-      const unsigned long long key = gain_key(__ldcg(J.cnt + v), (uint32_t)v);
-      b = key > b ? key : b;
-    }
-    return block_max(b, s_red);
-  };
-  for (int i = 0; i < J.k; ++i) {
+  int n_argmax = 0, n_hist = 0, i = 0;
+  bool first = true, bulk = J.bulk_first != 0, flat = false;
+  if (tid == 0) s_phase = 0u;  // the host zeroed the release word (sense 0)
+  unsigned long long info = 0;
+
+  // One pass over the gains: histogram of bin(key) (-1: not counted) merged
+  // into the next global histogram, and the largest key into the next argmax
+  // slot, which the barrier publishes in `info`.
+  // exact_bins: bin(key) is gain_bin of every gain.
+  auto scan_gains = [&](const int32_t* cnt, bool exact_bins, auto&& bin, unsigned int** hist) -> bool {
+    for (int t = tid; t < GBINS; t += blockDim.x) s_hist[t] = 0u;
+    __syncthreads();
     unsigned long long best = 0;
-    bool have = false;
-    if (cached) {
-      bool valid = false;
-      if (stage) {
-        // first pick on a new cache: every block stages all of it, and the
-        // blocks scan interleaved slices of it for this pick's argmax
-        const int cb = (rebuilds - 1) & 1;
-        const unsigned int m = __ldcg(J.cache_n + cb);
-        nc = m <= (unsigned int)CACHE_MAX ? (int)m : 0;
-        const int32_t* cache = J.cache + (size_t)cb * CACHE_MAX;
-        for (int t = threadIdx.x; t < nc; t += blockDim.x) s_cache[t] = __ldcg(cache + t);
-        __syncthreads();
-        stage = false;
-        if (m <= (unsigned int)CACHE_MAX) {
-          for (int t = blockIdx.x + (int)threadIdx.x * (int)gridDim.x; t < nc; t += (int)(blockDim.x * gridDim.x)) {
-            const int32_t v = s_cache[t];
-            const unsigned long long key = gain_key(__ldcg(J.cnt + v), (uint32_t)v);
-            best = key > best ? key : best;
-          }
-          if (!grid_argmax<CLUSTER>(J, best, s_red, n_argmax, &s_phase)) return;
-          valid = true;
+    // most nodes are in no set, one or two: those are counted in registers
+    unsigned int ones = 0, twos = 0;
+    int32_t one = -1, two = -1;  // the thread's first (smallest) of each
+    auto take = [&](int64_t q, const int4& c) {
+      const int32_t cv[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (exact_bins) {
+          const bool is1 = cv[u] == 1, is2 = cv[u] == 2;
+          ones += is1;
+          twos += is2;
+          if (is1 && one < 0) one = (int32_t)(q * 4 + u);
+          if (is2 && two < 0) two = (int32_t)(q * 4 + u);
         }
-      } else if (fused_ok) {
-        best = fused_key;
-        valid = true;
-      }
-      // every block holds the same maximum, so all take the same branch
-      have = valid && best != 0 && key_gain(best) >= gstar;
-      if (!have) {
-        cached = false;
-        if (i - built_at < REBUILD_MIN) {
-          next_try = i + backoff;
-          backoff = min(2 * backoff, 512);
-        } else {
-          backoff = REBUILD_MIN;
+        if (cv[u] > (exact_bins ? 2 : 0)) {
+          const unsigned long long key = gain_key(cv[u], (uint32_t)(q * 4 + u));
+          best = key > best ? key : best;
+          const int b = bin(cv[u], key);
+          if (b >= 0) atomicAdd(s_hist + b, 1u);
         }
       }
+    };
+    const int4* c4 = reinterpret_cast<const int4*>(cnt);
+    int64_t q = gtid;
+    for (; q + 3 * gthreads < n4; q += 4 * gthreads) {  // four loads in flight
+      const int4 a = c4[q], b = c4[q + gthreads], c = c4[q + 2 * gthreads], d = c4[q + 3 * gthreads];
+      take(q, a);
+      take(q + gthreads, b);
+      take(q + 2 * gthreads, c);
+      take(q + 3 * gthreads, d);
     }
-    if (!have) {
-      const bool rebuild = i >= next_try && J.k - i >= REBUILD_MIN;
-      // the histogram counts gains >= floor only (bin c - floor, the top bin
-      // "at least"): the cache threshold sits near the top, and low gains,
-      // the bulk of the nodes, would only contend on a few bins
-      const int floor_g = max(1, g_prev >> 2);
-      const int hb = rebuilds & 1;
-      if (rebuild) {
-        for (int t = threadIdx.x; t < HBINS; t += blockDim.x) s_hist[t] = 0u;
-        __syncthreads();
-      }
-      best = 0;
-      for (int64_t q = gtid; q < n4; q += gthreads) {
-        const int4 c = __ldcg(c4 + q);
-        const uint32_t v = (uint32_t)(q * 4);
-        unsigned long long key;
-        key = gain_key(c.x, v);     best = key > best ? key : best;
-        key = gain_key(c.y, v + 1); best = key > best ? key : best;
-        key = gain_key(c.z, v + 2); best = key > best ? key : best;
-        key = gain_key(c.w, v + 3); best = key > best ? key : best;
-        if (rebuild) {
-          if (c.x >= floor_g) atomicAdd(s_hist + min(c.x - floor_g, HBINS - 1), 1u);
-          if (c.y >= floor_g) atomicAdd(s_hist + min(c.y - floor_g, HBINS - 1), 1u);
-          if (c.z >= floor_g) atomicAdd(s_hist + min(c.z - floor_g, HBINS - 1), 1u);
-          if (c.w >= floor_g) atomicAdd(s_hist + min(c.w - floor_g, HBINS - 1), 1u);
-        }
-      }
-      if (rebuild) {
-        unsigned int* h = J.hist + (size_t)hb * HBINS;
-        __syncthreads();
-        for (int t = threadIdx.x; t < HBINS; t += blockDim.x)
-          if (s_hist[t]) atomicAdd(h + t, s_hist[t]);
-      }
-      if (!grid_argmax<CLUSTER>(J, best, s_red, n_argmax, &s_phase)) return;
-      if (rebuild) {
-        // g* = floor + the smallest bin b with at most CACHE_MAX nodes in
-        // bins >= b: a descending block scan of the merged histogram (thread t
-        // holds bins HBINS-1-PER*t down to HBINS-PER*(t+1)); none when the
-        // top bin alone holds too many nodes
-        constexpr int PER = HBINS / 1024;
-        const unsigned int* h = J.hist + (size_t)hb * HBINS;
-        const int top = HBINS - 1 - (int)threadIdx.x * PER;
-        unsigned int hv[PER];
-        long long mine = 0;
-#pragma unroll
-        for (int u = 0; u < PER; ++u) {
-          hv[u] = __ldcg(h + top - u);
-          mine += hv[u];
-        }
-        long long above = block_exclusive_scan<long long>(mine, s_scan, &s_scan_tot);
-        unsigned long long key = 0;  // HBINS - b of the smallest qualifying bin
-#pragma unroll
-        for (int u = 0; u < PER; ++u) {
-          above += hv[u];
-          if (above <= (long long)CACHE_MAX) key = (unsigned long long)(HBINS - (top - u));
-        }
-        key = block_max(key, s_red);
-        int g = key ? floor_g + (HBINS - (int)key) : 0;
-        // a threshold above the best gain would leave the best node outside
-        if (g > key_gain(best)) g = 0;
-        if (g > 0) {
-          // Some blocks may already be covering for this pick, so a gain read
-          // here may have fallen since the scan: below g* it stays below for
-          // good; at or above g* it was counted in the histogram, which bounds
-          // the cache at CACHE_MAX entries.
-          const int32_t vstar = key_node(best);
-          unsigned int* nout = J.cache_n + hb;
-          int32_t* out = J.cache + (size_t)hb * CACHE_MAX;
-          // warp-uniform trip count, so the ballots below see all 32 lanes
-          for (int64_t q0 = gtid - lane; q0 < n4; q0 += gthreads) {
-            const int64_t q = q0 + lane;
-            int4 c = make_int4(-1, -1, -1, -1);
-            if (q < n4) c = __ldcg(c4 + q);
-            const int32_t v = (int32_t)(q * 4);
-            const int32_t cv[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const bool take = cv[u] >= g && v + u != vstar;
-              const unsigned int m = __ballot_sync(FULL_MASK, take);
-              if (m == 0u) continue;
-              const int leader = __ffs(m) - 1;
-              unsigned int at = 0;
-              if (lane == leader) at = atomicAdd(nout, (unsigned int)__popc(m));
-              at = __shfl_sync(FULL_MASK, at, leader) + (unsigned int)__popc(m & ((1u << lane) - 1u));
-              if (take && at < (unsigned int)CACHE_MAX) out[at] = v + u;
-            }
-          }
-          gstar = g;
-          cached = true;
-          built_at = i;
-          stage = true;
-        } else {
-          next_try = i + backoff;  // the top is too flat: full scans for a while
-          backoff = min(2 * backoff, 512);
-        }
-        // this parity's histogram and cache stay read-only until the next
-        // rebuild, which uses the other parity: clear that one now (nobody
-        // reads it any more: its last staging ended before the barrier above)
-        if (blockIdx.x == 0) {
-          for (int t = threadIdx.x; t < HBINS; t += blockDim.x) J.hist[(size_t)(hb ^ 1) * HBINS + t] = 0u;
-          if (threadIdx.x == 0) J.cache_n[hb ^ 1] = 0u;
-        }
-        rebuilds += 1;
-      }
+    for (; q < n4; q += gthreads) take(q, c4[q]);
+    if (ones) atomicAdd(s_hist + 1, ones);
+    if (twos) atomicAdd(s_hist + 2, twos);
+    if (best == 0ull && (ones || twos)) best = twos ? gain_key(2, (uint32_t)two) : gain_key(1, (uint32_t)one);
+    __syncthreads();
+    unsigned int* h = J.hist + (size_t)(n_hist % GHISTS) * GBINS;
+    for (int t = tid; t < GBINS; t += blockDim.x)
+      if (s_hist[t]) atomicAdd(h + t, s_hist[t]);
+    best = block_max(best, s_red);
+    unsigned long long* at = J.argmax + (n_argmax % 3) * ARGMAX_STRIDE;
+    if (tid == 0 && best) atomicMax(at, best);
+    if (!greedy_barrier<CLUSTER>(J, &s_phase, [&] { return __ldcg(at); }, info)) return false;
+    // clear the slot and the histogram of two scans on: nobody has touched
+    // them since the barrier before this one
+    if (blockIdx.x == 0) {
+      if (tid == 0) J.argmax[((n_argmax + 2) % 3) * ARGMAX_STRIDE] = 0ull;
+      unsigned int* z = J.hist + (size_t)((n_hist + 2) % GHISTS) * GBINS;
+      for (int t = tid; t < GBINS; t += blockDim.x) z[t] = 0u;
+    }
+    n_argmax += 1;
+    n_hist += 1;
+    *hist = h;
+    return true;
+  };
+  // The lowest bin b such that, with `have` nodes of `sum` list entries taken
+  // already, the nodes of bins >= b still fit (GCANDS nodes, ents_cap list
+  // entries; top(b): largest gain of bin b).  Returns b, adds what they take to
+  // have and sum; *total: nodes in all bins.
+  auto cut = [&](const unsigned int* hist, auto&& top, long long& have, long long& sum, long long* total) -> int {
+    const int b = GBINS - 1 - tid;  // 1024 threads: one bin each, from the top
+    const long long c = __ldcg(hist + b);
+    const long long e = c ? c * (long long)top(b) : 0;
+    const long long ic = block_exclusive_scan<long long>(c, s_scan, &s_scan_tot) + c;
+    *total = s_scan_tot;
+    __syncthreads();
+    const long long is = block_exclusive_scan<long long>(e, s_scan, &s_scan_tot) + e;
+    const bool fits = have + ic <= GCANDS && sum + is <= (long long)J.ents_cap;
+    // bins fit from the top down to the first that does not
+    const unsigned long long n_fit = GBINS - block_max(fits ? 0ull : (unsigned long long)(GBINS - tid), s_red);
+    __shared__ long long s_have, s_sum;
+    if (n_fit > 0 && tid == (int)n_fit - 1) {
+      s_have = ic;
+      s_sum = is;
+    }
+    __syncthreads();
+    if (n_fit > 0) {
+      have += s_have;
+      sum += s_sum;
+    }
+    __syncthreads();
+    return GBINS - (int)n_fit;
+  };
+
+  for (;;) {
+    // ---- candidates: key* and the best node ----
+    const int32_t* cnt = first ? J.cnt0 : J.cnt;
+    unsigned int* hist = nullptr;
+    if (!scan_gains(cnt, true, [](int32_t c, unsigned long long) { return gain_bin(c); }, &hist)) return;
+    const unsigned long long best = info;
+    if (best == 0ull) {  // no gain is left
+      flat = true;
+      break;
     }
     const int32_t vstar = key_node(best);
-    g_prev = key_gain(best);
-    if (threadIdx.x < J.nlists) {
-      s_lo[threadIdx.x] = J.lists[threadIdx.x].off[vstar];
-      s_hi[threadIdx.x] = J.lists[threadIdx.x].off[vstar + 1];
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      J.seeds[i] = vstar;
-      J.gains[i] = key_gain(best);
-    }
-    if (threadIdx.x == 0) {
-      s_cov_e = 0ull;
-      s_queued_e = 0ull;
-    }
-    __syncthreads();
-    unsigned int* chunks = J.sync + SYNC_CHUNKS + (i & 1) * 16;
-    for (int b = 0; b < J.nlists; ++b) {
-      const int32_t* samp = J.lists[b].samp;
-      for (int64_t q = s_lo[b] + warp; q < s_hi[b]; q += nwarps) {
-        const int32_t j = samp[q];
-        // the set's extent loads alongside its covered flag (one round trip, not two)
-        const uint8_t was = __ldcg(J.covered + j);
-        const int32_t len = J.set_len[j];
-        const int64_t start = J.set_start[j];
-        if (was) continue;
-        __syncwarp();
-        if (lane == 0) J.covered[j] = 1;
-        if (lane == 0) atomicAdd(&s_cov_e, (unsigned long long)len);
-        if (len > DEC_CHUNK) {
-          // the whole set goes to the queue, for a drain or a recount after the barrier
-          const int nq = (len + DEC_CHUNK - 1) / DEC_CHUNK;
-          unsigned int at = 0;
-          if (lane == 0) {
-            at = atomicAdd(chunks, (unsigned int)nq);
-            atomicAdd(&s_queued_e, (unsigned long long)len);
+    const bool wide = key_gain(best) >= GMAX;  // gains that a session's keys cannot hold
+    bulk = bulk || wide;
+    if (bulk) {
+      if (blockIdx.x == 0 && tid == 0) {
+        J.seeds[i] = vstar;
+        J.gains[i] = key_gain(best);
+      }
+      i += 1;
+      if (i == J.k) break;
+      // every set that holds v* is covered (four entries a thread and load)
+      const int64_t q4n = J.total_entries >> 2;
+      const int4* e4 = reinterpret_cast<const int4*>(J.pool_nodes);
+      for (int64_t q = gtid; q < q4n; q += gthreads) {
+        const int4 e = __ldg(e4 + q);
+        const int32_t ev[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (ev[u] == vstar) {
+            const int32_t s = __ldg(J.pool_samp + q * 4 + u);
+            if (s < J.n_sets) J.covered[s] = 1;
           }
-          at = __shfl_sync(FULL_MASK, at, 0);
-          if ((int64_t)at + nq > J.chunk_cap) {  // cannot happen with the host's sizing
-            if (lane == 0) atomicExch(J.sync + SYNC_ERR, 2u);
-            continue;
-          }
-          for (int c = lane; c < nq; c += 32)
-            J.chunk_q[at + c] = ((unsigned long long)(uint32_t)j << 32) | (uint32_t)(c * DEC_CHUNK);
-          continue;
+      }
+      for (int64_t q = q4n * 4 + gtid; q < (int64_t)J.total_entries; q += gthreads)
+        if (__ldg(J.pool_nodes + q) == vstar) {
+          const int32_t s = __ldg(J.pool_samp + q);
+          if (s < J.n_sets) J.covered[s] = 1;
         }
-        decrement_members(J.cnt, J.pool_nodes + start, len, lane);
-      }
     }
-    // v* leaves the candidates for good (its remaining decrements keep it negative)
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(J.cnt + vstar, INT32_MIN / 2);
-    // The barrier that ends the pick also yields the next pick's argmax when
-    // the next pick uses a staged cache; queued chunks come first, and then
-    // the drain's barrier yields it instead.
-    const bool fuse = cached && !stage;
-    unsigned long long pay = 0;
-    __syncthreads();
-    // plain stores to the block's own slots, only when they change
-    if (threadIdx.x == 0) {
-      if (s_cov_e) {
-        my_done += s_cov_e;
-        J.argmax[ACC_DONE + blockIdx.x] = my_done;
+    const bool session = !bulk || (first && !wide);  // else recount before the next session
+    unsigned long long keystar = 0;
+    if (session) {
+      long long have = 0, sum = 0, total = 0;
+      int b = cut(hist, [](int x) { return bin_gain(x + 1) - 1; }, have, sum, &total);
+      b = max(b, 1);
+      keystar = gain_floor_key(bin_gain(b));
+      // too few: cut the bin below by key until some of it fits
+      unsigned long long lo = b > 1 ? gain_floor_key(bin_gain(b - 1)) : keystar, hi = keystar;
+      while (have < 64 && have < total && lo < hi) {
+        if ((lo >> 31) == ((hi - 1) >> 31))  // one gain: only ids below n occur
+          lo = max(lo, ((lo >> 31) << 31) | (unsigned long long)(0x7FFFFFFFu - (uint32_t)(J.n - 1)));
+        const unsigned long long width = (hi - lo + GBINS - 1) / GBINS;
+        const int32_t g_hi = key_gain(hi - 1);
+        if (!scan_gains(cnt, false, [=](int32_t, unsigned long long key) {
+              return key >= lo && key < hi ? (int)((key - lo) / width) : -1;
+            }, &hist)) return;
+        long long in_range = 0;
+        b = cut(hist, [=](int) { return g_hi; }, have, sum, &in_range);
+        keystar = min(hi, lo + (unsigned long long)b * width);
+        hi = keystar;
+        lo = b > 0 && width > 1 ? lo + (unsigned long long)(b - 1) * width : hi;
       }
-      if (s_queued_e != my_queued) {
-        my_queued = s_queued_e;
-        J.argmax[ACC_QUEUED + blockIdx.x] = my_queued;
+      // ---- the candidates get local ids and list space ----
+      const int4* c4 = reinterpret_cast<const int4*>(cnt);
+      const int32_t gmin = key_gain(keystar);
+      const int32_t skip = bulk ? vstar : -1;
+      // marked first, then numbered in id order, so that of equal gains the
+      // smaller local id is the smaller node id.  Block b numbers the mark words
+      // [b * per, (b + 1) * per); a warp's 128 nodes are four words of one block.
+      // (Counted per block in shared memory first: hubs with neighbouring ids
+      // would queue on one global counter.)
+      const unsigned int words = (unsigned int)((J.n_pad + 31) >> 5);
+      const unsigned int per = (words + 4 * gridDim.x - 1) / (4 * gridDim.x) * 4;
+      unsigned int* s_blk = reinterpret_cast<unsigned int*>(s_dyn);
+      if (tid < (int)gridDim.x) s_blk[tid] = 0u;
+      __syncthreads();
+      auto select = [&](int64_t q, const int4& c) {
+        const bool any = c.x >= gmin || c.y >= gmin || c.z >= gmin || c.w >= gmin;
+        if (!any) return;
+        const uint32_t v = (uint32_t)(q * 4);
+        const int32_t cv[4] = {c.x, c.y, c.z, c.w};
+        unsigned int take = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (cv[u] > 0 && gain_key(cv[u], v + u) >= keystar && (int32_t)(v + u) != skip) take |= 1u << u;
+        if (!take) return;
+        atomicOr(J.mark + (v >> 5), take << (v & 31u));
+        atomicAdd(s_blk + (v >> 5) / per, (unsigned int)__popc(take));
+      };
+      int64_t q = gtid;
+      for (; q + 3 * gthreads < n4; q += 4 * gthreads) {  // four loads in flight
+        const int4 a = c4[q], b = c4[q + gthreads], c = c4[q + 2 * gthreads], d = c4[q + 3 * gthreads];
+        select(q, a);
+        select(q + gthreads, b);
+        select(q + 2 * gthreads, c);
+        select(q + 3 * gthreads, d);
       }
-    }
-    if (!greedy_barrier<CLUSTER>(J, &s_phase, [&]() -> unsigned long long {
-          const unsigned int m = __ldcg(chunks);
-          if (m > 0u) {
-            // entries still in uncovered sets after this pick, against the queued ones
-            unsigned long long done = 0, q = 0;
-            if (threadIdx.x < gridDim.x) {
-              done = __ldcg(J.argmax + ACC_DONE + threadIdx.x);
-              q = __ldcg(J.argmax + ACC_QUEUED + threadIdx.x);
+      for (; q < n4; q += gthreads) select(q, c4[q]);
+      __syncthreads();
+      if (tid < (int)gridDim.x && s_blk[tid]) atomicAdd(J.blk + tid, s_blk[tid]);
+      if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
+      int nc;
+      {
+        const long long own_b = tid < (int)gridDim.x ? (long long)__ldcg(J.blk + tid) : 0ll;
+        const long long before = block_exclusive_scan<long long>(own_b, s_scan, &s_scan_tot);
+        nc = (int)s_scan_tot;
+        __shared__ int s_base;
+        if (tid == (int)blockIdx.x) s_base = (int)before;
+        __syncthreads();
+        // a run of words per thread
+        const unsigned int wpt = (per + 1023) >> 10;
+        const unsigned int w0 = min(words, blockIdx.x * per + tid * wpt);
+        const unsigned int w1 = min(min(words, (blockIdx.x + 1) * per), w0 + wpt);
+        int c = 0;
+        for (unsigned int w = w0; w < w1; ++w) c += __popc(J.mark[w]);
+        int l = s_base + (int)block_exclusive_scan<long long>((long long)c, s_scan, &s_scan_tot);
+        if (c)
+          for (unsigned int w = w0; w < w1; ++w) {
+            for (unsigned int m = J.mark[w]; m; m &= m - 1u) {
+              const unsigned int v = (w << 5) + (unsigned int)__ffs(m) - 1u;
+              J.cand_id[l] = (int32_t)v;
+              J.lid[v] = (uint16_t)(++l);
             }
-            done = block_reduce<true>(done, s_red);
-            q = block_reduce<true>(q, s_red);
-            // a recount costs an increment per entry left, a pass over the sets'
-            // flags and the gains, and two more barriers: it must win clearly
-            const unsigned long long left = done < J.total_entries ? J.total_entries - done : 0ull;
-            const unsigned long long fixed = (unsigned long long)(J.n_sets + J.n_pad) / 8 + (1ull << 20);
-            return PENDING | (q > 2 * left + fixed ? RECOUNT : 0ull) | m;
+            J.mark[w] = 0u;
           }
-          return fuse ? cache_argmax() : 0ull;
-        }, pay)) return;
-    // the other parity's queue was drained in the previous pick: reset it for the next one
-    if (blockIdx.x == 0 && threadIdx.x == 0) J.sync[SYNC_CHUNKS + ((i + 1) & 1) * 16] = 0u;
-    if ((pay & PENDING) && (pay & RECOUNT)) {
-      // gains from scratch: zero every unpicked node (picked and padding
-      // nodes stay negative), then one increment per member of each set still
-      // uncovered; no uncovered set holds a picked node
-      for (int64_t q = gtid; q < n4; q += gthreads) {
-        int4 c = __ldcg(c4 + q);
-        c.x = c.x < 0 ? c.x : 0;
-        c.y = c.y < 0 ? c.y : 0;
-        c.z = c.z < 0 ? c.z : 0;
-        c.w = c.w < 0 ? c.w : 0;
-        reinterpret_cast<int4*>(J.cnt)[q] = c;
       }
-      unsigned long long unused = 0;
-      if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, unused)) return;
-      for (int64_t j = warp; j < J.n_sets; j += nwarps) {
-        if (__ldcg(J.covered + j)) continue;
-        const int32_t* mem = J.pool_nodes + J.set_start[j];
-        const int32_t len = J.set_len[j];
-        for (int t = lane; t < len; t += 32) atomicAdd(J.cnt + __ldg(mem + t), 1);
+      if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
+      // list space, as many entries as the count that chose the candidate
+      for (int t0 = (int)blockIdx.x * 1024; t0 < nc; t0 += (int)gridDim.x * 1024) {
+        const int t = t0 + tid;
+        const long long g = t < nc ? (long long)cnt[J.cand_id[t]] : 0ll;
+        const long long at = block_exclusive_scan<long long>(g, s_scan, &s_scan_tot);
+        __shared__ unsigned int s_list;
+        if (tid == 0) s_list = atomicAdd(J.ncand + 4, (unsigned int)s_scan_tot);
+        __syncthreads();
+        if (t < nc) {
+          J.cand_len[t] = 0;
+          J.cand_off[t] = s_list + (unsigned int)at;
+        }
+        __syncthreads();
       }
-      if (!greedy_barrier<CLUSTER>(J, &s_phase, [&]() -> unsigned long long { return fuse ? cache_argmax() : 0ull; }, pay)) return;
-    } else if (pay & PENDING) {
-      const int64_t nchunks = (int64_t)(pay & (RECOUNT - 1ull));
-      for (int64_t c = warp; c < nchunks; c += nwarps) {
-        const unsigned long long e = J.chunk_q[c];
-        const int32_t j = (int32_t)(e >> 32), from = (int32_t)(uint32_t)e;
-        const int32_t len = J.set_len[j];
-        const int32_t cnt = min(DEC_CHUNK, len - from);
-        decrement_members(J.cnt, J.pool_nodes + J.set_start[j] + from, cnt, lane);
+      if (blockIdx.x == 0 && tid == 0) J.ncand[0] = (unsigned int)nc;
+      if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
+      // ---- candidate lists of the sets left ----
+      // a member's local id (1 + id, 0: no candidate) goes to its place `r` in
+      // the set's chunks at cs, and the chunks to the candidate's list
+      auto put = [&](unsigned int l, unsigned int cs, unsigned int off, int pos, int r) {
+        reinterpret_cast<uint16_t*>(J.chunks + cs)[4 + r] = (uint16_t)(l - 1u);
+        J.ents[off + (unsigned int)pos] = cs;
+      };
+      unsigned int cs = 0;  // this lane's set: its first chunk
+      int run = 0;          // and the candidates found so far
+      bool over = false;
+      for_live_members(
+          J, warp, nwarps, lane,
+          [&](int64_t j, int64_t, int& len) {
+            // room for every member: chunks are cheap (2 bytes a member) and a counting pass is not
+            const int nch = len ? ((len + 19) >> 4) * 2 : 0;
+            const int incl = warp_inclusive_scan(nch, lane);
+            unsigned long long at = 0;
+            if (lane == 31) at = atomicAdd(J.nchunk, (unsigned long long)incl);
+            at = __shfl_sync(FULL_MASK, at, 31);
+            over = at + (unsigned long long)__shfl_sync(FULL_MASK, incl, 31) > J.chunk_cap;
+            cs = (unsigned int)(at + (unsigned long long)(incl - nch));
+            run = 0;
+            // a long set would keep its warp long after the others: its parts go to the queue
+            if (len > GLONG && !over) {
+              const unsigned int parts = (unsigned int)((len + GLONG - 1) / GLONG);
+              const unsigned int t0 = atomicAdd(J.ncand + 3, parts);
+              *reinterpret_cast<uint2*>(J.chunks + cs) = make_uint2(0u, (unsigned int)j);
+              for (unsigned int t = 0; t < parts; ++t) J.tasks[t0 + t] = make_uint4(cs, (unsigned int)j, t * GLONG, 0u);
+              len = 0;
+            }
+          },
+          [&](const int32_t* node, const int* own, int b0, int excl, int incl) {
+            if (over) return;
+            unsigned int l[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) l[t] = node[t] >= 0 ? J.lid[node[t]] : 0u;
+            int pos[4];
+            unsigned int off[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+              if (l[t]) {
+                off[t] = J.cand_off[l[t] - 1u];
+                pos[t] = atomicAdd(J.cand_len + (l[t] - 1u), 1);
+              }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+              const int b = b0 + 32 * t;
+              const unsigned int m = __ballot_sync(FULL_MASK, l[t] != 0u);
+              if (m == 0u) continue;
+              const int o = own[t];
+              // the owner's members of this round sit in lanes [max(excl - b, 0), min(incl - b, 32))
+              const int oex = __shfl_sync(FULL_MASK, excl, o);
+              const unsigned int ocs = __shfl_sync(FULL_MASK, cs, o);
+              const int orun = __shfl_sync(FULL_MASK, run, o);
+              const int f = max(oex - b, 0);
+              if (l[t]) {
+                const unsigned int below = ((1u << lane) - 1u) & (FULL_MASK << f);
+                put(l[t], ocs, off[t], pos[t], orun + __popc(m & below));
+              }
+              const int s0 = min(max(excl - b, 0), 32), s1 = min(max(incl - b, 0), 32);
+              const unsigned int upto = s1 >= 32 ? FULL_MASK : (1u << s1) - 1u;
+              const unsigned int from = s0 >= 32 ? 0u : FULL_MASK << s0;
+              run += __popc(m & upto & from);
+            }
+          },
+          [&](int64_t j, int len) {
+            if (over) {
+              if (lane == 0) atomicExch(J.ncand + 1, 1u);
+            } else if (len > 0 && run > 0) {
+              *reinterpret_cast<uint2*>(J.chunks + cs) = make_uint2((unsigned int)run, (unsigned int)j);
+            }
+          });
+      if (!greedy_barrier<CLUSTER>(J, &s_phase, [&] {
+            return ((unsigned long long)__ldcg(J.ncand + 1) << 32) | (unsigned long long)__ldcg(J.ncand + 3);
+          }, info)) return;
+      const unsigned int ntasks = (unsigned int)info;
+      if (ntasks > 0u && (info >> 32) == 0ull) {
+        // parts of the long sets, a warp each: places in the set's chunks by its running count
+        for (int64_t q = warp; q < ntasks; q += nwarps) {
+          const uint4 t = J.tasks[q];
+          const int64_t start = J.set_start[t.y];
+          const int end = min(J.set_len[t.y], (int)t.z + GLONG);
+          unsigned int l[GLONG / 32];
+          int mine = 0;
+#pragma unroll
+          for (int u = 0; u < GLONG / 32; ++u) {
+            const int x = (int)t.z + u * 32 + lane;
+            l[u] = x < end ? (unsigned int)__ldg(J.pool_nodes + start + x) : 0xFFFFFFFFu;
+          }
+#pragma unroll
+          for (int u = 0; u < GLONG / 32; ++u) {
+            l[u] = l[u] != 0xFFFFFFFFu ? J.lid[l[u]] : 0u;
+            mine += l[u] != 0u;
+          }
+          const int mi = warp_inclusive_scan(mine, lane);
+          int r = 0;
+          if (lane == 31 && mi) r = (int)atomicAdd(reinterpret_cast<unsigned int*>(J.chunks + t.x), (unsigned int)mi);
+          r = __shfl_sync(FULL_MASK, r, 31) + mi - mine;
+#pragma unroll
+          for (int u = 0; u < GLONG / 32; ++u)
+            if (l[u]) put(l[u], t.x, J.cand_off[l[u] - 1u], atomicAdd(J.cand_len + (l[u] - 1u), 1), r++);
+        }
+        if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
+        info = 0ull;
+      } else {
+        info >>= 32;
       }
-      if (!greedy_barrier<CLUSTER>(J, &s_phase, [&]() -> unsigned long long { return fuse ? cache_argmax() : 0ull; }, pay)) return;
     }
-    fused_key = pay;
-    fused_ok = fuse;
+    bool overflow = session && info != 0ull;
+    // ---- the session's picks ----
+    if (session) {
+      const int nc = (int)__ldcg(J.ncand);
+      overflow = overflow || nc == 0;
+      if (blockIdx.x == 0 && !overflow) {
+        const int ncp = (nc + 1023) & ~1023;
+        for (int t = tid; t < ncp; t += 1024) {
+          s_key[t] = t < nc ? ((unsigned int)__ldcg(J.cand_len + t) << GBITS) | (unsigned int)(GCANDS - 1 - t) : 0u;
+          s_id[t] = t < nc ? (unsigned int)__ldcg(J.cand_id + t) : 0u;
+          s_off[t] = t < nc ? __ldcg(J.cand_off + t) : 0u;
+        }
+        __syncthreads();
+        // best key of the thread's candidates tid, tid + 1024, ...; gains only
+        // fall, so it stands until that candidate's own key changes
+        unsigned int bk = 0xFFFFFFFFu;
+        int par = 0;
+        while (i < J.k) {
+          if (bk && s_key[GCANDS - 1 - (bk & (GCANDS - 1))] != bk) {
+            bk = 0u;
+#pragma unroll
+            for (int r = 0; r < GCANDS / 1024; ++r)
+              if (r * 1024 < ncp) bk = max(bk, s_key[r * 1024 + tid]);
+          }
+          const unsigned int wk = __reduce_max_sync(FULL_MASK, bk);
+          if (lane == 0) s_w[par][wid] = wk;
+          __syncthreads();
+          const unsigned int top = __reduce_max_sync(FULL_MASK, s_w[par][lane]);
+          par ^= 1;
+          const int l = GCANDS - 1 - (int)(top & (GCANDS - 1));
+          const int g = (int)(top >> GBITS);
+          const unsigned int off = s_off[l], v = s_id[l];
+          if (top == 0u || gain_key(g, v) < keystar) break;
+          const int len = __ldcg(J.cand_len + l);
+          // lanes per set: eight chunks of each set at once while the sets are few, else two
+          const unsigned int spec = __ldcg(J.ents + off + (tid >> 3));  // the buffer has spare entries past the last list
+          const int sh = len <= 128 ? 3 : 1;
+          const int per_set = 1 << sh, r0 = lane & (per_set - 1), first_slots = 8 * per_set - 4;
+          unsigned int cs = sh == 3 ? spec : __ldcg(J.ents + off + (tid >> 1));
+          if (tid == 0) {
+            J.seeds[i] = (int32_t)v;
+            J.gains[i] = g;
+            s_key[l] = 0u;  // never again; the loop below leaves it alone
+          }
+          auto lower = [&](unsigned int pair, int slot, int cnt) {  // slots `slot` and `slot` + 1 of a list of cnt
+            const int x = (int)(pair & 0xFFFFu), y = (int)(pair >> 16);
+            if (slot < cnt && x != l) atomicSub(s_key + x, 1u << GBITS);
+            if (slot + 1 < cnt && y != l) atomicSub(s_key + y, 1u << GBITS);
+          };
+          for (int base = (tid & ~31) >> sh; base < len; base += 1024 >> sh) {
+            const unsigned int c0 = cs;
+            if (base + (1024 >> sh) < len) cs = __ldcg(J.ents + off + base + (1024 >> sh) + (lane >> sh));
+            uint4 a = make_uint4(0u, 0u, 0u, 0u);
+            if (base + (lane >> sh) < len) a = __ldcg(J.chunks + c0 + r0);  // may run past the list: spare chunks
+            const int cnt_l = (int)__shfl_sync(FULL_MASK, a.x, lane & ~(per_set - 1));  // 0: covered
+            if (r0 == 0) {
+              if (cnt_l) {
+                J.covered[a.y] = 1;
+                *reinterpret_cast<unsigned int*>(J.chunks + c0) = 0u;
+              }
+            } else {
+              lower(a.x, 8 * r0 - 4, cnt_l);
+              lower(a.y, 8 * r0 - 2, cnt_l);
+            }
+            lower(a.z, 8 * r0, cnt_l);
+            lower(a.w, 8 * r0 + 2, cnt_l);
+            // what is left of the warp's sets is dealt to the lanes chunk by chunk
+            const int rest = r0 == 0 && cnt_l > first_slots ? (cnt_l - first_slots + 7) >> 3 : 0;
+            if (!__any_sync(FULL_MASK, rest)) continue;
+            const int incl = warp_inclusive_scan(rest, lane);
+            const int total = __shfl_sync(FULL_MASK, incl, 31);
+            for (int q0 = 0; q0 < total; q0 += 32) {
+              const int q = q0 + lane;
+              int o = 0;
+#pragma unroll
+              for (int s = 16; s; s >>= 1) {
+                const int x = __shfl_sync(FULL_MASK, incl, o + s - 1);
+                if (x <= q) o += s;
+              }
+              o = o > 31 ? 31 : o;
+              const int r = q - (__shfl_sync(FULL_MASK, incl, o) - __shfl_sync(FULL_MASK, rest, o));
+              const unsigned int oc = __shfl_sync(FULL_MASK, c0, o);
+              const int ocnt = __shfl_sync(FULL_MASK, cnt_l, o);
+              if (q < total) {
+                const uint4 w = __ldcg(J.chunks + oc + per_set + r);
+                lower(w.x, first_slots + 8 * r, ocnt);
+                lower(w.y, first_slots + 8 * r + 2, ocnt);
+                lower(w.z, first_slots + 8 * r + 4, ocnt);
+                lower(w.w, first_slots + 8 * r + 6, ocnt);
+              }
+            }
+          }
+          i += 1;
+          __syncthreads();
+        }
+      }
+      // the local ids go back to 0 for the next session
+      const int64_t b0 = gridDim.x > 1 ? blockIdx.x - 1 : 0, nb = gridDim.x > 1 ? gridDim.x - 1 : 1;
+      if (b0 >= 0)
+        for (int64_t t = b0 * 1024 + tid; t < nc; t += nb * 1024) J.lid[__ldcg(J.cand_id + t)] = 0;
+      if (blockIdx.x == 0 && tid == 0) J.ncand[2] = (unsigned int)i;
+      if (!greedy_barrier<CLUSTER>(J, &s_phase, [&] { return (unsigned long long)__ldcg(J.ncand + 2); }, info)) return;
+      i = (int)info;
+      if (i >= J.k) break;
+    }
+    // ---- gains again over the sets left ----
+    for (int64_t q = gtid; q < n4; q += gthreads) reinterpret_cast<int4*>(J.cnt)[q] = make_int4(0, 0, 0, 0);
+    if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
+    if (blockIdx.x == 0) {
+      for (int t = tid; t < i; t += 1024) J.cnt[__ldcg(J.seeds + t)] = -1;  // in no set that is left
+      if (tid < (int)gridDim.x) J.blk[tid] = 0u;
+      if (tid == 0) {
+        J.ncand[1] = J.ncand[3] = J.ncand[4] = 0u;
+        *J.nchunk = 0ull;
+      }
+    }
+    for_live_members(
+        J, warp, nwarps, lane, [](int64_t, int64_t, int&) {},
+        [&](const int32_t* node, const int*, int, int, int) {
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+            if (node[t] >= 0) atomicAdd(J.cnt + node[t], 1);
+        },
+        [](int64_t, int) {});
+    if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
+    bulk = overflow;  // lists that did not fit: cover the best node's sets first
+    first = false;
+  }
+  // every gain is 0: the smallest ids not picked yet
+  if (flat && blockIdx.x == 0) {
+    const int32_t* cnt = first ? J.cnt0 : J.cnt;
+    for (int64_t v0 = 0; v0 < J.n && i < J.k; v0 += 1024) {
+      const int64_t v = v0 + tid;
+      const bool free_v = v < J.n && cnt[v] >= 0;
+      const long long at = block_exclusive_scan<long long>(free_v ? 1 : 0, s_scan, &s_scan_tot);
+      const long long tot = s_scan_tot;
+      __syncthreads();
+      if (free_v && i + at < J.k) {
+        J.seeds[i + at] = (int32_t)v;
+        J.gains[i + at] = 0;
+      }
+      i = (int)min((long long)J.k, i + tot);
+    }
   }
   if constexpr (CLUSTER) {
     // no block may leave while another can still read its shared memory: the
     // payload of the last barrier lives in block 0's
     cooperative_groups::this_cluster().sync();
   }
-}
-
-__global__ void k_add_counts(int32_t* __restrict__ total, const int32_t* __restrict__ add, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    total[i] += add[i];
 }
 
 // ---- stare ----
@@ -771,29 +957,8 @@ cudaError_t launch_count_nodes(const int32_t* nodes, const int32_t* samp, int64_
   return cudaGetLastError();
 }
 
-size_t scan_tmp_bytes(int64_t n) { return sizeof(long long) * (size_t)((n + SCAN_TILE - 1) / SCAN_TILE + 1); }
-
-cudaError_t launch_exclusive_scan(const int32_t* in, int64_t n, int64_t* out, void* tmp, cudaStream_t st,
-                                  int* launches) {
-  const int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-  long long* part = static_cast<long long*>(tmp);
-  k_tile_sums<<<(unsigned)tiles, 1024, 0, st>>>(in, n, part);
-  k_scan_parts<<<1, 1024, 0, st>>>(part, tiles);
-  k_tile_scan<<<(unsigned)tiles, 1024, 0, st>>>(in, n, part, out);
-  *launches += 3;
-  return cudaGetLastError();
-}
-
-cudaError_t launch_scatter_index(const int32_t* nodes, const int32_t* samp, int64_t e0, int64_t e1, int64_t jlo,
-                                 int64_t jhi, unsigned long long* cur, int32_t* inv_samp, cudaStream_t st,
-                                 int num_sms) {
-  if (e1 <= e0) return cudaSuccess;
-  k_scatter_index<<<grid_stride_blocks(e1 - e0, num_sms), TPB, 0, st>>>(nodes, samp, e0, e1, jlo, jhi, cur,
-                                                                        inv_samp);
-  return cudaGetLastError();
-}
-
 namespace {
+constexpr int GREEDY_SMEM = GCANDS * 12;  // candidates' gains, ids and list offsets
 // Largest cluster of 1024-thread greedy blocks the device can schedule (16 or
 // 8), 0 if none; computed once per process.
 int greedy_cluster_size() {
@@ -802,12 +967,15 @@ int greedy_cluster_size() {
   std::lock_guard<std::mutex> lock(mu);
   if (size >= 0) return size;
   size = 0;
+  if (cudaFuncSetAttribute(k_greedy<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GREEDY_SMEM) != cudaSuccess)
+    (void)cudaGetLastError();
   if (cudaFuncSetAttribute(k_greedy<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
     (void)cudaGetLastError();
   for (int c : {16, 8}) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(c);
     cfg.blockDim = dim3(1024);
+    cfg.dynamicSmemBytes = GREEDY_SMEM;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)c;
@@ -829,51 +997,42 @@ std::atomic<int> g_greedy_mode{0};
 
 void set_greedy_mode(int mode) { g_greedy_mode.store(mode); }
 
-cudaError_t launch_greedy(const GreedyJob& J, cudaStream_t st, int num_sms, int* blocks_used, bool shared_gpu) {
+cudaError_t launch_greedy(const GreedyJob& J, cudaStream_t st, int num_sms, bool shared_gpu) {
   // A solve that shares the GPU with others (serving) runs all picks of a pool
   // of up to GREEDY_CLUSTER_ENTRIES entries in one thread-block cluster: 16 SMs,
   // hardware cluster barriers, and the rest of the GPU free for the other
-  // solves.  Otherwise (and for larger pools, whose first picks decrement
-  // millions of gains) one 1024-thread block per SM in a cooperative launch,
-  // the faster shape for a solve that has the GPU to itself.
+  // solves.  Otherwise a cooperative grid of one 1024-thread block per SM, or
+  // a single block where the passes over counts and entries are too short to
+  // share.
   const int mode = g_greedy_mode.load();
   const int csize = mode == 1 ? 0 : greedy_cluster_size();
-  if (csize > 0 && (mode == 2 || (shared_gpu && J.total_entries <= GREEDY_CLUSTER_ENTRIES))) {
-    *blocks_used = csize;
-    cudaLaunchConfig_t cfg{};
+  const unsigned long long work = (unsigned long long)J.n_pad + J.total_entries;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[1];
+  cfg.blockDim = dim3(1024);
+  cfg.dynamicSmemBytes = GREEDY_SMEM;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  if (mode == 0 && work <= GREEDY_BLOCK_WORK) {
+    cfg.gridDim = dim3(1);
+  } else if (csize > 0 && (mode == 2 || (shared_gpu && J.total_entries <= GREEDY_CLUSTER_ENTRIES))) {
     cfg.gridDim = dim3(csize);
-    cfg.blockDim = dim3(1024);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)csize;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k_greedy<true>, J);
+  } else {
+    cfg.gridDim = dim3(num_sms);
+    // a cooperative launch (all blocks resident at once), also valid inside a stream capture
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.numAttrs = 1;
   }
-  // one 1024-thread block per SM: the fewest barrier arrivals with a full machine
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_greedy<false>, 1024, 0);
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_greedy<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, GREEDY_SMEM);
   if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const int blocks = num_sms;
-  // cache slices fit in shared memory; one tally slot and one reducing thread per block
-  if ((long long)blocks * HBINS < CACHE_MAX || blocks > 1024) return cudaErrorInvalidConfiguration;
-  *blocks_used = blocks;
-  // a cooperative launch (all blocks resident at once), also valid inside a stream capture
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(blocks);
-  cfg.blockDim = dim3(1024);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_greedy<false>, J);
 }
 
@@ -884,11 +1043,6 @@ cudaError_t device_code_version(int* binary, int* ptx) {
   *binary = a.binaryVersion;
   *ptx = a.ptxVersion;
   return cudaSuccess;
-}
-
-cudaError_t launch_add_counts(int32_t* total, const int32_t* add, int64_t n, cudaStream_t st, int num_sms) {
-  k_add_counts<<<grid_stride_blocks(n, num_sms, 4), TPB, 0, st>>>(total, add, n);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_mark_hits(const int32_t* nodes, const int32_t* samp, int64_t e0, int64_t e1,

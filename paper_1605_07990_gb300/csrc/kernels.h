@@ -154,61 +154,71 @@ size_t mid_queue_per_warp();
 cudaError_t launch_sample_warp(const SampleJob& J, const LaunchCfg& c, cudaStream_t st);
 cudaError_t launch_sample_cta(const SampleJob& J, const LaunchCfg& c, cudaStream_t st);
 
-// ---- index, greedy, stare -----------------------------------------------
+// ---- counts, greedy, stare ----------------------------------------------
 cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t st);
 // entries [e0, e1); with samp non-null only samples in [jlo, jhi) count
 cudaError_t launch_count_nodes(const int32_t* nodes, const int32_t* samp, int64_t e0, int64_t e1, int64_t jlo,
                                int64_t jhi, int32_t* cnt, cudaStream_t st, int num_sms);
-// exclusive scan of int32 counts into int64 offsets (n+1 outputs); tmp >= scan_tmp_bytes(n)
-size_t scan_tmp_bytes(int64_t n);
-cudaError_t launch_exclusive_scan(const int32_t* in, int64_t n, int64_t* out, void* tmp, cudaStream_t st,
-                                  int* launches);
-cudaError_t launch_scatter_index(const int32_t* nodes, const int32_t* samp, int64_t e0, int64_t e1, int64_t jlo,
-                                 int64_t jhi, unsigned long long* cur, int32_t* inv_samp, cudaStream_t st,
-                                 int num_sms);
 
-constexpr int GREEDY_MAX_LISTS = 48;
-struct InvList {
-  const int64_t* off;           // n+1 offsets of one index batch
-  const int32_t* samp;          // its sample ids
-};
 struct GreedyJob {
-  int32_t* cnt;                 // n_pad working gains; negative = picked or padding
-  int64_t n_pad;                // multiple of 4
-  InvList lists[GREEDY_MAX_LISTS];
-  int nlists;
-  const int32_t* pool_nodes;
+  const int32_t* cnt0;          // n_pad counts over the sets [0, n_sets); padding 0
+  int32_t* cnt;                 // n_pad working gains (written before they are read)
+  int64_t n, n_pad;             // nodes; padded to a multiple of 4
+  const int32_t* pool_nodes;    // entries [0, total_entries) hold the sets [0, n_sets), maybe others
+  const int32_t* pool_samp;
   const int64_t* set_start;
   const int32_t* set_len;
+  unsigned long long total_entries;
+  int64_t n_sets;               // N: sets [0, N) take part
+  int bulk_first;               // the first pick by a pass over the entries
   uint8_t* covered;             // per sample id, zeroed
   int32_t* seeds;               // k (device)
   int32_t* gains;               // k (device)
   int k;
-  unsigned long long* argmax;   // 64 + 2 x 1024 words, zeroed: 3 argmax slots 16 words apart,
-                                // then per-block covered-entry [64 + b] and queued-entry
-                                // [64 + 1024 + b] tallies
-  int64_t n_sets;               // N: sets [0, N) take part
-  unsigned long long total_entries;  // entries of those sets
-  unsigned int* sync;           // 128 words, zeroed: count [0], release word (64-bit) [32],
-                                // timeout flag [64], chunk-queue lengths [96], [112]
-  unsigned long long* chunk_q;  // (set, first member) of queued decrement chunks
-  int64_t chunk_cap;
-  unsigned int* hist;           // 2 x 4096 gain-histogram bins, zeroed
-  int32_t* cache;               // 2 x 8192 candidate nodes
-  unsigned int* cache_n;        // 2 counts, zeroed
+  // control block, zeroed: GREEDY_CTL_BYTES
+  unsigned int* sync;           // 128 words: count [0], release word (64-bit) [32], error flag [64]
+  unsigned long long* argmax;   // 3 slots 16 words apart
+  unsigned long long* nchunk;   // chunks handed out
+  unsigned int* ncand;          // candidates, chunk overflow, picks made, queued parts, list entries
+  unsigned int* hist;           // 4 x 1024 bins
+  unsigned int* blk;            // 1024: candidates among the nodes that a block numbers
+  // candidates of a session
+  unsigned int* mark;           // n_pad bits, zero between launches: the candidates
+  uint16_t* lid;                // n_pad, zero between launches: 1 + local id
+  int32_t* cand_id;             // GREEDY_CANDS node ids
+  int32_t* cand_len;            // gain when the lists were made = entries of the list
+  unsigned int* cand_off;       // first entry of the candidate's list
+  unsigned int* ents;           // ents_cap (+ GREEDY_ENTS_SPARE) first chunks of the candidates' sets
+  long long ents_cap;
+  uint4* chunks;                // chunk_cap (+ GREEDY_CHUNKS_SPARE) chunks of the sets' candidates
+  unsigned long long chunk_cap;
+  uint4* tasks;                 // parts of long sets (first chunk, set, first member): chunk_cap / 16 + 1
   long long wait_polls;         // polls after which a grid-barrier wait gives up
 };
+constexpr int GREEDY_CANDS = 16384;
+constexpr int GREEDY_ENTS_SPARE = 2048, GREEDY_CHUNKS_SPARE = 16;
+// byte offsets in the control block
+constexpr size_t GREEDY_CTL_ARGMAX = 512, GREEDY_CTL_NCHUNK = 896, GREEDY_CTL_NCAND = 912, GREEDY_CTL_HIST = 1024,
+                 GREEDY_CTL_BLK = 1024 + 4 * 1024 * 4, GREEDY_CTL_BYTES = GREEDY_CTL_BLK + 1024 * 4;
+// Pools of more entries make their first pick by a pass over the entries: the
+// pass costs a few us, the same pick out of the lists 0.1 us per 100 entries it
+// covers (104,000 of 195,660 entries: ~50 us).
+constexpr unsigned long long GREEDY_BULK_ENTRIES = 1ull << 18;
+// Counts and entries up to this many together are handled by a single block: it
+// saves the ~6 us of three grid barriers, but making the lists takes one block
+// 17-80 us from 10^4 to 4 x 10^4 entries on, a grid 6-8 us.
+constexpr unsigned long long GREEDY_BLOCK_WORK = 1ull << 13;
 constexpr long long GREEDY_DEFAULT_WAIT_POLLS = 1ll << 22;  // about a second with the poll back-off
 // Process-wide poll limit of the greedy kernel's grid-barrier waits (ssa_set_wait_polls).
 long long greedy_wait_polls();
-// All k picks in one launch: a cooperative grid (bounded grid barriers), or,
-// for a solve that shares the GPU with others and a pool of up to
-// GREEDY_CLUSTER_ENTRIES entries, one thread-block cluster.
+// All k picks in one launch: a cooperative grid (bounded grid barriers), a
+// single block for small pools, or, for a solve that shares the GPU with
+// others and a pool of up to GREEDY_CLUSTER_ENTRIES entries, one thread-block
+// cluster.
 constexpr unsigned long long GREEDY_CLUSTER_ENTRIES = 1ull << 26;
-cudaError_t launch_greedy(const GreedyJob& J, cudaStream_t st, int num_sms, int* blocks_used, bool shared_gpu);
+cudaError_t launch_greedy(const GreedyJob& J, cudaStream_t st, int num_sms, bool shared_gpu);
 // 0: by the rule above (default); 1: always the cooperative grid; 2: always a cluster (when the device has one)
 void set_greedy_mode(int mode);
-cudaError_t launch_add_counts(int32_t* total, const int32_t* add, int64_t n, cudaStream_t st, int num_sms);
 // SASS and PTX versions (major*10 + minor) of the device code the CUDA runtime loaded for this library
 cudaError_t device_code_version(int* binary, int* ptx);
 
