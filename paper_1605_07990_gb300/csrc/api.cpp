@@ -102,8 +102,9 @@ struct ssa_graph {
   int device = 0;
   int64_t n = 0, m = 0;
   int weighting = 0;
-  int64_t* off = nullptr;
-  uint2* edge = nullptr;
+  uint32_t* off = nullptr;
+  uint32_t* src = nullptr;
+  uint32_t* thr = nullptr;       // stored thresholds (see GraphView)
   uint64_t* wc_pow = nullptr;  // weighted cascade: gap powers per in-degree (build_wc_pow)
   int wc_pow_k = 0;
   int64_t bytes = 0;
@@ -119,7 +120,8 @@ struct ssa_graph {
     v.n = n;
     v.m = m;
     v.off = off;
-    v.edge = edge;
+    v.src = src;
+    v.thr = thr;
     v.wc_pow = wc_pow;
     v.wc_pow_k = wc_pow_k;
     return v;
@@ -1430,12 +1432,15 @@ ssa_status ssa_load_graph(int64_t n, int64_t m, const int32_t* src, const int32_
   do {
     const int64_t m_pad = ((m + 3) / 4) * 4 + 4;
     if ((rc = dev_alloc(&g->off, (size_t)n + 1, st)) != SSA_OK) break;
-    if ((rc = dev_alloc(&g->edge, (size_t)m_pad, st)) != SSA_OK) break;
-    if (cudaMemsetAsync(g->edge, 0, sizeof(uint2) * (size_t)m_pad, st) != cudaSuccess) {
+    if ((rc = dev_alloc(&g->src, (size_t)m_pad, st)) != SSA_OK) break;
+    const bool stored = weighting == SSA_W_EXPLICIT || (weighting == SSA_W_TRIVALENCY && n > TRI_PACK_NODES);
+    if (stored && (rc = dev_alloc(&g->thr, (size_t)m_pad, st)) != SSA_OK) break;
+    if (cudaMemsetAsync(g->src, 0, sizeof(uint32_t) * (size_t)m_pad, st) != cudaSuccess ||
+        (stored && cudaMemsetAsync(g->thr, 0, sizeof(uint32_t) * (size_t)m_pad, st) != cudaSuccess)) {
       rc = fail(SSA_E_CUDA, "memset failed");
       break;
     }
-    g->bytes = (int64_t)(sizeof(int64_t) * (size_t)(n + 1) + sizeof(uint2) * (size_t)m_pad);
+    g->bytes = (int64_t)(sizeof(uint32_t) * ((size_t)(n + 1) + (size_t)m_pad * (stored ? 2 : 1)));
     if ((rc = dev_alloc(&d_err, 1, st)) != SSA_OK) break;
     cudaMemsetAsync(d_err, 0, sizeof(unsigned int), st);
     if (m > 0) {
@@ -1449,7 +1454,7 @@ ssa_status ssa_load_graph(int64_t n, int64_t m, const int32_t* src, const int32_
       }
     }
     int launches = 0;
-    cudaError_t e = build_graph(n, m, d_src, d_dst, d_thr, weighting, weight_seed, g->off, g->edge, d_err, st,
+    cudaError_t e = build_graph(n, m, d_src, d_dst, d_thr, weighting, weight_seed, g->off, g->src, g->thr, d_err, st,
                                 &launches);
     if (e != cudaSuccess) {
       rc = fail(e == cudaErrorMemoryAllocation ? SSA_E_NOMEM : SSA_E_CUDA, "graph build: %s", cudaGetErrorString(e));
@@ -1483,7 +1488,8 @@ ssa_status ssa_load_graph(int64_t n, int64_t m, const int32_t* src, const int32_
   cudaStreamDestroy(st);
   if (rc != SSA_OK) {
     if (g->off) cudaFree(g->off);
-    if (g->edge) cudaFree(g->edge);
+    if (g->src) cudaFree(g->src);
+    if (g->thr) cudaFree(g->thr);
     if (g->wc_pow) cudaFree(g->wc_pow);
     delete g;
     return rc;
@@ -1520,21 +1526,22 @@ ssa_status ssa_gen_rmat(int32_t scale, int64_t m_draw, double a, double b, doubl
   int launches = 0;
   int64_t m = 0;
   cudaError_t e = rmat_graph(scale, m_draw, prob_threshold(a), prob_threshold(a + b), prob_threshold(a + b + c), seed,
-                             (int)weighting, weight_seed, &m, &g->off, &g->edge, st, &launches);
+                             (int)weighting, weight_seed, &m, &g->off, &g->src, st, &launches);
   if (e == cudaSuccess && weighting == SSA_W_WC) e = build_wc_pow(g->off, g->n, &g->wc_pow, &g->wc_pow_k, st);
   const cudaError_t e2 = cudaStreamSynchronize(st);
   cudaStreamDestroy(st);
   if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) {
     if (g->off) cudaFree(g->off);
-    if (g->edge) cudaFree(g->edge);
+    if (g->src) cudaFree(g->src);
+    if (g->thr) cudaFree(g->thr);
     if (g->wc_pow) cudaFree(g->wc_pow);
     delete g;
     return fail(e == cudaErrorMemoryAllocation ? SSA_E_NOMEM : SSA_E_CUDA, "R-MAT generation: %s",
                 cudaGetErrorString(e));
   }
   g->m = m;
-  g->bytes = (int64_t)(sizeof(int64_t) * (size_t)(g->n + 1) + sizeof(uint2) * (size_t)(((m + 3) / 4) * 4 + 4));
+  g->bytes = (int64_t)(sizeof(uint32_t) * ((size_t)(g->n + 1) + (size_t)(((m + 3) / 4) * 4 + 4)));
   if (g->wc_pow_k > 0) g->bytes += (int64_t)(sizeof(uint64_t) * (((size_t)g->wc_pow_k - 1) << g->wc_pow_k) + 8);
   *out = g;
   return SSA_OK;
@@ -1544,7 +1551,8 @@ ssa_status ssa_free_graph(ssa_graph* g) {
   if (!g) return SSA_OK;
   cudaDeviceSynchronize();
   if (g->off) cudaFree(g->off);
-  if (g->edge) cudaFree(g->edge);
+  if (g->src) cudaFree(g->src);
+  if (g->thr) cudaFree(g->thr);
   if (g->wc_pow) cudaFree(g->wc_pow);
   delete g;
   return SSA_OK;
@@ -1560,15 +1568,31 @@ ssa_status ssa_graph_info(const ssa_graph* g, int64_t* n, int64_t* m, int64_t* b
 
 ssa_status ssa_graph_export(const ssa_graph* g, int64_t* off, int32_t* src, uint32_t* thr) {
   if (!g) return fail(SSA_E_ARG, "null graph");
-  if (off) CU(cudaMemcpy(off, g->off, sizeof(int64_t) * (size_t)(g->n + 1), cudaMemcpyDeviceToHost));
-  if ((src || thr) && g->m > 0) {
-    std::vector<uint2> e((size_t)g->m);
-    CU(cudaMemcpy(e.data(), g->edge, sizeof(uint2) * (size_t)g->m, cudaMemcpyDeviceToHost));
-    for (int64_t i = 0; i < g->m; ++i) {
-      if (src) src[i] = (int32_t)e[(size_t)i].x;
-      if (thr) thr[i] = e[(size_t)i].y;
+  const size_t n = (size_t)g->n, m = (size_t)g->m;
+  std::vector<uint32_t> o;
+  if (off || (thr && g->weighting == SSA_W_WC)) {
+    o.resize(n + 1);
+    CU(cudaMemcpy(o.data(), g->off, sizeof(uint32_t) * (n + 1), cudaMemcpyDeviceToHost));
+  }
+  if (off)
+    for (size_t v = 0; v <= n; ++v) off[v] = (int64_t)o[v];
+  if (m == 0) return SSA_OK;
+  const bool packed = g->weighting == SSA_W_TRIVALENCY && !g->thr;
+  const uint32_t tri[4] = {TRI_THR0, TRI_THR1, TRI_THR2, 0u};
+  if (src || (thr && packed)) {
+    std::vector<uint32_t> e(m);
+    CU(cudaMemcpy(e.data(), g->src, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost));
+    for (size_t i = 0; i < m; ++i) {
+      if (src) src[i] = (int32_t)(packed ? e[i] & TRI_SRC_MASK : e[i]);
+      if (thr && packed) thr[i] = tri[e[i] >> 30];
     }
   }
+  if (thr && g->thr) CU(cudaMemcpy(thr, g->thr, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost));
+  if (thr && g->weighting == SSA_W_WC)
+    for (size_t v = 0; v < n; ++v) {
+      const uint32_t d = o[v + 1] - o[v];
+      for (uint32_t i = o[v]; i < o[v + 1]; ++i) thr[i] = d == 1 ? 0xFFFFFFFFu : (uint32_t)((uint64_t(1) << 32) / d);
+    }
   return SSA_OK;
 }
 

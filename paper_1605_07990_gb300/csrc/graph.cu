@@ -29,33 +29,30 @@ __global__ void k_make_keys(const int32_t* src, const int32_t* dst, int64_t n, i
 }
 
 // off[v] = first sorted position whose dst >= v.
-__global__ void k_offsets(const unsigned long long* keys, int64_t n, int64_t m, int bits, int64_t* off) {
+__global__ void k_offsets(const unsigned long long* keys, int64_t n, int64_t m, int bits, uint32_t* off) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e <= m; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t prev = (e == 0) ? -1 : (int64_t)(keys[e - 1] >> bits);
     const int64_t cur = (e == m) ? n : (int64_t)(keys[e] >> bits);
-    for (int64_t v = prev + 1; v <= cur; ++v) off[v] = e;
+    for (int64_t v = prev + 1; v <= cur; ++v) off[v] = (uint32_t)e;
   }
 }
 
-__global__ void k_fill_edges(const unsigned long long* keys, const int32_t* vals, const int64_t* off, int64_t m,
-                             int bits, int weighting, uint64_t weight_seed, const uint32_t* thr_in, uint2* edge) {
+// src (and thr where given): weighting 0 stores no weight, 1 the trivalency
+// class in src's high bits or, with thr, the threshold, 2 the given threshold
+__global__ void k_fill_edges(const unsigned long long* keys, const int32_t* vals, int64_t m, int bits, int weighting,
+                             uint64_t weight_seed, const uint32_t* thr_in, uint32_t* src, uint32_t* thr) {
   const unsigned long long mask = (1ull << bits) - 1ull;
-  const uint32_t TRI[3] = {429496729u, 42949672u, 4294967u};  // floor(2^32 p), p = 0.1, 0.01, 0.001
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long k = keys[e];
-    const uint32_t s = (uint32_t)(k & mask);
-    uint32_t t;
-    if (weighting == 0) {
-      const int64_t v = (int64_t)(k >> bits);
-      const uint64_t d = (uint64_t)(off[v + 1] - off[v]);
-      t = (d == 1) ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / d);
-    } else if (weighting == 1) {
+    uint32_t s = (uint32_t)(keys[e] & mask);
+    if (weighting == 1) {
       const uint4 r = keyed_draw(weight_seed, PURPOSE_WEIGHT, 0, 0, (uint64_t)e);
-      t = TRI[__umulhi(r.x, 3u)];
-    } else {
-      t = thr_in[vals[e]];
+      const uint32_t c = __umulhi(r.x, 3u);
+      if (thr) thr[e] = c == 0u ? TRI_THR0 : c == 1u ? TRI_THR1 : TRI_THR2;
+      else s |= c << 30;
+    } else if (weighting == 2) {
+      thr[e] = thr_in[vals[e]];
     }
-    edge[e] = make_uint2(s, t);
+    src[e] = s;
   }
 }
 
@@ -101,7 +98,7 @@ int grid_for(int64_t work, int threads) {
 }  // namespace
 
 cudaError_t rmat_graph(int scale, int64_t m_draw, uint32_t ta, uint32_t tab, uint32_t tabc, uint64_t seed,
-                       int weighting, uint64_t weight_seed, int64_t* m_out, int64_t** d_off, uint2** d_edge,
+                       int weighting, uint64_t weight_seed, int64_t* m_out, uint32_t** d_off, uint32_t** d_src,
                        cudaStream_t st, int* launches) {
   const int64_t n = int64_t(1) << scale;
   const unsigned long long drop = 1ull << (2 * scale);  // after every (dst, src) key
@@ -111,7 +108,7 @@ cudaError_t rmat_graph(int scale, int64_t m_draw, uint32_t ta, uint32_t tab, uin
   void* tmp = nullptr;
   size_t tmp_sort = 0, tmp_uniq = 0;
   *d_off = nullptr;
-  *d_edge = nullptr;
+  *d_src = nullptr;
   cudaError_t e = cudaSuccess;
   do {
     const size_t cnt = (size_t)(m_draw > 0 ? m_draw : 1);
@@ -147,16 +144,16 @@ cudaError_t rmat_graph(int scale, int64_t m_draw, uint32_t ta, uint32_t tab, uin
       m = (uniq > 0 && last == drop) ? uniq - 1 : uniq;
     }
     const int64_t m_pad = ((m + 3) / 4) * 4 + 4;
-    if ((e = cudaMallocAsync(d_off, sizeof(int64_t) * (size_t)(n + 1), st)) != cudaSuccess) break;
-    if ((e = cudaMallocAsync(d_edge, sizeof(uint2) * (size_t)m_pad, st)) != cudaSuccess) break;
-    if ((e = cudaMemsetAsync(*d_edge, 0, sizeof(uint2) * (size_t)m_pad, st)) != cudaSuccess) break;
+    if ((e = cudaMallocAsync(d_off, sizeof(uint32_t) * (size_t)(n + 1), st)) != cudaSuccess) break;
+    if ((e = cudaMallocAsync(d_src, sizeof(uint32_t) * (size_t)m_pad, st)) != cudaSuccess) break;
+    if ((e = cudaMemsetAsync(*d_src, 0, sizeof(uint32_t) * (size_t)m_pad, st)) != cudaSuccess) break;
     if (m == 0) {
-      e = cudaMemsetAsync(*d_off, 0, sizeof(int64_t) * (size_t)(n + 1), st);
+      e = cudaMemsetAsync(*d_off, 0, sizeof(uint32_t) * (size_t)(n + 1), st);
     } else {
       // the unique keys are the CSR order (dst, src): offsets and records as for a loaded graph
       k_offsets<<<grid_for(m + 1, 256), 256, 0, st>>>(k_in, n, m, scale, *d_off);
-      k_fill_edges<<<grid_for(m, 256), 256, 0, st>>>(k_in, nullptr, *d_off, m, scale, weighting, weight_seed,
-                                                     nullptr, *d_edge);
+      k_fill_edges<<<grid_for(m, 256), 256, 0, st>>>(k_in, nullptr, m, scale, weighting, weight_seed, nullptr, *d_src,
+                                                     nullptr);
       *launches += 2;
       e = cudaGetLastError();
     }
@@ -168,21 +165,21 @@ cudaError_t rmat_graph(int scale, int64_t m_draw, uint32_t ta, uint32_t tab, uin
   if (tmp) cudaFreeAsync(tmp, st);
   if (e != cudaSuccess) {
     if (*d_off) cudaFreeAsync(*d_off, st);
-    if (*d_edge) cudaFreeAsync(*d_edge, st);
+    if (*d_src) cudaFreeAsync(*d_src, st);
     *d_off = nullptr;
-    *d_edge = nullptr;
+    *d_src = nullptr;
   }
   return e;
 }
 
 cudaError_t build_graph(int64_t n, int64_t m, const int32_t* d_src, const int32_t* d_dst, const uint32_t* d_thr_in,
-                        int weighting, uint64_t weight_seed, int64_t* d_off, uint2* d_edge, unsigned int* d_err,
-                        cudaStream_t st, int* launches) {
+                        int weighting, uint64_t weight_seed, uint32_t* d_off, uint32_t* d_src_out, uint32_t* d_thr,
+                        unsigned int* d_err, cudaStream_t st, int* launches) {
   int bits = 1;
   while ((1ll << bits) < n) ++bits;
   cudaError_t e = cudaSuccess;
   if (m == 0) {
-    e = cudaMemsetAsync(d_off, 0, sizeof(int64_t) * (size_t)(n + 1), st);
+    e = cudaMemsetAsync(d_off, 0, sizeof(uint32_t) * (size_t)(n + 1), st);
     return e;
   }
   unsigned long long *k_in = nullptr, *k_out = nullptr;
@@ -208,8 +205,8 @@ cudaError_t build_graph(int64_t n, int64_t m, const int32_t* d_src, const int32_
     k_offsets<<<grid_for(m + 1, 256), 256, 0, st>>>(k_out, n, m, bits, d_off);
     ++*launches;
     if ((e = cudaGetLastError()) != cudaSuccess) break;
-    k_fill_edges<<<grid_for(m, 256), 256, 0, st>>>(k_out, v_out, d_off, m, bits, weighting, weight_seed, d_thr_in,
-                                                   d_edge);
+    k_fill_edges<<<grid_for(m, 256), 256, 0, st>>>(k_out, v_out, m, bits, weighting, weight_seed, d_thr_in, d_src_out,
+                                                   d_thr);
     ++*launches;
     e = cudaGetLastError();
   } while (false);
@@ -222,7 +219,7 @@ cudaError_t build_graph(int64_t n, int64_t m, const int32_t* d_src, const int32_
 }
 
 namespace {
-__global__ void k_max_in_degree(const int64_t* off, int64_t n, unsigned long long* out) {
+__global__ void k_max_in_degree(const uint32_t* off, int64_t n, unsigned long long* out) {
   unsigned long long best = 0;
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
     const unsigned long long d = (unsigned long long)(off[v + 1] - off[v]);
@@ -255,7 +252,7 @@ __global__ void k_wc_pow_rows(uint64_t* tab, int K) {
 }
 }  // namespace
 
-cudaError_t build_wc_pow(const int64_t* d_off, int64_t n, uint64_t** tab, int* k_out, cudaStream_t st) {
+cudaError_t build_wc_pow(const uint32_t* d_off, int64_t n, uint64_t** tab, int* k_out, cudaStream_t st) {
   *tab = nullptr;
   *k_out = 0;
   unsigned long long* d_max = nullptr;

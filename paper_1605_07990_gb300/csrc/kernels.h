@@ -9,13 +9,24 @@ namespace ssa {
 // Sets the calling thread's message returned by ssa_last_error().
 void set_last_error(const char* msg);
 
-// Device-resident in-edge CSR (Sec. 2).  Edge records interleave the tail
-// node and the uint32 live threshold so one 8-byte load serves an edge and a
-// 4-edge group (the unit of one Philox draw) is one aligned 32-byte sector.
+// Device-resident in-edge CSR (Sec. 2).  Positions fit 32 bits (m < 2^31), and
+// what a sampler can do without is not stored beside what it reads: a random
+// access moves a 32-byte sector, and what stays in the 129 MB L2 decides the rate.
+//   off   n+1 positions
+//   src   the tail node of every in-edge.  Weighted cascade stores nothing else:
+//         its threshold follows from the in-degree.  Trivalency (n <= 2^30) keeps
+//         the edge's class (0.1, 0.01, 0.001) in the two high bits.
+//   thr   uint32 live thresholds: explicit weights, and trivalency beyond 2^30 nodes
+// A 4-edge group (the unit of one Philox draw) is one aligned 16-byte load of each.
+// Against 64-bit offsets and 8-byte {src, thr} records, on GB300: half the graph
+// memory (5.3 for 10.5 GB at 1.26e9 edges) at the same speed for weighted
+// cascade (latency-bound); trivalency graphs of 16M edges (64 MB) stay in L2
+// whole, where the coin kernels read them (hit rate 64 -> 91%).
 struct GraphView {
   int64_t n = 0, m = 0;
-  const int64_t* off = nullptr;  // n+1
-  const uint2* edge = nullptr;   // m rounded up to a multiple of 4 (+4): {src, thr}
+  const uint32_t* off = nullptr;  // n+1
+  const uint32_t* src = nullptr;  // m rounded up to a multiple of 4 (+4)
+  const uint32_t* thr = nullptr;  // as src, or null
   // weighted cascade: the gap form's powers q^(2^i) of every in-degree d < 2^wc_pow_k
   // (rows of bit-length entries, in order of d; null / 0 for other weightings)
   const uint64_t* wc_pow = nullptr;
@@ -28,7 +39,7 @@ constexpr int WC_POW_K = 20;
 
 // The weighted-cascade power table of a CSR (rows for every in-degree below
 // min(2^WC_POW_K, 2 * max in-degree)); *tab stays null when no in-list has 2 edges.
-cudaError_t build_wc_pow(const int64_t* d_off, int64_t n, uint64_t** tab, int* k, cudaStream_t st);
+cudaError_t build_wc_pow(const uint32_t* d_off, int64_t n, uint64_t** tab, int* k, cudaStream_t st);
 
 // Device counters of one sampling batch.
 // Bounded waits of the weighted-cascade CTA tier that gave up (Counters::error).
@@ -126,20 +137,26 @@ struct LaunchCfg {
   int64_t smem_bitmap_bytes = 0;
 };
 
+// Trivalency classes ride in the two high bits of src up to this many nodes.
+constexpr int64_t TRI_PACK_NODES = int64_t(1) << 30;
+constexpr uint32_t TRI_SRC_MASK = 0x3FFFFFFFu;
+constexpr uint32_t TRI_THR0 = 429496729u, TRI_THR1 = 42949672u, TRI_THR2 = 4294967u;  // floor(2^32 p), p = 0.1, 0.01, 0.001
+
 // ---- graph build -------------------------------------------------------
-// Sorts edges by (dst, src, input position), builds off/edge records and
-// thresholds.  d_src/d_dst/d_thr_in are device arrays of length m.
+// Sorts edges by (dst, src, input position), builds off, src and (for weights
+// that keep them: d_thr not null) thr.  d_src/d_dst/d_thr_in are device arrays
+// of length m.
 cudaError_t build_graph(int64_t n, int64_t m, const int32_t* d_src, const int32_t* d_dst,
                         const uint32_t* d_thr_in, int weighting, uint64_t weight_seed,
-                        int64_t* d_off, uint2* d_edge, unsigned int* d_err, cudaStream_t st,
+                        uint32_t* d_off, uint32_t* d_src_out, uint32_t* d_thr, unsigned int* d_err, cudaStream_t st,
                         int* launches);
 
 // Directed R-MAT graph on 2^scale nodes from m_draw SplitMix64-keyed draws
 // (quadrant thresholds ta < tab < tabc of a 32-bit draw), self-loops and
 // duplicates removed, built straight into the in-edge CSR (allocated here,
-// stream-ordered; the caller owns *d_off and *d_edge).  *m_out: unique edges.
+// stream-ordered; the caller owns *d_off and *d_src).  *m_out: unique edges.
 cudaError_t rmat_graph(int scale, int64_t m_draw, uint32_t ta, uint32_t tab, uint32_t tabc, uint64_t seed,
-                       int weighting, uint64_t weight_seed, int64_t* m_out, int64_t** d_off, uint2** d_edge,
+                       int weighting, uint64_t weight_seed, int64_t* m_out, uint32_t** d_off, uint32_t** d_src,
                        cudaStream_t st, int* launches);
 
 // ---- sampling -----------------------------------------------------------

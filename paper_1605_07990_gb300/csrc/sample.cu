@@ -10,10 +10,14 @@
 //     (shared memory when it fits, else a per-CTA global slot).
 // IC with per-edge thresholds: frontier expansion is edge-balanced inside a
 // warp: 32 frontier nodes' in-edge ranges are cut into 4-edge groups (the
-// unit of one Philox draw, one aligned 32-byte sector of {src,thr} records)
-// dealt to lanes by a warp prefix sum; the CTA tier skips the draw of a group
-// whose edges all come from already-visited nodes and shares long in-lists
-// between its warps.
+// unit of one Philox draw, one aligned 16-byte load of tails) dealt to lanes by
+// a warp prefix sum, every group draws its coins, and the live tails are
+// visited 32 at a time; the CTA tier shares long in-lists between its warps.
+// Bound: integer issue (ALU pipe 58%, multiplier 52%, 69% of issue slots), 102
+// instructions per 32 groups, 39 of them Philox.  On the 2^20-node trivalency
+// R-MAT graph (giant sets of 137,000 nodes) 350 -> 205 ms of sampling per
+// D-SSA solve, 5.1e10 -> 1.5e11 draws/s over the solve, against the form that
+// asked for each tail first and visited slab by slab.
 // IC with weighted-cascade weights: every in-edge of a node has the same
 // probability, so each lane walks one frontier node's in-list by geometric
 // gaps between live edges (the gap form below); the work per node is a few
@@ -30,10 +34,19 @@ constexpr int WT_WARPS = 8;      // warps per warp-tier block
 constexpr int WT_HASH = 1024;    // hash slots per warp (power of two)
 constexpr int WT_QCAP = 512;     // largest IC set kept in the warp tier
 constexpr int LT_QCAP = 1024;    // largest LT walk kept in the warp tier
-constexpr int STAGE = 128;       // live candidates of one slab (32 lanes x 4 edges)
+constexpr int STAGE = 160;       // live tails waiting for a visit: 31 and those of one slab (32 lanes x 4 edges)
 constexpr int CTA_HEAVY_GROUPS = 512;    // the CTA tier splits longer in-lists over all its warps
 constexpr int CTA_HEAVY_CAP = 256;       // heavy in-lists per level shared this way
 constexpr int SMALL_CTA_THREADS = 128;   // CTAs of the first stage when the visited bitmap is in global memory
+
+// How a sampler kernel learns which edges are live: coins against stored
+// thresholds (the LT walk runs in this instantiation too), weighted-cascade
+// gaps, or coins against packed trivalency classes.
+enum : int { W_COINS = 0, W_GAPS = 1, W_TRI = 2 };
+inline int weights_of(const SampleJob& J) {
+  if (J.model != 0) return W_COINS;
+  return J.wc_implicit ? W_GAPS : J.g.thr ? W_COINS : W_TRI;
+}
 
 constexpr uint32_t PHILOX_M0 = 0xD2511F53u, PHILOX_M1 = 0xCD9E8D57u;
 
@@ -52,29 +65,29 @@ __device__ __forceinline__ SampleConst sample_const(const uint32_t* rk, uint32_t
   return c;
 }
 
-__device__ __forceinline__ uint4 philox_x(uint32_t x, const SampleConst& sc, const uint32_t* rk) {
-  // round 1 with c.y = 0 and the sample constants folded in
-  uint4 c = make_uint4(sc.s0, sc.s1, __umulhi(PHILOX_M0, x) ^ sc.s2, PHILOX_M0 * x);
+// Rounds 2 to 10.  Both halves of a product come from one 32x32->64 multiply
+// (one instruction; asked for as a low and a high product they are two).
+__device__ __forceinline__ uint4 philox_rounds(uint4 c, const uint32_t* rk) {
 #pragma unroll
   for (int r = 1; r < 10; ++r) {
-    const uint32_t lo0 = PHILOX_M0 * c.x, hi0 = __umulhi(PHILOX_M0, c.x);
-    const uint32_t lo1 = PHILOX_M1 * c.z, hi1 = __umulhi(PHILOX_M1, c.z);
-    c = make_uint4(hi1 ^ c.y ^ rk[2 * r], lo1, hi0 ^ c.w ^ rk[2 * r + 1], lo0);
+    const uint64_t p0 = (uint64_t)PHILOX_M0 * c.x, p1 = (uint64_t)PHILOX_M1 * c.z;
+    c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ rk[2 * r], (uint32_t)p1,
+                   (uint32_t)(p0 >> 32) ^ c.w ^ rk[2 * r + 1], (uint32_t)p0);
   }
   return c;
+}
+
+__device__ __forceinline__ uint4 philox_x(uint32_t x, const SampleConst& sc, const uint32_t* rk) {
+  // round 1 with c.y = 0 and the sample constants folded in
+  const uint64_t p = (uint64_t)PHILOX_M0 * x;
+  return philox_rounds(make_uint4(sc.s0, sc.s1, (uint32_t)(p >> 32) ^ sc.s2, (uint32_t)p), rk);
 }
 
 // Philox4x32-10 of the counter (x, y, jlo, cw): philox_x with a second
 // counter word y, which enters the first round beside the sample constants.
 __device__ __forceinline__ uint4 philox_xy(uint32_t x, uint32_t y, const SampleConst& sc, const uint32_t* rk) {
-  uint4 c = make_uint4(sc.s0 ^ y, sc.s1, __umulhi(PHILOX_M0, x) ^ sc.s2, PHILOX_M0 * x);
-#pragma unroll
-  for (int r = 1; r < 10; ++r) {
-    const uint32_t lo0 = PHILOX_M0 * c.x, hi0 = __umulhi(PHILOX_M0, c.x);
-    const uint32_t lo1 = PHILOX_M1 * c.z, hi1 = __umulhi(PHILOX_M1, c.z);
-    c = make_uint4(hi1 ^ c.y ^ rk[2 * r], lo1, hi0 ^ c.w ^ rk[2 * r + 1], lo0);
-  }
-  return c;
+  const uint64_t p = (uint64_t)PHILOX_M0 * x;
+  return philox_rounds(make_uint4(sc.s0 ^ y, sc.s1, (uint32_t)(p >> 32) ^ sc.s2, (uint32_t)p), rk);
 }
 
 __device__ __forceinline__ int64_t sample_at(const SampleJob& J, unsigned long long idx) {
@@ -136,76 +149,90 @@ __device__ __forceinline__ bool hash_insert(uint32_t* H, uint32_t u, uint32_t* s
   return false;  // not reached: the table is never more than half full
 }
 
-template <class Visit>
-__device__ __forceinline__ bool deliver(uint32_t cand, uint32_t u0, uint32_t u1, uint32_t u2, uint32_t u3, int lane,
-                                        uint32_t* stage, Visit&& visit);
-
-// One slab: each lane holds one 4-edge group `grp` of an in-list [olo, ohi)
-// (when `valid`).  Edges whose tail may be new draw their coins; the live
-// ones are compacted through `stage` (STAGE entries, private to the warp) and
-// handed to visit(u) in rounds of 32 (NO_NODE for idle lanes).  known(u) may
-// report tails already in the set so their edges need no draw.  Returns the
-// warp-uniform "stop" of visit.
-template <class Known, class Visit>
-__device__ __forceinline__ bool process_slab(const GraphView& g, bool valid, uint32_t grp, uint32_t olo, uint32_t ohi,
-                                             const uint32_t* rk, const SampleConst& sc, int lane, uint32_t* stage,
-                                             unsigned long long& draws, Known&& known, Visit&& visit) {
-  uint32_t cand = 0, u0 = 0, u1 = 0, u2 = 0, u3 = 0;
-  if (valid) {
-    const uint32_t e = grp * 4u;
-    // edges e..e+3 that belong to the in-list
-    const uint32_t a = olo > e ? olo - e : 0u;
-    const uint32_t b = ohi - e;
-    uint32_t need = (b >= 4u ? 0xFu : ((1u << b) - 1u)) & ((0xFu << a) & 0xFu);
-    const uint4* p = reinterpret_cast<const uint4*>(g.edge) + (size_t)grp * 2;
-    const uint4 A = __ldg(p), B = __ldg(p + 1);
-    u0 = A.x; u1 = A.z; u2 = B.x; u3 = B.z;
-    if ((need & 1u) && known(u0)) need &= ~1u;
-    if ((need & 2u) && known(u1)) need &= ~2u;
-    if ((need & 4u) && known(u2)) need &= ~4u;
-    if ((need & 8u) && known(u3)) need &= ~8u;
-    if (need) {
-      ++draws;
-      const uint4 r = philox_x(grp, sc, rk);
-      if ((need & 1u) && edge_live(r.x, A.y)) cand |= 1u;
-      if ((need & 2u) && edge_live(r.y, A.w)) cand |= 2u;
-      if ((need & 4u) && edge_live(r.z, B.y)) cand |= 4u;
-      if ((need & 8u) && edge_live(r.w, B.w)) cand |= 8u;
-    }
-  }
-  return deliver(cand, u0, u1, u2, u3, lane, stage, visit);
+// Threshold of a packed trivalency edge (its class in the two high bits).
+__device__ __forceinline__ uint32_t tri_thr(uint32_t s) {
+  return (s >> 31) ? TRI_THR2 : (s >> 30) ? TRI_THR1 : TRI_THR0;
 }
 
-// Hand the live candidates of one slab (lane-held masks over 4 tails) to
-// visit(u) in rounds of 32 (NO_NODE for idle lanes), compacted through
-// `stage` when some lane holds more than one.  Returns visit's "stop".
+// Live tails wait in a warp's stage (shared memory: STAGE entries and their
+// count) until 32 of them are there, so that the visits -- a look at the visited
+// set, an atomic, a queue slot -- run with full warps.  A slab of 32 groups
+// gives 4 to 5 live tails under trivalency; visited one slab at a time they
+// took longer than the coins.
+struct Stage {
+  uint32_t* buf;
+  unsigned int* cnt;
+};
+
+// Visit staged tails, 32 at a time; `all`: also the last ones.  Returns the
+// warp-uniform "stop" of visit, after which the stage is empty.
 template <class Visit>
-__device__ __forceinline__ bool deliver(uint32_t cand, uint32_t u0, uint32_t u1, uint32_t u2, uint32_t u3, int lane,
-                                        uint32_t* stage, Visit&& visit) {
-  const unsigned lt_mask = (1u << lane) - 1u;
-  const unsigned any = __ballot_sync(FULL_MASK, cand != 0u);
-  if (!any) return false;
-  if (!__any_sync(FULL_MASK, (cand & (cand - 1u)) != 0u)) {
-    // at most one candidate per lane (the common case): no staging
-    const uint32_t u = !cand ? NO_NODE : (cand & 1u) ? u0 : (cand & 2u) ? u1 : (cand & 4u) ? u2 : u3;
-    return visit(u, lt_mask);
-  }
-  const int c = __popc(cand);
-  const int cin = warp_inclusive_scan(c, lane);
-  const int ctot = __shfl_sync(FULL_MASK, cin, 31);
-  int pos = cin - c;
-  if (cand & 1u) stage[pos++] = u0;
-  if (cand & 2u) stage[pos++] = u1;
-  if (cand & 4u) stage[pos++] = u2;
-  if (cand & 8u) stage[pos++] = u3;
+__device__ __forceinline__ bool drain(const Stage& st, bool all, int lane, Visit&& visit) {
   __syncwarp();
+  int n = (int)*(volatile unsigned int*)st.cnt;
+  if (n < 32 && !(all && n > 0)) return false;
+  const unsigned lt_mask = (1u << lane) - 1u;
   bool stop = false;
-  for (int s0 = 0; s0 < ctot && !stop; s0 += 32) {
-    const uint32_t u = (s0 + lane < ctot) ? stage[s0 + lane] : NO_NODE;
+  do {
+    const int take = min(n, 32);
+    n -= take;
+    const uint32_t u = lane < take ? st.buf[n + lane] : NO_NODE;
     stop = visit(u, lt_mask);
-  }
+  } while (!stop && (n >= 32 || (all && n > 0)));
+  __syncwarp();
+  if (lane == 0) *st.cnt = stop ? 0u : (unsigned int)n;
   __syncwarp();
   return stop;
+}
+
+// Two 4-edge groups per lane, gA and gB of the in-lists [loA, hiA) and
+// [loB, hiB) (when vA, vB): coins for their edges (the tails' loads are in
+// flight meanwhile), live tails to the stage, full rounds of visits.  Returns
+// visit's "stop".  Whether a tail is in the set already is only asked of live
+// ones: asking first saves the draws of 43% of the groups of a trivalency set,
+// but a warp draws as long as one lane must.
+template <bool TRI, class Visit>
+__device__ __forceinline__ bool two_groups(const GraphView& g, bool vA, uint32_t gA, uint32_t loA, uint32_t hiA,
+                                           bool vB, uint32_t gB, uint32_t loB, uint32_t hiB, const uint32_t* rk,
+                                           const SampleConst& sc, int lane, const Stage& st, Visit&& visit) {
+  uint4 sA = make_uint4(0u, 0u, 0u, 0u), sB = sA, tA = sA, tB = sA;
+  const uint4* src = reinterpret_cast<const uint4*>(g.src);
+  const uint4* thr = reinterpret_cast<const uint4*>(g.thr);
+  if (vA) sA = __ldg(src + gA);
+  if (vB) sB = __ldg(src + gB);
+  if (!TRI) {
+    if (vA) tA = __ldg(thr + gA);
+    if (vB) tB = __ldg(thr + gB);
+  }
+  const uint4 rA = philox_x(gA, sc, rk), rB = philox_x(gB, sc, rk);
+  // edges 4 grp .. 4 grp + 3 that belong to the in-list
+  auto inside = [](bool v, uint32_t grp, uint32_t lo, uint32_t hi) -> uint32_t {
+    const uint32_t e = grp * 4u;
+    const uint32_t a = lo > e ? lo - e : 0u, b = min(hi - e, 4u);
+    return v ? (0xFu << a) & ((1u << b) - 1u) : 0u;
+  };
+  auto live = [](uint32_t need, const uint4& s, const uint4& t, const uint4& r) -> uint32_t {
+    uint32_t m = 0;
+    if (edge_live(r.x, TRI ? tri_thr(s.x) : t.x)) m |= 1u;
+    if (edge_live(r.y, TRI ? tri_thr(s.y) : t.y)) m |= 2u;
+    if (edge_live(r.z, TRI ? tri_thr(s.z) : t.z)) m |= 4u;
+    if (edge_live(r.w, TRI ? tri_thr(s.w) : t.w)) m |= 8u;
+    return m & need;
+  };
+  auto push = [&](uint32_t m, const uint4& s) {
+    constexpr uint32_t SRC = TRI ? TRI_SRC_MASK : 0xFFFFFFFFu;
+    if (m) {
+      unsigned int at = atomicAdd(st.cnt, (unsigned int)__popc(m));
+      if (m & 1u) st.buf[at++] = s.x & SRC;
+      if (m & 2u) st.buf[at++] = s.y & SRC;
+      if (m & 4u) st.buf[at++] = s.z & SRC;
+      if (m & 8u) st.buf[at] = s.w & SRC;
+    }
+  };
+  push(live(inside(vA, gA, loA, hiA), sA, tA, rA), sA);
+  if (drain(st, false, lane, visit)) return true;
+  push(live(inside(vB, gB, loB, hiB), sB, tB, rB), sB);
+  return drain(st, false, lane, visit);
 }
 
 // Edge-balanced expansion of up to 32 frontier nodes (lane i holds node v or
@@ -213,41 +240,64 @@ __device__ __forceinline__ bool deliver(uint32_t cand, uint32_t u0, uint32_t u1,
 // warp prefix sum.  A node with more than heavy_groups groups is first offered
 // to take_heavy(v, lo, hi, ng) (per lane); when it takes the node, the node is
 // skipped here.  Returns 0, 1 when visit asked to stop, or 2 when
-// take_heavy(...) == HEAVY_ABORT for some lane (the caller hands the sample on).
+// take_heavy(...) == HEAVY_ABORT for some lane (the caller hands the sample
+// on).  Up to 31 live tails stay in the stage.
 constexpr int HEAVY_SKIP = 1, HEAVY_ABORT = 2;
 
-template <class Known, class Visit, class Heavy>
+template <bool TRI, class Visit, class Heavy>
 __device__ __forceinline__ int expand_ic(const GraphView& g, int32_t v, const uint32_t* rk, const SampleConst& sc,
-                                         int lane, uint32_t* stage, unsigned long long& ev, unsigned long long& draws,
-                                         int heavy_groups, Known&& known, Visit&& visit, Heavy&& take_heavy) {
+                                         int lane, const Stage& st, unsigned long long& ev, unsigned long long& draws,
+                                         int heavy_groups, Visit&& visit, Heavy&& take_heavy) {
   uint32_t lo = 0, hi = 0;  // edge positions fit 32 bits (m < 2^31)
   if (v >= 0) {
-    lo = (uint32_t)__ldg(g.off + v);
-    hi = (uint32_t)__ldg(g.off + v + 1);
+    lo = __ldg(g.off + v);
+    hi = __ldg(g.off + v + 1);
   }
   int ng = (hi > lo) ? (int)(((hi + 3) >> 2) - (lo >> 2)) : 0;
   int heavy = 0;
   if (ng > heavy_groups) heavy = take_heavy(v, lo, hi, ng);
   if (__any_sync(FULL_MASK, heavy == HEAVY_ABORT)) return 2;
-  if (heavy == HEAVY_SKIP) ng = 0;  // counted and expanded by the taker
-  else ev += hi - lo;
+  ev += hi - lo;
+  draws += (unsigned long long)ng;
+  if (heavy == HEAVY_SKIP) ng = 0;  // expanded by the taker
+  // the nodes with groups go to the low lanes (through the stage's upper part,
+  // free while fewer than 32 tails wait)
+  const unsigned nz = __ballot_sync(FULL_MASK, ng > 0);
+  const int nn = __popc(nz);
+  if (nn == 0) return 0;
+  if (ng > 0) {
+    const int r = __popc(nz & ((1u << lane) - 1u));
+    st.buf[64 + r] = lo;
+    st.buf[96 + r] = hi;
+    st.buf[128 + r] = (uint32_t)ng;
+  }
+  __syncwarp();
+  lo = lane < nn ? st.buf[64 + lane] : 0u;
+  hi = lane < nn ? st.buf[96 + lane] : 0u;
+  ng = lane < nn ? (int)st.buf[128 + lane] : 0;
+  __syncwarp();
   const int incl = warp_inclusive_scan(ng, lane);
   const int excl = incl - ng;
   const int total = __shfl_sync(FULL_MASK, incl, 31);
-  for (int base = 0; base < total; base += 32) {
-    const int q = base + lane;
-    int owner = 0;
-#pragma unroll
-    for (int s = 16; s; s >>= 1) {
-      const int t = __shfl_sync(FULL_MASK, incl, owner + s - 1);
-      if (t <= q) owner += s;
-    }
-    owner = owner > 31 ? 31 : owner;
-    const uint32_t olo = __shfl_sync(FULL_MASK, lo, owner);
-    const uint32_t ohi = __shfl_sync(FULL_MASK, hi, owner);
-    const int oex = __shfl_sync(FULL_MASK, excl, owner);
-    const uint32_t grp = (olo >> 2) + (uint32_t)(q - oex);
-    if (process_slab(g, q < total, grp, olo, ohi, rk, sc, lane, stage, draws, known, visit)) return 1;
+  const uint32_t g0 = (lo >> 2) - (uint32_t)excl;  // group of item q: q + g0
+  const unsigned le_mask = 0xFFFFFFFFu >> (31 - lane);
+  int before = 0;  // nodes whose first group lies before the slab
+  auto owner = [&](int base) -> int {
+    const unsigned d = (unsigned)(excl - base);
+    const unsigned starts = __reduce_or_sync(FULL_MASK, lane < nn && d < 32u ? 1u << d : 0u);
+    const int o = before + __popc(starts & le_mask) - 1;
+    before += __popc(starts);
+    return o;
+  };
+  for (int base = 0; base < total; base += 64) {
+    const int qA = base + lane, qB = qA + 32;
+    const int oA = owner(base), oB = owner(base + 32);
+    const uint32_t gA = (uint32_t)qA + __shfl_sync(FULL_MASK, g0, oA);
+    const uint32_t gB = (uint32_t)qB + __shfl_sync(FULL_MASK, g0, oB);
+    const uint32_t loA = __shfl_sync(FULL_MASK, lo, oA), hiA = __shfl_sync(FULL_MASK, hi, oA);
+    const uint32_t loB = __shfl_sync(FULL_MASK, lo, oB), hiB = __shfl_sync(FULL_MASK, hi, oB);
+    if (two_groups<TRI>(g, qA < total, gA, loA, hiA, qB < total, gB, loB, hiB, rk, sc, lane, st, visit))
+      return 1;
   }
   return 0;
 }
@@ -318,8 +368,8 @@ struct GapWalk {
 
 // Start the walk of node v; false when it has no in-edges.
 __device__ __forceinline__ bool walk_begin(GapWalk& w, const GraphView& g, int32_t v, uint64_t* own) {
-  w.lo = (uint32_t)__ldg(g.off + v);
-  w.d = (uint32_t)__ldg(g.off + v + 1) - w.lo;
+  w.lo = __ldg(g.off + v);
+  w.d = __ldg(g.off + v + 1) - w.lo;
   w.pos = 0;
   w.c = 0;
   w.J = 32 - __clz((int)w.d);
@@ -355,7 +405,7 @@ __device__ __forceinline__ uint32_t walk_step(GapWalk& w, const GraphView& g, in
     ++w.c;
   }
   *more = w.pos < w.d;
-  return __ldg(&g.edge[e].x);
+  return __ldg(g.src + e);
 }
 
 // Weighted-cascade BFS of one sample by one warp over its private queue
@@ -386,8 +436,8 @@ __device__ __forceinline__ void wc_bfs_warp(const GraphView& g, const int32_t* Q
       const int r = __popc(nm & lt_mask);
       if (r < take) {
         v = Q[head + r];
-        lo = (uint32_t)__ldg(g.off + v);
-        d = (uint32_t)__ldg(g.off + v + 1) - lo;
+        lo = __ldg(g.off + v);
+        d = __ldg(g.off + v + 1) - lo;
         ev += d;
         pos = 0;
         c = 0;
@@ -402,7 +452,7 @@ __device__ __forceinline__ void wc_bfs_warp(const GraphView& g, const int32_t* Q
       if (d == 0u) {
         v = -1;
       } else if (d == 1u) {
-        u = __ldg(&g.edge[lo].x);
+        u = __ldg(g.src + lo);
         v = -1;
       } else {
         uint64_t U;
@@ -418,7 +468,7 @@ __device__ __forceinline__ void wc_bfs_warp(const GraphView& g, const int32_t* Q
         if (G >= d - pos) {
           v = -1;
         } else {
-          u = __ldg(&g.edge[lo + pos + G].x);
+          u = __ldg(g.src + lo + pos + G);
           pos += G + 1u;
           ++c;
           if (pos >= d) v = -1;
@@ -476,17 +526,21 @@ __device__ __forceinline__ void warp_store_set(const SampleJob& J, int64_t j, co
   }
 }
 
-template <int MODE, int TIER, bool WC>
+template <int MODE, int TIER, int W>
 __global__ void __launch_bounds__(WT_WARPS * 32, 4) k_sample_warp_ic(SampleJob J) {
+  constexpr bool WC = W == W_GAPS;
   constexpr int HBITS = Tier<TIER>::HBITS, QCAP = Tier<TIER>::QCAP;
   __shared__ __align__(16) uint32_t s_hash[TIER == 0 ? WT_WARPS : 1][TIER == 0 ? WT_HASH : 4];
   __shared__ int32_t s_q[TIER == 0 ? WT_WARPS : 1][TIER == 0 ? WT_QCAP : 4];
   __shared__ uint32_t s_stage[WT_WARPS][WC ? 1 : STAGE];  // the gap walk needs no staging
+  __shared__ unsigned int s_staged[WT_WARPS];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const size_t gwarp = (size_t)blockIdx.x * WT_WARPS + wid;
   uint32_t* H = TIER == 0 ? s_hash[wid] : J.mid_hash + gwarp * MID_HASH;
   int32_t* Q = TIER == 0 ? s_q[wid] : J.mid_queue + gwarp * MID_QSLOTS;
   uint32_t* slots = TIER == 0 ? nullptr : J.mid_slots + gwarp * MID_QSLOTS;
+  const Stage stage{s_stage[wid], &s_staged[wid]};
+  if (lane == 0) s_staged[wid] = 0u;
   if (TIER == 0) {
     uint4* H4 = reinterpret_cast<uint4*>(H);
     for (int i = lane; i < WT_HASH / 4; i += 32) H4[i] = make_uint4(0, 0, 0, 0);
@@ -518,7 +572,6 @@ __global__ void __launch_bounds__(WT_WARPS * 32, 4) k_sample_warp_ic(SampleJob J
     // tier 1's hand-over size is tuned at run time (at most its queue capacity)
     const int cap = TIER == 0 ? QCAP : min(QCAP, J.mid_cap);
     __syncwarp();
-    auto known = [](uint32_t) { return false; };
     auto visit = [&](uint32_t u, unsigned lt_mask) -> bool {
       uint32_t slot = 0;
       const bool is_new = (u != NO_NODE) && hash_insert<HBITS>(H, u, &slot);
@@ -551,17 +604,18 @@ __global__ void __launch_bounds__(WT_WARPS * 32, 4) k_sample_warp_ic(SampleJob J
         __syncwarp();
         const int32_t v = (lane < cnt) ? Q[head + lane] : -1;
         __syncwarp();
-        if (expand_ic(J.g, v, J.rk, sc, lane, s_stage[wid], ev, dr, J.warp_heavy_groups, known, visit, to_cta) ==
-            2) {
+        if (expand_ic<W == W_TRI>(J.g, v, J.rk, sc, lane, stage, ev, dr, J.warp_heavy_groups, visit, to_cta) == 2) {
           handoff = true;
           break;
         }
+        if (!overflow && !hit) drain(stage, true, lane, visit);
         head += cnt;
       }
     }
     __syncwarp();
     if (handoff) {
       if (lane == 0) {
+        *stage.cnt = 0u;
         const unsigned long long b = atomicAdd(&J.ctr->big_count, 1ull);
         J.big_list[b] = j;
       }
@@ -701,8 +755,8 @@ __global__ void __launch_bounds__(256) k_sample_lane_wc(SampleJob J) {
     bool overflow = false;
     for (int h = 0; h < tail && !hit && !overflow; ++h) {
       const int32_t v = q[h];
-      const uint32_t lo = (uint32_t)__ldg(J.g.off + v);
-      const uint32_t d = (uint32_t)__ldg(J.g.off + v + 1) - lo;
+      const uint32_t lo = __ldg(J.g.off + v);
+      const uint32_t d = __ldg(J.g.off + v + 1) - lo;
       ev += d;
       if (d == 0u) continue;
       const int Jb = 32 - __clz((int)d);
@@ -730,7 +784,7 @@ __global__ void __launch_bounds__(256) k_sample_lane_wc(SampleJob J) {
           pos += G + 1u;
           ++c;
         }
-        const int32_t u = (int32_t)__ldg(&J.g.edge[e].x);
+        const int32_t u = (int32_t)__ldg(J.g.src + e);
         bool seen = false;
         for (int i = 0; i < tail; ++i) seen |= q[i] == u;
         if (seen) continue;
@@ -806,7 +860,7 @@ __global__ void __launch_bounds__(WT_WARPS * 32) k_sample_warp_lt(SampleJob J) {
         unsigned long long carry = 0;
         for (int64_t b = lo; b < hi; b += 32) {
           const int64_t e = b + lane;
-          unsigned long long incl = e < hi ? (unsigned long long)__ldg(&J.g.edge[e].y) : 0ull;
+          unsigned long long incl = e < hi ? (unsigned long long)__ldg(J.g.thr + e) : 0ull;
 #pragma unroll
           for (int dd = 1; dd < 32; dd <<= 1) {
             const unsigned long long t = __shfl_up_sync(FULL_MASK, incl, dd);
@@ -821,7 +875,7 @@ __global__ void __launch_bounds__(WT_WARPS * 32) k_sample_warp_lt(SampleJob J) {
         }
         if (pick < 0) break;  // no in-edge kept: the walk ends here
       }
-      const int32_t u = (int32_t)__ldg(&J.g.edge[pick].x);
+      const int32_t u = (int32_t)__ldg(J.g.src + pick);
       if (lane == 0) {
         ev += 1;
         dr += 1;
@@ -860,15 +914,17 @@ __global__ void __launch_bounds__(WT_WARPS * 32) k_sample_warp_lt(SampleJob J) {
 // KIND 1: small CTAs (bitmap in global memory, queue of small_qcap entries);
 //         a set that outgrows the queue goes on to KIND 2.
 // KIND 2: full-size CTAs (global bitmap, queue of n entries) for those sets.
-template <int MODE, bool SMEM_BITMAP, int KIND, bool WC>
+template <int MODE, bool SMEM_BITMAP, int KIND, int W>
 __global__ void __launch_bounds__(KIND == 1 ? SMALL_CTA_THREADS : 1024, KIND == 1 ? 1024 / SMALL_CTA_THREADS : 1)
     k_sample_cta(SampleJob J) {
+  constexpr bool WC = W == W_GAPS;
   constexpr int WARPS = KIND == 1 ? SMALL_CTA_THREADS / 32 : 32;
   extern __shared__ __align__(16) uint32_t s_bits[];
   __shared__ long long s_item;
   __shared__ int s_tail, s_next, s_hit, s_ok;
   __shared__ unsigned long long s_pos;
   __shared__ uint32_t s_stage[WARPS][WC ? 1 : STAGE];
+  __shared__ unsigned int s_staged[WARPS];
   // heavy in-lists of the current level, expanded by all warps together
   __shared__ uint32_t s_hlo[WC ? 1 : CTA_HEAVY_CAP], s_hhi[WC ? 1 : CTA_HEAVY_CAP];
   __shared__ int s_hpref[WC ? 1 : CTA_HEAVY_CAP];
@@ -881,7 +937,8 @@ __global__ void __launch_bounds__(KIND == 1 ? SMALL_CTA_THREADS : 1024, KIND == 
   uint32_t* bits = SMEM_BITMAP ? s_bits
                    : (KIND == 1 ? J.small_bitmap : J.slot_bitmap) + (size_t)blockIdx.x * (size_t)J.bitmap_words;
   int32_t* Q = (KIND == 1 ? J.small_queue : J.slot_queue) + (size_t)blockIdx.x * (size_t)qcap;
-  uint32_t* stage = s_stage[tid >> 5];
+  const Stage stage{s_stage[tid >> 5], &s_staged[tid >> 5]};
+  if (lane == 0) *stage.cnt = 0u;
   if (SMEM_BITMAP)
     for (int64_t i = tid; i < J.bitmap_words; i += nthr) bits[i] = 0u;
   unsigned long long* work = KIND == 2 ? &J.ctr->big2_work : &J.ctr->big_work;
@@ -906,18 +963,15 @@ __global__ void __launch_bounds__(KIND == 1 ? SMALL_CTA_THREADS : 1024, KIND == 
     __syncthreads();
     if (J.model == 0) {
       const SampleConst sc = sample_const(J.rk, (uint32_t)j, ctr_word3(WC ? PURPOSE_SKIP : PURPOSE_IC, J.stream, j));
-      // a stale 0 only costs a draw; bits are never cleared during a sample.  With the
-      // bitmap in global memory the check would cost an L2 round trip per group, more
-      // than the draw it can save, so only the shared-memory bitmap is consulted.
-      auto known = [&](uint32_t u) -> bool {
-        if (!SMEM_BITMAP) return false;
-        return (bits[u >> 5] >> (u & 31)) & 1u;
-      };
       auto visit = [&](uint32_t u, unsigned lt_mask) -> bool {
         bool is_new = false;
         if (u != NO_NODE) {
           const uint32_t mask = 1u << (u & 31);
-          is_new = !(atomicOr(bits + (u >> 5), mask) & mask);
+          // most live tails are in a large set already: a look is cheaper than the
+          // atomic (bits are only ever set during a sample; one in global memory
+          // would cost a second round trip)
+          if (!SMEM_BITMAP || WC || !(*(volatile uint32_t*)(bits + (u >> 5)) & mask))
+            is_new = !(atomicOr(bits + (u >> 5), mask) & mask);
         }
         const unsigned m = __ballot_sync(FULL_MASK, is_new);
         int base = 0;
@@ -1036,7 +1090,6 @@ __global__ void __launch_bounds__(KIND == 1 ? SMALL_CTA_THREADS : 1024, KIND == 
         if (slot >= CTA_HEAVY_CAP) return 0;  // list full: this warp expands it itself
         s_hlo[slot] = lo;
         s_hhi[slot] = hi;
-        ev += hi - lo;
         return HEAVY_SKIP;
       };
       if (tid == 0) s_nheavy = 0;
@@ -1054,20 +1107,21 @@ __global__ void __launch_bounds__(KIND == 1 ? SMALL_CTA_THREADS : 1024, KIND == 
           if (b >= lvl_end) break;
           const int cnt = min(32, lvl_end - b);
           const int32_t v = (lane < cnt) ? Q[b + lane] : -1;
-          if (expand_ic(J.g, v, J.rk, sc, lane, stage, ev, dr, CTA_HEAVY_GROUPS, known, visit, take_heavy))
+          if (expand_ic<W == W_TRI>(J.g, v, J.rk, sc, lane, stage, ev, dr, CTA_HEAVY_GROUPS, visit, take_heavy))
             break;
         }
+        drain(stage, true, lane, visit);
         __syncthreads();
         const int nh = min(s_nheavy, CTA_HEAVY_CAP);
         if (nh > 0 && !s_hit && !(KIND == 1 && s_tail > qcap)) {
-          // groups of the heavy in-lists, dealt to all warps 32 at a time
+          // the heavy in-lists in pieces of 64 groups, dealt to all warps
           if (wid == 0) {
             int carry = 0;
             for (int base = 0; base < nh; base += 32) {
               const int i = base + lane;
-              const int ng = i < nh ? (int)(((s_hhi[i] + 3) >> 2) - (s_hlo[i] >> 2)) : 0;
-              const int incl = warp_inclusive_scan(ng, lane);
-              if (i < nh) s_hpref[i] = carry + incl - ng;
+              const int np = i < nh ? (int)(((s_hhi[i] + 3) >> 2) - (s_hlo[i] >> 2) + 63) >> 6 : 0;
+              const int incl = warp_inclusive_scan(np, lane);
+              if (i < nh) s_hpref[i] = carry + incl - np;
               carry += __shfl_sync(FULL_MASK, incl, 31);
             }
             if (lane == 0) {
@@ -1079,18 +1133,20 @@ __global__ void __launch_bounds__(KIND == 1 ? SMALL_CTA_THREADS : 1024, KIND == 
           const int htotal = s_htotal;
           for (;;) {
             int c = 0;
-            if (lane == 0) c = atomicAdd(&s_hnext, 32);
+            if (lane == 0) c = atomicAdd(&s_hnext, 1);
             c = __shfl_sync(FULL_MASK, c, 0);
             if (c >= htotal) break;
-            const int q = c + lane;
-            int it = 0;  // last heavy list whose first group is <= q
+            int it = 0;  // last heavy list whose first piece is <= c
             for (int step = CTA_HEAVY_CAP / 2; step; step >>= 1)
-              if (it + step < nh && s_hpref[it + step] <= q) it += step;
+              if (it + step < nh && s_hpref[it + step] <= c) it += step;
             const uint32_t olo = s_hlo[it], ohi = s_hhi[it];
-            const uint32_t grp = (olo >> 2) + (uint32_t)(q - s_hpref[it]);
-            if (process_slab(J.g, q < htotal, grp, olo, ohi, J.rk, sc, lane, stage, dr, known, visit))
+            const uint32_t grp = (olo >> 2) + (uint32_t)(c - s_hpref[it]) * 64u + (uint32_t)lane;
+            const uint32_t end = (ohi + 3) >> 2;
+            if (two_groups<W == W_TRI>(J.g, grp < end, grp, olo, ohi, grp + 32u < end, grp + 32u, olo, ohi, J.rk, sc,
+                                       lane, stage, visit))
               break;
           }
+          drain(stage, true, lane, visit);
         }
         __syncthreads();
         if (tid == 0) s_nheavy = 0;
@@ -1114,7 +1170,7 @@ __global__ void __launch_bounds__(KIND == 1 ? SMALL_CTA_THREADS : 1024, KIND == 
         } else {
           unsigned long long cum = 0;
           for (int64_t e = lo; e < hi; ++e) {
-            cum += J.g.edge[e].y;
+            cum += J.g.thr[e];
             if ((unsigned long long)r.x < cum) {
               pick = e;
               break;
@@ -1122,7 +1178,7 @@ __global__ void __launch_bounds__(KIND == 1 ? SMALL_CTA_THREADS : 1024, KIND == 
           }
           if (pick < 0) break;
         }
-        const int32_t u = (int32_t)J.g.edge[pick].x;
+        const int32_t u = (int32_t)J.g.src[pick];
         ev += 1;
         dr += 1;
         const uint32_t mask = 1u << (u & 31);
@@ -1204,9 +1260,9 @@ LaunchCfg sampler_config(const GraphView& g, int model, bool wc) {
   cudaDeviceGetAttribute(&c.num_sms, cudaDevAttrMultiProcessorCount, dev);
   int per_sm = 0;
   if (model == 0 && wc)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample_warp_ic<MODE_STORE, 0, true>, WT_WARPS * 32, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample_warp_ic<MODE_STORE, 0, W_GAPS>, WT_WARPS * 32, 0);
   else if (model == 0)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample_warp_ic<MODE_STORE, 0, false>, WT_WARPS * 32,
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample_warp_ic<MODE_STORE, 0, W_COINS>, WT_WARPS * 32,
                                                   0);
   else
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample_warp_lt<MODE_STORE>, WT_WARPS * 32, 0);
@@ -1221,10 +1277,10 @@ LaunchCfg sampler_config(const GraphView& g, int model, bool wc) {
     // global bitmap: many small CTAs first, a few full-size ones for the largest sets
     int small_per_sm = 0;
     if (model == 0 && wc)
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&small_per_sm, k_sample_cta<MODE_STORE, false, 1, true>,
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&small_per_sm, k_sample_cta<MODE_STORE, false, 1, W_GAPS>,
                                                     SMALL_CTA_THREADS, 0);
     else
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&small_per_sm, k_sample_cta<MODE_STORE, false, 1, false>,
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&small_per_sm, k_sample_cta<MODE_STORE, false, 1, W_COINS>,
                                                     SMALL_CTA_THREADS, 0);
     if (small_per_sm < 1) small_per_sm = 1;
     c.small_blocks = c.num_sms * small_per_sm;
@@ -1260,11 +1316,20 @@ size_t sampler_scratch_bytes(const GraphView& g, const LaunchCfg& c) {
   return per_slot * (size_t)c.cta_blocks + ((size_t)c.small_qcap * 4 + words * 4) * (size_t)c.small_blocks;
 }
 
-template <int MODE, bool WC>
-static void launch_warp_ic(const SampleJob& J, const LaunchCfg& c, cudaStream_t st) {
+template <int MODE, int W>
+static void launch_warp_ic_w(const SampleJob& J, const LaunchCfg& c, cudaStream_t st) {
   const dim3 block(WT_WARPS * 32);
-  k_sample_warp_ic<MODE, 0, WC><<<c.warp_blocks, block, 0, st>>>(J);
-  if (J.mid_cap > 0) k_sample_warp_ic<MODE, 1, WC><<<c.mid_blocks, block, 0, st>>>(J);
+  k_sample_warp_ic<MODE, 0, W><<<c.warp_blocks, block, 0, st>>>(J);
+  if (J.mid_cap > 0) k_sample_warp_ic<MODE, 1, W><<<c.mid_blocks, block, 0, st>>>(J);
+}
+
+template <int MODE>
+static void launch_warp_ic(const SampleJob& J, const LaunchCfg& c, cudaStream_t st) {
+  switch (weights_of(J)) {
+    case W_GAPS: return launch_warp_ic_w<MODE, W_GAPS>(J, c, st);
+    case W_TRI: return launch_warp_ic_w<MODE, W_TRI>(J, c, st);
+    default: return launch_warp_ic_w<MODE, W_COINS>(J, c, st);
+  }
 }
 
 cudaError_t launch_sample_warp(const SampleJob& J, const LaunchCfg& c, cudaStream_t st) {
@@ -1277,13 +1342,8 @@ cudaError_t launch_sample_warp(const SampleJob& J, const LaunchCfg& c, cudaStrea
     if (J.mode == MODE_STORE) k_sample_warp_wcg<MODE_STORE><<<c.wg_blocks, block, 0, st>>>(J);
     else k_sample_warp_wcg<MODE_HIT><<<c.wg_blocks, block, 0, st>>>(J);
   } else if (J.model == 0) {
-    if (J.mode == MODE_STORE) {
-      if (J.wc_implicit) launch_warp_ic<MODE_STORE, true>(J, c, st);
-      else launch_warp_ic<MODE_STORE, false>(J, c, st);
-    } else {
-      if (J.wc_implicit) launch_warp_ic<MODE_HIT, true>(J, c, st);
-      else launch_warp_ic<MODE_HIT, false>(J, c, st);
-    }
+    if (J.mode == MODE_STORE) launch_warp_ic<MODE_STORE>(J, c, st);
+    else launch_warp_ic<MODE_HIT>(J, c, st);
   } else {
     if (J.mode == MODE_STORE) k_sample_warp_lt<MODE_STORE><<<grid, block, 0, st>>>(J);
     else k_sample_warp_lt<MODE_HIT><<<grid, block, 0, st>>>(J);
@@ -1291,26 +1351,28 @@ cudaError_t launch_sample_warp(const SampleJob& J, const LaunchCfg& c, cudaStrea
   return cudaGetLastError();
 }
 
-template <int MODE, bool SB, bool WC>
+template <int MODE, bool SB, int W>
 static cudaError_t launch_cta_t(const SampleJob& J, const LaunchCfg& c, cudaStream_t st) {
   if (SB) {
     const size_t smem = (size_t)c.smem_bitmap_bytes;
-    cudaError_t e = cudaFuncSetAttribute(k_sample_cta<MODE, true, 0, WC>,
+    cudaError_t e = cudaFuncSetAttribute(k_sample_cta<MODE, true, 0, W>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_sample_cta<MODE, true, 0, WC><<<c.cta_blocks, c.cta_threads, smem, st>>>(J);
+    k_sample_cta<MODE, true, 0, W><<<c.cta_blocks, c.cta_threads, smem, st>>>(J);
   } else {
-    k_sample_cta<MODE, false, 1, WC><<<c.small_blocks, SMALL_CTA_THREADS, 0, st>>>(J);
-    k_sample_cta<MODE, false, 2, WC><<<c.cta_blocks, c.cta_threads, 0, st>>>(J);
+    k_sample_cta<MODE, false, 1, W><<<c.small_blocks, SMALL_CTA_THREADS, 0, st>>>(J);
+    k_sample_cta<MODE, false, 2, W><<<c.cta_blocks, c.cta_threads, 0, st>>>(J);
   }
   return cudaGetLastError();
 }
 
 template <int MODE, bool SB>
 static cudaError_t launch_cta_w(const SampleJob& J, const LaunchCfg& c, cudaStream_t st) {
-  // the LT walk reads no thresholds: one instantiation serves it
-  return (J.model == 0 && J.wc_implicit) ? launch_cta_t<MODE, SB, true>(J, c, st)
-                                         : launch_cta_t<MODE, SB, false>(J, c, st);
+  switch (weights_of(J)) {
+    case W_GAPS: return launch_cta_t<MODE, SB, W_GAPS>(J, c, st);
+    case W_TRI: return launch_cta_t<MODE, SB, W_TRI>(J, c, st);
+    default: return launch_cta_t<MODE, SB, W_COINS>(J, c, st);
+  }
 }
 
 cudaError_t launch_sample_cta(const SampleJob& J, const LaunchCfg& c, cudaStream_t st) {
