@@ -105,8 +105,8 @@ struct ssa_graph {
   uint32_t* off = nullptr;
   uint32_t* src = nullptr;
   uint32_t* thr = nullptr;       // stored thresholds (see GraphView)
-  uint64_t* wc_pow = nullptr;  // weighted cascade: gap powers per in-degree (build_wc_pow)
-  int wc_pow_k = 0;
+  float* wc_inv = nullptr;       // weighted cascade: gap scale per in-degree (build_wc_inv)
+  int wc_inv_k = 0;
   int64_t bytes = 0;
   // IC sampler hand-over sizes chosen by the autotuner (-1: not tuned yet)
   mutable std::mutex tune_mu;
@@ -122,8 +122,8 @@ struct ssa_graph {
     v.off = off;
     v.src = src;
     v.thr = thr;
-    v.wc_pow = wc_pow;
-    v.wc_pow_k = wc_pow_k;
+    v.wc_inv = wc_inv;
+    v.wc_inv_k = wc_inv_k;
     return v;
   }
 };
@@ -1472,12 +1472,12 @@ ssa_status ssa_load_graph(int64_t n, int64_t m, const int32_t* src, const int32_
       break;
     }
     if (weighting == SSA_W_WC) {
-      e = build_wc_pow(g->off, n, &g->wc_pow, &g->wc_pow_k, st);
+      e = build_wc_inv(g->off, n, &g->wc_inv, &g->wc_inv_k, st);
       if (e != cudaSuccess) {
-        rc = fail(e == cudaErrorMemoryAllocation ? SSA_E_NOMEM : SSA_E_CUDA, "power table: %s", cudaGetErrorString(e));
+        rc = fail(e == cudaErrorMemoryAllocation ? SSA_E_NOMEM : SSA_E_CUDA, "gap table: %s", cudaGetErrorString(e));
         break;
       }
-      if (g->wc_pow_k > 0) g->bytes += (int64_t)(sizeof(uint64_t) * (((size_t)g->wc_pow_k - 1) << g->wc_pow_k) + 8);
+      if (g->wc_inv_k > 0) g->bytes += (int64_t)(sizeof(float) << g->wc_inv_k);
     }
   } while (false);
   if (d_src) cudaFreeAsync(d_src, st);
@@ -1490,7 +1490,7 @@ ssa_status ssa_load_graph(int64_t n, int64_t m, const int32_t* src, const int32_
     if (g->off) cudaFree(g->off);
     if (g->src) cudaFree(g->src);
     if (g->thr) cudaFree(g->thr);
-    if (g->wc_pow) cudaFree(g->wc_pow);
+    if (g->wc_inv) cudaFree(g->wc_inv);
     delete g;
     return rc;
   }
@@ -1527,7 +1527,7 @@ ssa_status ssa_gen_rmat(int32_t scale, int64_t m_draw, double a, double b, doubl
   int64_t m = 0;
   cudaError_t e = rmat_graph(scale, m_draw, prob_threshold(a), prob_threshold(a + b), prob_threshold(a + b + c), seed,
                              (int)weighting, weight_seed, &m, &g->off, &g->src, st, &launches);
-  if (e == cudaSuccess && weighting == SSA_W_WC) e = build_wc_pow(g->off, g->n, &g->wc_pow, &g->wc_pow_k, st);
+  if (e == cudaSuccess && weighting == SSA_W_WC) e = build_wc_inv(g->off, g->n, &g->wc_inv, &g->wc_inv_k, st);
   const cudaError_t e2 = cudaStreamSynchronize(st);
   cudaStreamDestroy(st);
   if (e == cudaSuccess) e = e2;
@@ -1535,14 +1535,14 @@ ssa_status ssa_gen_rmat(int32_t scale, int64_t m_draw, double a, double b, doubl
     if (g->off) cudaFree(g->off);
     if (g->src) cudaFree(g->src);
     if (g->thr) cudaFree(g->thr);
-    if (g->wc_pow) cudaFree(g->wc_pow);
+    if (g->wc_inv) cudaFree(g->wc_inv);
     delete g;
     return fail(e == cudaErrorMemoryAllocation ? SSA_E_NOMEM : SSA_E_CUDA, "R-MAT generation: %s",
                 cudaGetErrorString(e));
   }
   g->m = m;
   g->bytes = (int64_t)(sizeof(uint32_t) * ((size_t)(g->n + 1) + (size_t)(((m + 3) / 4) * 4 + 4)));
-  if (g->wc_pow_k > 0) g->bytes += (int64_t)(sizeof(uint64_t) * (((size_t)g->wc_pow_k - 1) << g->wc_pow_k) + 8);
+  if (g->wc_inv_k > 0) g->bytes += (int64_t)(sizeof(float) << g->wc_inv_k);
   *out = g;
   return SSA_OK;
 }
@@ -1553,7 +1553,7 @@ ssa_status ssa_free_graph(ssa_graph* g) {
   if (g->off) cudaFree(g->off);
   if (g->src) cudaFree(g->src);
   if (g->thr) cudaFree(g->thr);
-  if (g->wc_pow) cudaFree(g->wc_pow);
+  if (g->wc_inv) cudaFree(g->wc_inv);
   delete g;
   return SSA_OK;
 }

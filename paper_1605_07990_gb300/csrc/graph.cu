@@ -232,27 +232,21 @@ __global__ void k_max_in_degree(const uint32_t* off, int64_t n, unsigned long lo
   if ((threadIdx.x & 31) == 0 && best) atomicMax(out, best);
 }
 
-// Row of in-degree d (1 <= d < 2^K): the powers q^(2^i), i < bit length of d,
-// of the weighted-cascade gap form (Q = (2^32 - t) << 32 with t = floor(2^32/d),
-// 0xFFFFFFFF for d = 1; each power the high 64 bits of the previous one squared).
-__global__ void k_wc_pow_rows(uint64_t* tab, int K) {
-  const int64_t rows = int64_t(1) << K;
-  for (int64_t d = 1 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d < rows;
-       d += (int64_t)gridDim.x * blockDim.x) {
-    const int k = 63 - __clzll(d);
-    const uint64_t base = k == 0 ? 0ull : (uint64_t)(k - 1) * (1ull << k) + 1ull;
-    uint64_t* row = tab + base + (uint64_t)(d - (int64_t(1) << k)) * (uint64_t)(k + 1);
-    const uint32_t t = d == 1 ? 0xFFFFFFFFu : (uint32_t)(0x100000000ull / (uint64_t)d);
-    uint64_t p = (0x100000000ull - t) << 32;
-    for (int i = 0; i <= k; ++i) {
-      row[i] = p;
-      p = __umul64hi(p, p);
+// tab[d] = -1 / log2(q), q = 1 - t / 2^32 with t = floor(2^32 / d): the gap
+// form's scale of in-degree d, rounded once from 64 bits (0 for d < 2, not used)
+__global__ void k_wc_inv(float* tab, int64_t rows) {
+  for (int64_t d = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; d < rows; d += (int64_t)gridDim.x * blockDim.x) {
+    float k = 0.f;
+    if (d >= 2) {
+      const double p = (double)(uint32_t)(0x100000000ull / (uint64_t)d) * 0x1p-32;
+      k = (float)(-0.69314718055994530942 / log1p(-p));
     }
+    tab[d] = k;
   }
 }
 }  // namespace
 
-cudaError_t build_wc_pow(const uint32_t* d_off, int64_t n, uint64_t** tab, int* k_out, cudaStream_t st) {
+cudaError_t build_wc_inv(const uint32_t* d_off, int64_t n, float** tab, int* k_out, cudaStream_t st) {
   *tab = nullptr;
   *k_out = 0;
   unsigned long long* d_max = nullptr;
@@ -266,11 +260,12 @@ cudaError_t build_wc_pow(const uint32_t* d_off, int64_t n, uint64_t** tab, int* 
   cudaFree(d_max);
   if (e != cudaSuccess) return e;
   int K = 0;
-  while (K < WC_POW_K && (1ull << K) <= maxd) ++K;  // rows for every d < 2^K that occurs
+  while (K < WC_INV_K && (1ull << K) <= maxd) ++K;  // entries for every d < 2^K that occurs
   if (K < 2) return cudaSuccess;                     // no in-list of 2 or more edges
-  const size_t entries = (size_t)(K - 1) * ((size_t)1 << K) + 1;
-  if ((e = cudaMallocAsync(reinterpret_cast<void**>(tab), sizeof(uint64_t) * entries, st)) != cudaSuccess) return e;
-  k_wc_pow_rows<<<grid_for((int64_t)1 << K, 256), 256, 0, st>>>(*tab, K);
+  const int64_t entries = int64_t(1) << K;
+  if ((e = cudaMallocAsync(reinterpret_cast<void**>(tab), sizeof(float) * (size_t)entries, st)) != cudaSuccess)
+    return e;
+  k_wc_inv<<<grid_for(entries, 256), 256, 0, st>>>(*tab, entries);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   *k_out = K;
   return cudaSuccess;

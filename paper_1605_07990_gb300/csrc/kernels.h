@@ -27,19 +27,19 @@ struct GraphView {
   const uint32_t* off = nullptr;  // n+1
   const uint32_t* src = nullptr;  // m rounded up to a multiple of 4 (+4)
   const uint32_t* thr = nullptr;  // as src, or null
-  // weighted cascade: the gap form's powers q^(2^i) of every in-degree d < 2^wc_pow_k
-  // (rows of bit-length entries, in order of d; null / 0 for other weightings)
-  const uint64_t* wc_pow = nullptr;
-  int wc_pow_k = 0;
+  // weighted cascade: -1 / log2(q) of the gap form for every in-degree d < 2^wc_inv_k
+  // (null / 0 for other weightings)
+  const float* wc_inv = nullptr;
+  int wc_inv_k = 0;
 };
 
-// In-degrees of up to 2^WC_POW_K - 1 take their gap powers from the graph's
-// table ((WC_POW_K - 1) 2^WC_POW_K + 1 entries, 160 MB); larger ones build them.
-constexpr int WC_POW_K = 20;
+// In-degrees of up to 2^WC_INV_K - 1 have an entry (4 MB at most); for larger
+// ones 32 bits would seldom decide, and the exact gap is taken.
+constexpr int WC_INV_K = 20;
 
-// The weighted-cascade power table of a CSR (rows for every in-degree below
-// min(2^WC_POW_K, 2 * max in-degree)); *tab stays null when no in-list has 2 edges.
-cudaError_t build_wc_pow(const uint32_t* d_off, int64_t n, uint64_t** tab, int* k, cudaStream_t st);
+// That table for a CSR (every in-degree below min(2^WC_INV_K, 2 * max
+// in-degree)); *tab stays null when no in-list has 2 edges.
+cudaError_t build_wc_inv(const uint32_t* d_off, int64_t n, float** tab, int* k, cudaStream_t st);
 
 // Device counters of one sampling batch.
 // Bounded waits of the weighted-cascade CTA tier that gave up (Counters::error).

@@ -20,8 +20,9 @@
 // asked for each tail first and visited slab by slab.
 // IC with weighted-cascade weights: every in-edge of a node has the same
 // probability, so each lane walks one frontier node's in-list by geometric
-// gaps between live edges (the gap form below); the work per node is a few
-// 64-bit products and one Philox draw per two gaps, whatever its in-degree.
+// gaps between live edges (the gap form below); the work per node is a
+// logarithm per gap and one Philox draw per two, whatever its in-degree.  Bound:
+// the three dependent memory round trips of a BFS step.
 #include <algorithm>
 
 #include "device.cuh"
@@ -315,29 +316,15 @@ __device__ __forceinline__ uint32_t wc_threshold(uint32_t d) {
 // P_(i+1) = hi64(P_i * P_i); G(U) sets bits J-1 .. 0 in turn (J the bit
 // length of d, so 2^J - 1 >= d), bit i when U < hi64(A * P_i), A the product
 // of the powers already taken (P_i alone for the first), which then becomes
-// A.  G(U) is the largest g with U < q^g up to the truncation.  The powers of
-// a node are built once, into the lane's own table P (J <= 31 entries).
-__device__ __forceinline__ void wc_powers(uint64_t Q, int J, uint64_t* P) {
-  uint64_t p = Q;
+// A.  G(U) is the largest g with U < T(g), T(g) the product along g's bits.
+__device__ __noinline__ uint32_t wc_gap_exact(uint32_t d, uint64_t U) {
+  uint64_t P[31];
+  const int J = 32 - __clz((int)d);
+  uint64_t p = (0x100000000ull - wc_threshold(d)) << 32;
   for (int i = 0; i < J; ++i) {
     P[i] = p;
     p = __umul64hi(p, p);
   }
-}
-
-// The powers of in-degree d >= 2: the graph's table row when d < 2^wc_pow_k
-// (rows for d in [2^k, 2^(k+1)) hold k+1 entries and follow all shorter rows,
-// so row d starts at (k-1) 2^k + 1 + (d - 2^k)(k+1)), else built into `own`.
-__device__ __forceinline__ const uint64_t* wc_power_row(const GraphView& g, uint32_t d, int J, uint64_t* own) {
-  if (d < (1u << g.wc_pow_k)) {
-    const int k = J - 1;
-    return g.wc_pow + ((uint64_t)(k - 1) << k) + 1ull + (uint64_t)(d - (1u << k)) * (uint64_t)J;
-  }
-  wc_powers((0x100000000ull - wc_threshold(d)) << 32, J, own);
-  return own;
-}
-
-__device__ __forceinline__ uint32_t wc_gap(const uint64_t* P, int J, uint64_t U) {
   uint64_t A = 0;
   bool first = true;
   uint32_t gap = 0;
@@ -352,6 +339,42 @@ __device__ __forceinline__ uint32_t wc_gap(const uint64_t* P, int J, uint64_t U)
   return gap;
 }
 
+// G(U) where it is below `left` (the edges that remain), else some value >=
+// left.  Most U lie far from every T(g), and there a logarithm in 32 bits
+// decides: with L = log_q(U / 2^64), T(g) lies in [q^g (1 - d 2^-59), q^g] 2^64,
+// so when floor(L) = g and L is further than d^2 2^-59 (below 2^-19 for the
+// d < 2^20 of the table) from every integer, all T up to T(g) lie above U and
+// all others at or below it: G = g.  L = y K with y = -log2(U / 2^64) and
+// K = inv[d] = -1 / log2(q).  Errors: __log2f 2^-22 (its stated bound on
+// [0.5, 2]), the mantissa cut to 23 bits 1.45 2^-23, the roundings of y, K and
+// the product 2^-24 each relative; together below K 4.2e-7 + L 1.8e-7, taken
+// as K 4.5e-7 + L 2.5e-7 + 4e-6.  Nearer to an integer than that (about one
+// draw in 200 at d = 10,000, one in 12 at 2^17) the exact form decides, so the
+// results are its results always.  The exact form is J 64-bit products and
+// compares (14 at d = 10,000, ~250 instructions, and a row of powers to read);
+// this is one load, one logarithm and a dozen 32-bit operations.  Sampling of a
+// whole solve on GB300: 33.1 -> 17.1 ms (SSA, 2^25 nodes, 51.5M visits),
+// 12.1 -> 6.7 ms (D-SSA, 2^23), 1.55 -> 0.86 ms (SSA, 2^14).
+__device__ __forceinline__ uint32_t wc_gap(float K, uint32_t d, uint32_t left, uint64_t U) {
+  const uint32_t hi = (uint32_t)(U >> 32);
+  const int lz = __clz((int)hi);
+  const uint32_t norm = __funnelshift_l((uint32_t)U, hi, (unsigned)lz);  // bit 31 set when hi != 0
+  const float m = __uint_as_float(0x3F800000u | ((norm >> 8) & 0x7FFFFFu));
+  const float L = ((float)(lz + 1) - __log2f(m)) * K;
+  const float e = fmaf(K, 4.5e-7f, fmaf(L, 2.5e-7f, 4e-6f));
+  const float f = floorf(L), r = L - f;
+  const bool sure = K > 0.f && hi != 0u;
+  if (sure && L - e >= (float)left) return left;
+  if (sure && r > e && r < 1.f - e) return (uint32_t)f;
+  return wc_gap_exact(d, U);
+}
+
+// K of in-degree d: the graph's table below 2^wc_inv_k, 0 (always exact) beyond;
+// in-degrees 0 and 1 draw no gaps (a graph of those alone has no table)
+__device__ __forceinline__ float wc_inv_of(const GraphView& g, uint32_t d) {
+  return d >= 2u && d < (1u << g.wc_inv_k) ? __ldg(g.wc_inv + d) : 0.f;
+}
+
 // The gap walk of one weighted-cascade node as a state machine, for the CTA
 // tier, whose lanes keep a node across rounds: d = 1 is one live edge
 // (probability 1, no draw); otherwise gap c takes the 64-bit uniform of
@@ -361,19 +384,17 @@ __device__ __forceinline__ uint32_t wc_gap(const uint64_t* P, int J, uint64_t U)
 struct GapWalk {
   uint32_t lo = 0, d = 0;   // the node's in-list
   uint32_t pos = 0, c = 0;  // position in it; gaps drawn
-  int J = 0;                // bit length of d
-  const uint64_t* P = nullptr;
+  float K = 0.f;            // -1 / log2(q)
   uint64_t spare = 0;
 };
 
 // Start the walk of node v; false when it has no in-edges.
-__device__ __forceinline__ bool walk_begin(GapWalk& w, const GraphView& g, int32_t v, uint64_t* own) {
+__device__ __forceinline__ bool walk_begin(GapWalk& w, const GraphView& g, int32_t v) {
   w.lo = __ldg(g.off + v);
   w.d = __ldg(g.off + v + 1) - w.lo;
   w.pos = 0;
   w.c = 0;
-  w.J = 32 - __clz((int)w.d);
-  w.P = w.d >= 2u ? wc_power_row(g, w.d, w.J, own) : nullptr;
+  w.K = wc_inv_of(g, w.d);
   return w.d > 0u;
 }
 
@@ -395,7 +416,7 @@ __device__ __forceinline__ uint32_t walk_step(GapWalk& w, const GraphView& g, in
     } else {
       U = w.spare;
     }
-    const uint32_t G = wc_gap(w.P, w.J, U);
+    const uint32_t G = wc_gap(w.K, w.d, w.d - w.pos, U);
     if (G >= w.d - w.pos) {
       *more = false;
       return NO_NODE;
@@ -423,10 +444,8 @@ __device__ __forceinline__ void wc_bfs_warp(const GraphView& g, const int32_t* Q
   int head = 0;
   int32_t v = -1;
   uint32_t lo = 0, d = 0, pos = 0, c = 0;
-  int Jb = 0;
+  float K = 0.f;
   uint64_t spare = 0;
-  uint64_t own[31];  // q^(2^i), i < Jb, of the lane's node when the graph's table has no row for it
-  const uint64_t* P = nullptr;
   for (;;) {
     __syncwarp();  // queue entries written by other lanes in the last round
     const bool need = v < 0;
@@ -441,8 +460,7 @@ __device__ __forceinline__ void wc_bfs_warp(const GraphView& g, const int32_t* Q
         ev += d;
         pos = 0;
         c = 0;
-        Jb = 32 - __clz((int)d);
-        if (d >= 2u) P = wc_power_row(g, d, Jb, own);
+        K = wc_inv_of(g, d);
       }
     }
     head += take;
@@ -464,7 +482,7 @@ __device__ __forceinline__ void wc_bfs_warp(const GraphView& g, const int32_t* Q
         } else {
           U = spare;
         }
-        const uint32_t G = wc_gap(P, Jb, U);
+        const uint32_t G = wc_gap(K, d, d - pos, U);
         if (G >= d - pos) {
           v = -1;
         } else {
@@ -735,7 +753,6 @@ template <int MODE>
 __global__ void __launch_bounds__(256) k_sample_lane_wc(SampleJob J) {
   const int lane = threadIdx.x & 31;
   int32_t q[LANE_Q];
-  uint64_t own[31];  // powers of a node whose in-degree has no row in the graph's table
   unsigned long long ev = 0, nv = 0, dr = 0;
   for (;;) {
     // one sample per lane; the lanes that arrive together share one atomic
@@ -759,8 +776,7 @@ __global__ void __launch_bounds__(256) k_sample_lane_wc(SampleJob J) {
       const uint32_t d = __ldg(J.g.off + v + 1) - lo;
       ev += d;
       if (d == 0u) continue;
-      const int Jb = 32 - __clz((int)d);
-      const uint64_t* P = d >= 2u ? wc_power_row(J.g, d, Jb, own) : nullptr;
+      const float K = wc_inv_of(J.g, d);
       uint32_t pos = 0, c = 0;
       uint64_t spare = 0;
       while (pos < d) {
@@ -778,7 +794,7 @@ __global__ void __launch_bounds__(256) k_sample_lane_wc(SampleJob J) {
           } else {
             U = spare;
           }
-          const uint32_t G = wc_gap(P, Jb, U);
+          const uint32_t G = wc_gap(K, d, d - pos, U);
           if (G >= d - pos) break;
           e = lo + pos + G;
           pos += G + 1u;
@@ -1019,7 +1035,6 @@ __global__ void __launch_bounds__(KIND == 1 ? SMALL_CTA_THREADS : 1024, KIND == 
         const unsigned lt_mask = (1u << lane) - 1u;
         int32_t v = -1;
         GapWalk w;
-        uint64_t own[31];  // powers of a weighted-cascade in-degree beyond the graph's table
         for (;;) {
           if (__any_sync(FULL_MASK, stopped())) break;
           const bool need = v < 0;
@@ -1049,7 +1064,7 @@ __global__ void __launch_bounds__(KIND == 1 ? SMALL_CTA_THREADS : 1024, KIND == 
                   break;
                 }
               }
-              if (x >= 0 && walk_begin(w, J.g, x, own)) v = x;
+              if (x >= 0 && walk_begin(w, J.g, x)) v = x;
               else empty = true;
               if (x >= 0) ev += w.d;
             }
