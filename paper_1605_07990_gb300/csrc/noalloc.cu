@@ -49,32 +49,59 @@ __global__ void k_na_seed_bits(const int32_t* seeds, int k, int64_t n, uint32_t*
   }
 }
 
-// hit bit of sample s - first for every entry (node, s) with a seed node
-__global__ void k_na_mark(const int32_t* __restrict__ nodes, const int32_t* __restrict__ samp, int64_t entries,
-                          int64_t n, int64_t first, int64_t count, const uint32_t* __restrict__ seed_bits,
-                          uint32_t* hit_bits, ScratchHeader* h) {
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < entries;
-       q += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t s = samp[q];
-    if (s < first || s >= first + count) continue;
-    const int32_t v = nodes[q];
-    if (v < 0 || v >= n) {
-      atomicExch(&h->bad_id, 1u);
-      continue;
-    }
-    if ((seed_bits[v >> 5] >> (v & 31)) & 1u) {
-      const int64_t i = s - first;
-      atomicOr(hit_bits + (i >> 5), 1u << (i & 31));
-    }
+// Hit bit of sample s - first for every entry (node, s) with a seed node; a bit
+// set for the first time counts, so no pass over the bits follows.  Four
+// entries per thread and 16-byte load where both arrays allow it (VEC), two
+// such loads of each in flight, the bit looked at before the atomic (the
+// entries of a hit set are neighbours).  Bound: the 8 bytes an entry.  20M
+// entries and 10^6 sets on GB300, whole call: 110 -> 75 us (scalar loads and a
+// pass over the hit bits before).
+__device__ __forceinline__ unsigned int mark_entry(int32_t v, int32_t sample, int64_t n, int64_t first, int64_t count,
+                                                   const uint32_t* __restrict__ seed_bits, uint32_t* hit_bits,
+                                                   ScratchHeader* h) {
+  const int64_t i = (int64_t)sample - first;
+  if (i < 0 || i >= count) return 0u;
+  if (v < 0 || v >= n) {
+    atomicExch(&h->bad_id, 1u);
+    return 0u;
   }
+  if (!((seed_bits[v >> 5] >> (v & 31)) & 1u)) return 0u;
+  const uint32_t mask = 1u << (i & 31);
+  if (*(volatile uint32_t*)(hit_bits + (i >> 5)) & mask) return 0u;
+  return atomicOr(hit_bits + (i >> 5), mask) & mask ? 0u : 1u;
 }
 
-__global__ void k_na_count(const uint32_t* __restrict__ hit_bits, int64_t words, ScratchHeader* h) {
-  unsigned long long c = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < words; i += (int64_t)gridDim.x * blockDim.x)
-    c += (unsigned long long)__popc(hit_bits[i]);
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_na_mark(const int32_t* __restrict__ nodes, const int32_t* __restrict__ samp,
+                                                 int64_t entries, int64_t n, int64_t first, int64_t count,
+                                                 const uint32_t* __restrict__ seed_bits, uint32_t* hit_bits,
+                                                 ScratchHeader* h) {
+  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nthr = (int64_t)gridDim.x * blockDim.x;
+  unsigned int c = 0;
+  int64_t done = 0;
+  if (VEC) {
+    const int4* n4 = reinterpret_cast<const int4*>(nodes);
+    const int4* s4 = reinterpret_cast<const int4*>(samp);
+    const int64_t quads = entries >> 2;
+    auto quad = [&](const int4& v, const int4& s) {
+      c += mark_entry(v.x, s.x, n, first, count, seed_bits, hit_bits, h);
+      c += mark_entry(v.y, s.y, n, first, count, seed_bits, hit_bits, h);
+      c += mark_entry(v.z, s.z, n, first, count, seed_bits, hit_bits, h);
+      c += mark_entry(v.w, s.w, n, first, count, seed_bits, hit_bits, h);
+    };
+    int64_t q = tid;
+    for (; q + nthr < quads; q += 2 * nthr) {
+      const int4 va = __ldcs(n4 + q), sa = __ldcs(s4 + q), vb = __ldcs(n4 + q + nthr), sb = __ldcs(s4 + q + nthr);
+      quad(va, sa);
+      quad(vb, sb);
+    }
+    if (q < quads) quad(__ldcs(n4 + q), __ldcs(s4 + q));
+    done = quads * 4;
+  }
+  for (int64_t q = done + tid; q < entries; q += nthr)
+    c += mark_entry(nodes[q], samp[q], n, first, count, seed_bits, hit_bits, h);
   c = ssa::warp_sum(c);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(&h->cov, c);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd(&h->cov, (unsigned long long)c);
 }
 
 int blocks_for(int64_t work) {
@@ -116,9 +143,13 @@ extern "C" ssa_status ssa_coverage_noalloc(int64_t n, const int32_t* nodes, cons
   if ((e = cudaMemsetAsync(base, 0, need, st)) != cudaSuccess)
     return fail_msg(SSA_E_CUDA, "ssa_coverage_noalloc: clearing scratch failed");
   if (k > 0) k_na_seed_bits<<<blocks_for(k), 256, 0, st>>>(seeds, k, n, seed_bits, h);
-  if (entries > 0 && count > 0)
-    k_na_mark<<<blocks_for(entries), 256, 0, st>>>(nodes, samp, entries, n, first, count, seed_bits, hit_bits, h);
-  if (hit_words > 0) k_na_count<<<blocks_for((int64_t)hit_words), 256, 0, st>>>(hit_bits, (int64_t)hit_words, h);
+  if (entries > 0 && count > 0) {
+    const bool vec = ((reinterpret_cast<uintptr_t>(nodes) | reinterpret_cast<uintptr_t>(samp)) & 15u) == 0;
+    if (vec) k_na_mark<true><<<blocks_for((entries + 3) / 4), 256, 0, st>>>(nodes, samp, entries, n, first, count,
+                                                                            seed_bits, hit_bits, h);
+    else k_na_mark<false><<<blocks_for(entries), 256, 0, st>>>(nodes, samp, entries, n, first, count, seed_bits,
+                                                               hit_bits, h);
+  }
   if ((e = cudaGetLastError()) != cudaSuccess) return fail_msg(SSA_E_CUDA, "ssa_coverage_noalloc: launch failed");
   ScratchHeader out{};
   if ((e = cudaMemcpyAsync(&out, h, sizeof(out), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
