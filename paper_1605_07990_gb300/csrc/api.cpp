@@ -105,6 +105,7 @@ struct ssa_graph {
   uint32_t* off = nullptr;
   uint32_t* src = nullptr;
   uint32_t* thr = nullptr;       // stored thresholds (see GraphView)
+  mutable uint32_t* lt_cum = nullptr;  // LT with explicit weights: running sums (lt_sums)
   float* wc_inv = nullptr;       // weighted cascade: gap scale per in-degree (build_wc_inv)
   int wc_inv_k = 0;
   int64_t bytes = 0;
@@ -124,7 +125,18 @@ struct ssa_graph {
     v.thr = thr;
     v.wc_inv = wc_inv;
     v.wc_inv_k = wc_inv_k;
+    v.lt_cum = lt_cum;
     return v;
+  }
+  // Running sums for LT with explicit weights, made once per graph.
+  cudaError_t lt_sums(cudaStream_t st) const {
+    std::lock_guard<std::mutex> lock(tune_mu);
+    if (lt_cum) return cudaSuccess;
+    uint32_t* c = nullptr;
+    cudaError_t e = build_lt_cum(off, thr, n, m, &c, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // other streams read them from here on
+    if (e == cudaSuccess) lt_cum = c;
+    return e;
   }
 };
 
@@ -347,9 +359,10 @@ struct Sampler {
   // every visited bit and hash slot they set, so the scratch stays ready for
   // the next batch and the next solve.
   ssa_status init_scratch(const ssa_graph* G, int mdl, Exec& X) {
-    g = G->view();
     model = mdl;
     lt_cumulative = (mdl == 1 && G->weighting == SSA_W_EXPLICIT) ? 1 : 0;
+    if (lt_cumulative) CU(G->lt_sums(X.st));
+    g = G->view();
     wc_implicit = G->weighting == SSA_W_WC ? 1 : 0;
     cfg = sampler_config(g, mdl, wc_implicit != 0);
     {
@@ -1554,6 +1567,7 @@ ssa_status ssa_free_graph(ssa_graph* g) {
   if (g->src) cudaFree(g->src);
   if (g->thr) cudaFree(g->thr);
   if (g->wc_inv) cudaFree(g->wc_inv);
+  if (g->lt_cum) cudaFree(g->lt_cum);
   delete g;
   return SSA_OK;
 }
@@ -1562,7 +1576,10 @@ ssa_status ssa_graph_info(const ssa_graph* g, int64_t* n, int64_t* m, int64_t* b
   if (!g) return fail(SSA_E_ARG, "null graph");
   if (n) *n = g->n;
   if (m) *m = g->m;
-  if (bytes) *bytes = g->bytes;
+  if (bytes) {
+    std::lock_guard<std::mutex> lock(g->tune_mu);
+    *bytes = g->bytes + (g->lt_cum ? (int64_t)sizeof(uint32_t) * g->m : 0);
+  }
   return SSA_OK;
 }
 

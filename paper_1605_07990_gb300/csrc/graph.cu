@@ -271,4 +271,101 @@ cudaError_t build_wc_inv(const uint32_t* d_off, int64_t n, float** tab, int* k_o
   return cudaSuccess;
 }
 
+namespace {
+constexpr uint32_t CUM_SHORT = 16, CUM_LONG = 4096;  // in-lists summed by a thread, by a warp, by a block
+
+__device__ __forceinline__ uint32_t cut32(unsigned long long x) {
+  return x < 0xFFFFFFFFull ? (uint32_t)x : 0xFFFFFFFFu;
+}
+
+__global__ void __launch_bounds__(256) k_lt_cum(const uint32_t* __restrict__ off, const uint32_t* __restrict__ thr,
+                                                int64_t n, uint32_t* cum, int32_t* longs, unsigned int* n_long) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t v0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) - lane; v0 < n;
+       v0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = v0 + lane;
+    const uint32_t lo = v < n ? off[v] : 0u, hi = v < n ? off[v + 1] : 0u;
+    if (hi - lo <= CUM_SHORT) {
+      unsigned long long c = 0;
+      for (uint32_t e = lo; e < hi; ++e) {
+        c += thr[e];
+        cum[e] = cut32(c);
+      }
+    } else if (hi - lo > CUM_LONG) {
+      longs[atomicAdd(n_long, 1u)] = (int32_t)v;
+    }
+    for (unsigned m = __ballot_sync(FULL_MASK, hi - lo > CUM_SHORT && hi - lo <= CUM_LONG); m; m &= m - 1u) {
+      const int o = __ffs(m) - 1;
+      const uint32_t a = __shfl_sync(FULL_MASK, lo, o), b = __shfl_sync(FULL_MASK, hi, o);
+      unsigned long long carry = 0;
+      for (uint32_t e0 = a; e0 < b; e0 += 32) {
+        unsigned long long x = e0 + lane < b ? (unsigned long long)thr[e0 + lane] : 0ull;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const unsigned long long t = __shfl_up_sync(FULL_MASK, x, d);
+          if (lane >= d) x += t;
+        }
+        x += carry;
+        if (e0 + lane < b) cum[e0 + lane] = cut32(x);
+        carry = __shfl_sync(FULL_MASK, x, 31);
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(1024) k_lt_cum_long(const uint32_t* __restrict__ off,
+                                                      const uint32_t* __restrict__ thr, uint32_t* cum,
+                                                      const int32_t* longs, const unsigned int* n_long) {
+  __shared__ unsigned long long s_w[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (unsigned int q = blockIdx.x; q < *n_long; q += gridDim.x) {
+    const int32_t v = longs[q];
+    const uint32_t a = off[v], b = off[v + 1];
+    unsigned long long carry = 0;
+    for (uint32_t e0 = a; e0 < b; e0 += 1024) {
+      const uint32_t e = e0 + threadIdx.x;
+      unsigned long long x = e < b ? (unsigned long long)thr[e] : 0ull;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const unsigned long long t = __shfl_up_sync(FULL_MASK, x, d);
+        if (lane >= d) x += t;
+      }
+      if (lane == 31) s_w[wid] = x;
+      __syncthreads();
+      unsigned long long before = carry, all = carry;
+      for (int w = 0; w < 32; ++w) {
+        if (w < wid) before += s_w[w];
+        all += s_w[w];
+      }
+      if (e < b) cum[e] = cut32(before + x);
+      carry = all;
+      __syncthreads();
+    }
+  }
+}
+}  // namespace
+
+cudaError_t build_lt_cum(const uint32_t* d_off, const uint32_t* d_thr, int64_t n, int64_t m, uint32_t** cum,
+                         cudaStream_t st) {
+  *cum = nullptr;
+  int32_t* longs = nullptr;  // one slot per long list, then their count
+  const size_t slots = (size_t)(m / CUM_LONG) + 2;
+  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&longs), sizeof(int32_t) * slots, st);
+  if (e != cudaSuccess) return e;
+  unsigned int* n_long = reinterpret_cast<unsigned int*>(longs + slots - 1);
+  e = cudaMallocAsync(reinterpret_cast<void**>(cum), sizeof(uint32_t) * (size_t)std::max<int64_t>(m, 1), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(n_long, 0, sizeof(unsigned int), st);
+  if (e == cudaSuccess) {
+    k_lt_cum<<<grid_for(n, 256), 256, 0, st>>>(d_off, d_thr, n, *cum, longs, n_long);
+    k_lt_cum_long<<<152, 1024, 0, st>>>(d_off, d_thr, *cum, longs, n_long);
+    e = cudaGetLastError();
+  }
+  cudaFreeAsync(longs, st);
+  if (e != cudaSuccess && *cum) {
+    cudaFreeAsync(*cum, st);
+    *cum = nullptr;
+  }
+  return e;
+}
+
 }  // namespace ssa

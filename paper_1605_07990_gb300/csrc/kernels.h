@@ -31,6 +31,9 @@ struct GraphView {
   // (null / 0 for other weightings)
   const float* wc_inv = nullptr;
   int wc_inv_k = 0;
+  // LT with explicit in-weights: running threshold sums of each in-list, at most
+  // 2^32 - 1 (m entries; made when the first LT sampler of the graph starts)
+  const uint32_t* lt_cum = nullptr;
 };
 
 // In-degrees of up to 2^WC_INV_K - 1 have an entry (4 MB at most); for larger
@@ -40,6 +43,10 @@ constexpr int WC_INV_K = 20;
 // That table for a CSR (every in-degree below min(2^WC_INV_K, 2 * max
 // in-degree)); *tab stays null when no in-list has 2 edges.
 cudaError_t build_wc_inv(const uint32_t* d_off, int64_t n, float** tab, int* k, cudaStream_t st);
+
+// Running sums of every in-list's thresholds, cut at 2^32 - 1 (m entries, allocated here).
+cudaError_t build_lt_cum(const uint32_t* d_off, const uint32_t* d_thr, int64_t n, int64_t m, uint32_t** cum,
+                         cudaStream_t st);
 
 // Device counters of one sampling batch.
 // Bounded waits of the weighted-cascade CTA tier that gave up (Counters::error).

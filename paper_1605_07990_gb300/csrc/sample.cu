@@ -839,15 +839,78 @@ __global__ void __launch_bounds__(256) k_sample_lane_wc(SampleJob J) {
   flush_stats(J.ctr, ev, nv, dr, lane, false);
 }
 
+// LT pick of node v with the in-list [lo, lo + d), d > 0, and its draw r: the
+// position of the kept in-edge, or NO_NODE when none is kept.  w = 1/d: one of
+// the d.  General in-weights: the first whose running threshold sum passes r,
+// found among the sums by 8-way search in a lane (seven loads at once) and
+// 33-way search in a warp (three round trips up to d = 35,000), where adding up
+// 32 thresholds at a time took d / 32 of them and the walks of a power-law
+// graph keep coming through hubs: load and D-SSA solve of 1,000,003 nodes and
+// 10M edges 8.7 -> 5.0 ms on GB300, its walks 5.6 -> 1.9.  The sums are cut at
+// 2^32 - 1, so r = 2^32 - 1 adds up the thresholds themselves.
+__device__ __noinline__ uint32_t lt_pick_sum(const GraphView& g, uint32_t lo, uint32_t d, uint32_t r) {
+  unsigned long long cum = 0;
+  for (uint32_t e = lo; e < lo + d; ++e) {
+    cum += g.thr[e];
+    if ((unsigned long long)r < cum) return e;
+  }
+  return NO_NODE;
+}
+
+__device__ __forceinline__ uint32_t lt_pick_lane(const SampleJob& J, uint32_t lo, uint32_t d, uint32_t r) {
+  if (!J.lt_cumulative) return lo + __umulhi(r, d);
+  if (r == 0xFFFFFFFFu) return lt_pick_sum(J.g, lo, d, r);
+  uint32_t a = lo, len = d;  // sums before a are <= r; the pick, if any, lies in [a, a + len)
+  while (len > 8u) {
+    uint32_t at[7];
+    int c = 0;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+      at[i] = a + (uint32_t)(((uint64_t)len * (uint32_t)(i + 1)) >> 3) - 1u;
+      c += __ldg(J.g.lt_cum + at[i]) <= r;
+    }
+    uint32_t from = a, to = a + len;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+      if (i < c) from = at[i] + 1u;
+      if (i == c) to = at[i] + 1u;
+    }
+    a = from;
+    len = to - from;
+  }
+  int c = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) c += (uint32_t)i < len && __ldg(J.g.lt_cum + a + i) <= r;
+  return a + (uint32_t)c < lo + d ? a + (uint32_t)c : NO_NODE;
+}
+
+__device__ __forceinline__ uint32_t lt_pick_warp(const SampleJob& J, uint32_t lo, uint32_t d, uint32_t r, int lane) {
+  if (!J.lt_cumulative) return lo + __umulhi(r, d);
+  if (r == 0xFFFFFFFFu) return lt_pick_sum(J.g, lo, d, r);
+  uint32_t a = lo, len = d;
+  while (len > 32u) {
+    auto at = [&](int i) { return a + (uint32_t)((uint64_t)len * (uint32_t)(i + 1) / 33u) - 1u; };
+    const int c = __popc(__ballot_sync(FULL_MASK, __ldg(J.g.lt_cum + at(lane)) <= r));
+    const uint32_t from = c ? at(c - 1) + 1u : a, to = c < 32 ? at(c) + 1u : a + len;
+    a = from;
+    len = to - from;
+  }
+  const unsigned m = __ballot_sync(FULL_MASK, (uint32_t)lane < len && __ldg(J.g.lt_cum + a + lane) > r);
+  return m ? a + (uint32_t)__ffs(m) - 1u : NO_NODE;
+}
+
 // LT live-edge walk (one keyed in-neighbour per node), warp per sample: every
 // lane follows the same walk; membership of the next node is checked by the
-// 32 lanes over the walk list in shared memory.
+// 32 lanes over the walk list in shared memory, while the loads of the next
+// step are under way.  Bound: two dependent round trips per node, and the
+// longest walk of a batch.  (A tier of one walk per lane in front, for walks of
+// up to 64 nodes, was slower: 4.3 -> 4.6 ms of walks in the 2^23-node solve.)
 template <int MODE>
 __global__ void __launch_bounds__(WT_WARPS * 32) k_sample_warp_lt(SampleJob J) {
   __shared__ int32_t s_q[WT_WARPS][LT_QCAP];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int32_t* Q = s_q[wid];
-  unsigned long long ev = 0, nv = 0, dr = 0;
+  unsigned long long ev = 0, nv = 0;
   for (;;) {
     unsigned long long idx = 0;
     if (lane == 0) idx = atomicAdd(&J.ctr->work, 1ull);
@@ -861,44 +924,23 @@ __global__ void __launch_bounds__(WT_WARPS * 32) k_sample_warp_lt(SampleJob J) {
     bool overflow = false;
     bool hit = (MODE == MODE_HIT) && test_bit(J.seed_bits, (uint32_t)root);
     int32_t cur = root;
+    uint32_t lo = __ldg(J.g.off + cur), hi = __ldg(J.g.off + cur + 1);
     __syncwarp();
-    while (!hit) {
-      const int64_t lo = __ldg(J.g.off + cur), hi = __ldg(J.g.off + cur + 1);
-      const int64_t d = hi - lo;
-      if (d == 0) break;
+    while (!hit && hi > lo) {
       const uint4 r = philox_x((uint32_t)cur, sc, J.rk);
-      int64_t pick;
-      if (!J.lt_cumulative) {
-        pick = lo + __umulhi(r.x, (uint32_t)d);  // w = 1/d_in: one of the d in-edges
-      } else {
-        // general in-weights: first in-edge whose running threshold sum passes r, or none
-        pick = -1;
-        unsigned long long carry = 0;
-        for (int64_t b = lo; b < hi; b += 32) {
-          const int64_t e = b + lane;
-          unsigned long long incl = e < hi ? (unsigned long long)__ldg(J.g.thr + e) : 0ull;
-#pragma unroll
-          for (int dd = 1; dd < 32; dd <<= 1) {
-            const unsigned long long t = __shfl_up_sync(FULL_MASK, incl, dd);
-            if (lane >= dd) incl += t;
-          }
-          const unsigned hitm = __ballot_sync(FULL_MASK, e < hi && (unsigned long long)r.x < carry + incl);
-          if (hitm) {
-            pick = b + __ffs(hitm) - 1;
-            break;
-          }
-          carry += __shfl_sync(FULL_MASK, incl, 31);
-        }
-        if (pick < 0) break;  // no in-edge kept: the walk ends here
-      }
+      const uint32_t pick = lt_pick_warp(J, lo, hi - lo, r.x, lane);
+      if (pick == NO_NODE) break;  // no in-edge kept: the walk ends here
       const int32_t u = (int32_t)__ldg(J.g.src + pick);
-      if (lane == 0) {
-        ev += 1;
-        dr += 1;
-      }
+      lo = __ldg(J.g.off + u);
+      hi = __ldg(J.g.off + u + 1);
+      if (MODE == MODE_HIT) hit = test_bit(J.seed_bits, (uint32_t)u);
+      if (lane == 0) ev += 1;
       bool found = false;
       for (int i = lane; i < tail; i += 32) found |= (Q[i] == u);
-      if (__any_sync(FULL_MASK, found)) break;
+      if (__any_sync(FULL_MASK, found)) {
+        hit = false;  // a node seen before was tested then
+        break;
+      }
       if (tail >= LT_QCAP) {
         overflow = true;
         break;
@@ -906,7 +948,6 @@ __global__ void __launch_bounds__(WT_WARPS * 32) k_sample_warp_lt(SampleJob J) {
       if (lane == 0) Q[tail] = u;
       ++tail;
       __syncwarp();
-      if (MODE == MODE_HIT) hit = test_bit(J.seed_bits, (uint32_t)u);
       cur = u;
     }
     __syncwarp();
@@ -922,7 +963,7 @@ __global__ void __launch_bounds__(WT_WARPS * 32) k_sample_warp_lt(SampleJob J) {
     }
     __syncwarp();
   }
-  flush_stats(J.ctr, ev, nv, dr, lane, false);
+  flush_stats(J.ctr, ev, nv, ev, lane, false);
 }
 
 // CTA tier: one CTA per large sample.
@@ -1176,23 +1217,10 @@ __global__ void __launch_bounds__(KIND == 1 ? SMALL_CTA_THREADS : 1024, KIND == 
       int tail = 1;
       bool hit = s_hit != 0;
       while (!hit) {
-        const int64_t lo = J.g.off[cur], hi = J.g.off[cur + 1];
-        if (hi == lo) break;
-        const uint4 r = philox_x((uint32_t)cur, sc, J.rk);
-        int64_t pick = -1;
-        if (!J.lt_cumulative) {
-          pick = lo + __umulhi(r.x, (uint32_t)(hi - lo));
-        } else {
-          unsigned long long cum = 0;
-          for (int64_t e = lo; e < hi; ++e) {
-            cum += J.g.thr[e];
-            if ((unsigned long long)r.x < cum) {
-              pick = e;
-              break;
-            }
-          }
-          if (pick < 0) break;
-        }
+        const uint32_t lo = J.g.off[cur], d = J.g.off[cur + 1] - lo;
+        if (d == 0u) break;
+        const uint32_t pick = lt_pick_lane(J, lo, d, philox_x((uint32_t)cur, sc, J.rk).x);
+        if (pick == NO_NODE) break;
         const int32_t u = (int32_t)J.g.src[pick];
         ev += 1;
         dr += 1;
