@@ -125,7 +125,7 @@ struct Tier<1> {
   static constexpr int HBITS = 15, QCAP = 16384;
 };
 constexpr int MID_HASH = 1 << Tier<1>::HBITS;
-constexpr int MID_QSLOTS = Tier<1>::QCAP + 32;  // queue/slot entries per warp (room for one round past the cap)
+constexpr int MID_QSLOTS = Tier<1>::QCAP + 64;  // queue/slot entries per warp (room for one round past the cap)
 
 template <int HBITS>
 __device__ __forceinline__ uint32_t hash_slot(uint32_t u) {
@@ -375,77 +375,87 @@ __device__ __forceinline__ float wc_inv_of(const GraphView& g, uint32_t d) {
   return d >= 2u && d < (1u << g.wc_inv_k) ? __ldg(g.wc_inv + d) : 0.f;
 }
 
-// The gap walk of one weighted-cascade node as a state machine, for the CTA
-// tier, whose lanes keep a node across rounds: d = 1 is one live edge
-// (probability 1, no draw); otherwise gap c takes the 64-bit uniform of
-// words 2(c&1), 2(c&1)+1 of the SKIP draw with counter words (v, c >> 1), the
-// next live edge is lo + pos + G, and the walk ends when G reaches past the
-// list.  (The lane tier and the warp BFS inline the same steps.)
+// The gap walk of one weighted-cascade node as a state machine: d = 1 is one
+// live edge (probability 1, no draw); otherwise gap c takes the 64-bit uniform
+// of words 2(c&1), 2(c&1)+1 of the SKIP draw with counter words (v, c >> 1), the
+// next live edge is lo + pos + G, and the walk ends when G reaches past the list.
 struct GapWalk {
   uint32_t lo = 0, d = 0;   // the node's in-list
-  uint32_t pos = 0, c = 0;  // position in it; gaps drawn
+  uint32_t pos = 0, k = 0;  // position in it; draws taken
   float K = 0.f;            // -1 / log2(q)
-  uint64_t spare = 0;
 };
 
-// Start the walk of node v; false when it has no in-edges.
-__device__ __forceinline__ bool walk_begin(GapWalk& w, const GraphView& g, int32_t v) {
-  w.lo = __ldg(g.off + v);
-  w.d = __ldg(g.off + v + 1) - w.lo;
+__device__ __forceinline__ void walk_begin(GapWalk& w, const GraphView& g, uint32_t lo, uint32_t d) {
+  w.lo = lo;
+  w.d = d;
   w.pos = 0;
-  w.c = 0;
-  w.K = wc_inv_of(g, w.d);
-  return w.d > 0u;
+  w.k = 0;
+  w.K = wc_inv_of(g, d);
 }
 
-// One step: the tail of the next live edge, or NO_NODE when the node has no
-// more; *more says whether the node may still give live edges.
-__device__ __forceinline__ uint32_t walk_step(GapWalk& w, const GraphView& g, int32_t v, const uint32_t* rk,
-                                              const SampleConst& skc, unsigned long long& draws, bool* more) {
-  uint32_t e;
-  if (w.d == 1u) {
-    e = w.lo;
-    w.pos = 1;
-  } else {
-    uint64_t U;
-    if (!(w.c & 1u)) {
-      const uint4 r = philox_xy((uint32_t)v, w.c >> 1, skc, rk);
-      ++draws;
-      U = (uint64_t)r.x | ((uint64_t)r.y << 32);
-      w.spare = (uint64_t)r.z | ((uint64_t)r.w << 32);
-    } else {
-      U = w.spare;
-    }
-    const uint32_t G = wc_gap(w.K, w.d, w.d - w.pos, U);
-    if (G >= w.d - w.pos) {
-      *more = false;
-      return NO_NODE;
-    }
-    e = w.lo + w.pos + G;
-    w.pos += G + 1u;
-    ++w.c;
+// One step: the two gaps of a draw at once, so that a node with at most one
+// live edge (three in four) is done in one round and two edges' loads go out
+// together.  e0, e1: CSR positions of the live edges found (NO_NODE: none).
+// Returns whether the node may still give live edges.
+__device__ __forceinline__ bool walk_step(GapWalk& w, int32_t v, const uint32_t* rk, const SampleConst& skc,
+                                          unsigned long long& draws, uint32_t& e0, uint32_t& e1) {
+  e0 = e1 = NO_NODE;
+  if (w.d < 2u) {
+    if (w.d == 1u) e0 = w.lo;
+    return false;
   }
-  *more = w.pos < w.d;
-  return __ldg(g.src + e);
+  const uint4 r = philox_xy((uint32_t)v, w.k, skc, rk);
+  ++draws;
+  ++w.k;
+  uint32_t left = w.d - w.pos;
+  uint32_t G = wc_gap(w.K, w.d, left, (uint64_t)r.x | ((uint64_t)r.y << 32));
+  if (G >= left) return false;
+  e0 = w.lo + w.pos + G;
+  w.pos += G + 1u;
+  left -= G + 1u;
+  if (left == 0u) return false;
+  G = wc_gap(w.K, w.d, left, (uint64_t)r.z | ((uint64_t)r.w << 32));
+  if (G >= left) return false;
+  e1 = w.lo + w.pos + G;
+  w.pos += G + 1u;
+  return w.pos < w.d;
 }
+
+// The last WRING nodes of a warp's queue with their in-lists, in shared memory:
+// entry p of the queue at p mod WRING.  (The queue of the global-memory tiers
+// is written in any case: it is the RR set.)
+constexpr int WRING = 64;
+struct WarpRing {
+  int32_t* node;  // null: the queue itself is in shared memory
+  uint32_t* lo;
+  uint32_t* d;
+};
 
 // Weighted-cascade BFS of one sample by one warp over its private queue
-// Q[0, tail) (head = 0 at the start): every lane holds at most one node and
-// takes one gap step per round; a lane whose node is done takes the next
-// queued node at the start of the next round, so the lanes stay busy while
-// the queue holds work (a node's walk is the gap walk of walk_step, the same
-// keyed draws).  visit(u, lt_mask) appends new nodes to Q and advances tail
-// (which this function reads through the reference); it returns "stop".
+// Q[0, tail) (head = 0 at the start; the root's ring entry is set): every lane
+// holds at most one node and takes one walk step (two gaps) per round; a lane
+// whose node is done takes the next queued node at the start of the next round,
+// so the lanes stay busy while the queue holds work.  visit(u, lo, d) with two
+// tails and their in-lists per lane (NO_NODE: none) appends the new ones to Q
+// and the ring and advances tail (which this function reads through the
+// reference); it returns "stop".
+//
+// Near-critical sets are deep and narrow (5000 nodes: over 100 levels), and a
+// batch ends with its largest set, so what counts is the chain of dependent
+// loads per level: the edge's tail, then the visited bit together with the
+// tail's offsets, which are loaded before it is known to be new and wait in the
+// ring.  Sampling of a whole solve on GB300, one gap and its offsets on demand
+// before: 17.2 -> 13.5 ms (SSA, 2^25 nodes), 6.7 -> 5.0 ms (D-SSA, 2^23).  (More
+// warps per SM at 40 or 48 registers gained nothing: the batches' ends wait on
+// single sets.)
 template <class Visit>
-__device__ __forceinline__ void wc_bfs_warp(const GraphView& g, const int32_t* Q, const int& tail,
-                                            const uint32_t* rk, const SampleConst& skc, int lane,
+__device__ __forceinline__ void wc_bfs_warp(const GraphView& g, const int32_t* Q, const WarpRing& ring,
+                                            const int& tail, const uint32_t* rk, const SampleConst& skc, int lane,
                                             unsigned long long& ev, unsigned long long& draws, Visit&& visit) {
   const unsigned lt_mask = (1u << lane) - 1u;
   int head = 0;
   int32_t v = -1;
-  uint32_t lo = 0, d = 0, pos = 0, c = 0;
-  float K = 0.f;
-  uint64_t spare = 0;
+  GapWalk w;
   for (;;) {
     __syncwarp();  // queue entries written by other lanes in the last round
     const bool need = v < 0;
@@ -454,46 +464,38 @@ __device__ __forceinline__ void wc_bfs_warp(const GraphView& g, const int32_t* Q
     if (need) {
       const int r = __popc(nm & lt_mask);
       if (r < take) {
-        v = Q[head + r];
-        lo = __ldg(g.off + v);
-        d = __ldg(g.off + v + 1) - lo;
+        const int h = head + r;
+        uint32_t lo, d;
+        if (tail - h <= WRING) {
+          v = ring.node ? ring.node[h & (WRING - 1)] : Q[h];
+          lo = ring.lo[h & (WRING - 1)];
+          d = ring.d[h & (WRING - 1)];
+        } else {
+          v = Q[h];
+          lo = __ldg(g.off + v);
+          d = __ldg(g.off + v + 1) - lo;
+        }
         ev += d;
-        pos = 0;
-        c = 0;
-        K = wc_inv_of(g, d);
+        walk_begin(w, g, lo, d);
       }
     }
     head += take;
     if (!__any_sync(FULL_MASK, v >= 0)) break;  // queue drained, no lane holds a node
-    uint32_t u = NO_NODE;
+    uint32_t u[2] = {NO_NODE, NO_NODE}, lo[2] = {0u, 0u}, hi[2] = {0u, 0u};
     if (v >= 0) {
-      if (d == 0u) {
-        v = -1;
-      } else if (d == 1u) {
-        u = __ldg(g.src + lo);
-        v = -1;
-      } else {
-        uint64_t U;
-        if (!(c & 1u)) {
-          const uint4 r = philox_xy((uint32_t)v, c >> 1, skc, rk);
-          ++draws;
-          U = (uint64_t)r.x | ((uint64_t)r.y << 32);
-          spare = (uint64_t)r.z | ((uint64_t)r.w << 32);
-        } else {
-          U = spare;
+      uint32_t e0, e1;
+      if (!walk_step(w, v, rk, skc, draws, e0, e1)) v = -1;
+      if (e0 != NO_NODE) u[0] = __ldg(g.src + e0);
+      if (e1 != NO_NODE) u[1] = __ldg(g.src + e1);
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+        if (u[t] != NO_NODE) {
+          lo[t] = __ldg(g.off + u[t]);
+          hi[t] = __ldg(g.off + u[t] + 1);
         }
-        const uint32_t G = wc_gap(K, d, d - pos, U);
-        if (G >= d - pos) {
-          v = -1;
-        } else {
-          u = __ldg(g.src + lo + pos + G);
-          pos += G + 1u;
-          ++c;
-          if (pos >= d) v = -1;
-        }
-      }
     }
-    if (visit(u, lt_mask)) return;
+    const uint32_t d[2] = {hi[0] - lo[0], hi[1] - lo[1]};
+    if (visit(u, lo, d, lt_mask)) return;
   }
 }
 
@@ -552,7 +554,10 @@ __global__ void __launch_bounds__(WT_WARPS * 32, 4) k_sample_warp_ic(SampleJob J
   __shared__ int32_t s_q[TIER == 0 ? WT_WARPS : 1][TIER == 0 ? WT_QCAP : 4];
   __shared__ uint32_t s_stage[WT_WARPS][WC ? 1 : STAGE];  // the gap walk needs no staging
   __shared__ unsigned int s_staged[WT_WARPS];
+  __shared__ uint32_t s_ring[WT_WARPS][WC ? (TIER == 0 ? 2 : 3) * WRING : 1];  // the gap walk's ring
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const WarpRing ring{TIER == 0 ? nullptr : reinterpret_cast<int32_t*>(s_ring[wid] + 2 * WRING), s_ring[wid],
+                      s_ring[wid] + WRING};
   const size_t gwarp = (size_t)blockIdx.x * WT_WARPS + wid;
   uint32_t* H = TIER == 0 ? s_hash[wid] : J.mid_hash + gwarp * MID_HASH;
   int32_t* Q = TIER == 0 ? s_q[wid] : J.mid_queue + gwarp * MID_QSLOTS;
@@ -583,6 +588,11 @@ __global__ void __launch_bounds__(WT_WARPS * 32, 4) k_sample_warp_ic(SampleJob J
       H[h0] = (uint32_t)root + 1u;
       Q[0] = root;
       if (TIER == 1) slots[0] = h0;
+      if (WC) {
+        ring.lo[0] = __ldg(J.g.off + root);
+        ring.d[0] = __ldg(J.g.off + root + 1) - ring.lo[0];
+        if (TIER == 1) ring.node[0] = root;
+      }
     }
     int tail = 1, head = 0;
     bool overflow = false;
@@ -590,32 +600,46 @@ __global__ void __launch_bounds__(WT_WARPS * 32, 4) k_sample_warp_ic(SampleJob J
     // tier 1's hand-over size is tuned at run time (at most its queue capacity)
     const int cap = TIER == 0 ? QCAP : min(QCAP, J.mid_cap);
     __syncwarp();
-    auto visit = [&](uint32_t u, unsigned lt_mask) -> bool {
-      uint32_t slot = 0;
-      const bool is_new = (u != NO_NODE) && hash_insert<HBITS>(H, u, &slot);
-      const unsigned m = __ballot_sync(FULL_MASK, is_new);
+    auto enter = [&](const uint32_t (&u)[2], const uint32_t (&ulo)[2], const uint32_t (&ud)[2],
+                     unsigned lt_mask) -> bool {
       bool h = false;
-      if (is_new) {
-        const int pos = tail + __popc(m & lt_mask);
-        if (TIER == 0) {
-          if (pos < QCAP) Q[pos] = (int32_t)u;
-        } else {
-          Q[pos] = (int32_t)u;  // pos <= cap + 31 < QCAP + 32: room for one round past the cap
-          slots[pos] = slot;
+#pragma unroll
+      for (int t = 0; t < (WC ? 2 : 1); ++t) {
+        if (t == 1 && !__any_sync(FULL_MASK, u[1] != NO_NODE)) break;
+        uint32_t slot = 0;
+        const bool is_new = (u[t] != NO_NODE) && hash_insert<HBITS>(H, u[t], &slot);
+        const unsigned m = __ballot_sync(FULL_MASK, is_new);
+        if (is_new) {
+          const int pos = tail + __popc(m & lt_mask);
+          if (WC) {
+            ring.lo[pos & (WRING - 1)] = ulo[t];
+            ring.d[pos & (WRING - 1)] = ud[t];
+            if (TIER == 1) ring.node[pos & (WRING - 1)] = (int32_t)u[t];
+          }
+          if (TIER == 0) {
+            if (pos < QCAP) Q[pos] = (int32_t)u[t];
+          } else {
+            Q[pos] = (int32_t)u[t];  // pos <= cap + 63 < QCAP + 64: room for one round past the cap
+            slots[pos] = slot;
+          }
+          if (MODE == MODE_HIT) h |= test_bit(J.seed_bits, u[t]);
         }
-        if (MODE == MODE_HIT) h = test_bit(J.seed_bits, u);
+        tail += __popc(m);
       }
-      tail += __popc(m);
       if (MODE == MODE_HIT) hit = __any_sync(FULL_MASK, h) || hit;
       if (tail > cap) overflow = true;
       return overflow || hit;
+    };
+    auto visit = [&](uint32_t u, unsigned lt_mask) -> bool {
+      const uint32_t us[2] = {u, NO_NODE}, none[2] = {0u, 0u};
+      return enter(us, none, none, lt_mask);
     };
     // a node with a very long in-list needs many warps: hand the sample to the CTA tier
     // (weighted cascade: no in-list is long, its gap walk costs the same at any degree)
     auto to_cta = [](int32_t, uint32_t, uint32_t, int) { return HEAVY_ABORT; };
     bool handoff = false;
     if constexpr (WC) {
-      if (!hit) wc_bfs_warp(J.g, Q, tail, J.rk, sc, lane, ev, dr, visit);
+      if (!hit) wc_bfs_warp(J.g, Q, ring, tail, J.rk, sc, lane, ev, dr, enter);
     } else {
       while (head < tail && !overflow && !hit) {
         const int cnt = min(32, tail - head);
@@ -657,7 +681,7 @@ __global__ void __launch_bounds__(WT_WARPS * 32, 4) k_sample_warp_ic(SampleJob J
       uint4* H4 = reinterpret_cast<uint4*>(H);
       for (int i = lane; i < WT_HASH / 4; i += 32) H4[i] = make_uint4(0, 0, 0, 0);
     } else {
-      // clear only the slots this sample used (tail <= QCAP + 32 entries recorded)
+      // clear only the slots this sample used (tail <= QCAP + 64 entries recorded)
       for (int i = lane; i < tail; i += 32) H[slots[i]] = 0u;
     }
     __syncwarp();
@@ -671,11 +695,13 @@ __global__ void __launch_bounds__(WT_WARPS * 32, 4) k_sample_warp_ic(SampleJob J
 // queue, where the hash tiers stop at 512 and 16384 nodes.  Larger sets go to
 // the CTA tier.
 constexpr int GQ_CAP = 1 << 16;
-constexpr int GQ_SLOTS = GQ_CAP + 32;  // room for one round past the cap
+constexpr int GQ_SLOTS = GQ_CAP + 64;  // room for one round past the cap
 
 template <int MODE>
 __global__ void __launch_bounds__(WT_WARPS * 32, 4) k_sample_warp_wcg(SampleJob J) {
+  __shared__ uint32_t s_ring[WT_WARPS][3 * WRING];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const WarpRing ring{reinterpret_cast<int32_t*>(s_ring[wid] + 2 * WRING), s_ring[wid], s_ring[wid] + WRING};
   const size_t gwarp = (size_t)blockIdx.x * WT_WARPS + wid;
   uint32_t* bits = J.wg_bitmap + gwarp * (size_t)J.bitmap_words;
   int32_t* Q = J.wg_queue + gwarp * (size_t)GQ_SLOTS;
@@ -696,29 +722,40 @@ __global__ void __launch_bounds__(WT_WARPS * 32, 4) k_sample_warp_wcg(SampleJob 
     if (lane == 0) {
       atomicOr(bits + (root >> 5), 1u << (root & 31));
       Q[0] = root;
+      ring.node[0] = root;
+      ring.lo[0] = __ldg(J.g.off + root);
+      ring.d[0] = __ldg(J.g.off + root + 1) - ring.lo[0];
     }
     int tail = 1;
     bool overflow = false;
     bool hit = (MODE == MODE_HIT) && test_bit(J.seed_bits, (uint32_t)root);
     __syncwarp();
-    auto visit = [&](uint32_t u, unsigned lt_mask) -> bool {
-      bool is_new = false;
-      if (u != NO_NODE) {
-        const uint32_t mask = 1u << (u & 31);
-        is_new = !(atomicOr(bits + (u >> 5), mask) & mask);
-      }
-      const unsigned m = __ballot_sync(FULL_MASK, is_new);
+    auto visit = [&](const uint32_t (&u)[2], const uint32_t (&ulo)[2], const uint32_t (&ud)[2],
+                     unsigned lt_mask) -> bool {
+      uint32_t old[2] = {0u, 0u};
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+        if (u[t] != NO_NODE) old[t] = atomicOr(bits + (u[t] >> 5), 1u << (u[t] & 31));
       bool h = false;
-      if (is_new) {
-        Q[tail + __popc(m & lt_mask)] = (int32_t)u;  // tail <= cap <= GQ_CAP before this round: fits GQ_SLOTS
-        if (MODE == MODE_HIT) h = test_bit(J.seed_bits, u);
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const bool is_new = u[t] != NO_NODE && !((old[t] >> (u[t] & 31)) & 1u);
+        const unsigned m = __ballot_sync(FULL_MASK, is_new);
+        if (is_new) {
+          const int pos = tail + __popc(m & lt_mask);
+          Q[pos] = (int32_t)u[t];  // tail <= cap <= GQ_CAP before this round: fits GQ_SLOTS
+          ring.node[pos & (WRING - 1)] = (int32_t)u[t];
+          ring.lo[pos & (WRING - 1)] = ulo[t];
+          ring.d[pos & (WRING - 1)] = ud[t];
+          if (MODE == MODE_HIT) h |= test_bit(J.seed_bits, u[t]);
+        }
+        tail += __popc(m);
       }
-      tail += __popc(m);
       if (MODE == MODE_HIT) hit = __any_sync(FULL_MASK, h) || hit;
       if (tail > cap) overflow = true;
       return overflow || hit;
     };
-    if (!hit) wc_bfs_warp(J.g, Q, tail, J.rk, sc, lane, ev, dr, visit);
+    if (!hit) wc_bfs_warp(J.g, Q, ring, tail, J.rk, sc, lane, ev, dr, visit);
     __syncwarp();
     if (overflow) {
       if (lane == 0) {
@@ -753,6 +790,7 @@ template <int MODE>
 __global__ void __launch_bounds__(256) k_sample_lane_wc(SampleJob J) {
   const int lane = threadIdx.x & 31;
   int32_t q[LANE_Q];
+  uint32_t qlo[LANE_Q], qd[LANE_Q];  // the queued nodes' in-lists, loaded when the node is found
   unsigned long long ev = 0, nv = 0, dr = 0;
   for (;;) {
     // one sample per lane; the lanes that arrive together share one atomic
@@ -767,51 +805,44 @@ __global__ void __launch_bounds__(256) k_sample_lane_wc(SampleJob J) {
     const SampleConst sc = sample_const(J.rk, (uint32_t)j, ctr_word3(PURPOSE_SKIP, J.stream, j));
     const int32_t root = pick_root(J, j);
     q[0] = root;
+    qlo[0] = __ldg(J.g.off + root);
+    qd[0] = __ldg(J.g.off + root + 1) - qlo[0];
     int tail = 1;
     bool hit = (MODE == MODE_HIT) && test_bit(J.seed_bits, (uint32_t)root);
     bool overflow = false;
     for (int h = 0; h < tail && !hit && !overflow; ++h) {
       const int32_t v = q[h];
-      const uint32_t lo = __ldg(J.g.off + v);
-      const uint32_t d = __ldg(J.g.off + v + 1) - lo;
-      ev += d;
-      if (d == 0u) continue;
-      const float K = wc_inv_of(J.g, d);
-      uint32_t pos = 0, c = 0;
-      uint64_t spare = 0;
-      while (pos < d) {
-        uint32_t e;
-        if (d == 1u) {
-          e = lo;
-          pos = 1;
-        } else {
-          uint64_t U;
-          if (!(c & 1u)) {
-            const uint4 r = philox_xy((uint32_t)v, c >> 1, sc, J.rk);
-            ++dr;
-            U = (uint64_t)r.x | ((uint64_t)r.y << 32);
-            spare = (uint64_t)r.z | ((uint64_t)r.w << 32);
-          } else {
-            U = spare;
+      GapWalk w;
+      walk_begin(w, J.g, qlo[h], qd[h]);
+      ev += w.d;
+      for (bool more = true; more && !hit && !overflow;) {
+        uint32_t e[2];
+        more = walk_step(w, v, J.rk, sc, dr, e[0], e[1]);
+        uint32_t u[2] = {NO_NODE, NO_NODE}, ulo[2] = {0u, 0u}, uhi[2] = {0u, 0u};
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+          if (e[t] != NO_NODE) u[t] = __ldg(J.g.src + e[t]);
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+          if (u[t] != NO_NODE) {
+            ulo[t] = __ldg(J.g.off + u[t]);
+            uhi[t] = __ldg(J.g.off + u[t] + 1);
           }
-          const uint32_t G = wc_gap(K, d, d - pos, U);
-          if (G >= d - pos) break;
-          e = lo + pos + G;
-          pos += G + 1u;
-          ++c;
-        }
-        const int32_t u = (int32_t)__ldg(J.g.src + e);
-        bool seen = false;
-        for (int i = 0; i < tail; ++i) seen |= q[i] == u;
-        if (seen) continue;
-        if (tail == LANE_Q) {
-          overflow = true;
-          break;
-        }
-        q[tail++] = u;
-        if (MODE == MODE_HIT && test_bit(J.seed_bits, (uint32_t)u)) {
-          hit = true;
-          break;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          if (u[t] == NO_NODE || hit || overflow) continue;
+          bool seen = false;
+          for (int i = 0; i < tail; ++i) seen |= q[i] == (int32_t)u[t];
+          if (seen) continue;
+          if (tail == LANE_Q) {
+            overflow = true;
+            continue;
+          }
+          q[tail] = (int32_t)u[t];
+          qlo[tail] = ulo[t];
+          qd[tail] = uhi[t] - ulo[t];
+          ++tail;
+          if (MODE == MODE_HIT && test_bit(J.seed_bits, u[t])) hit = true;
         }
       }
     }
@@ -1105,22 +1136,28 @@ __global__ void __launch_bounds__(KIND == 1 ? SMALL_CTA_THREADS : 1024, KIND == 
                   break;
                 }
               }
-              if (x >= 0 && walk_begin(w, J.g, x)) v = x;
+              if (x >= 0) {
+                const uint32_t lo = __ldg(J.g.off + x);
+                walk_begin(w, J.g, lo, __ldg(J.g.off + x + 1) - lo);
+                ev += w.d;
+              }
+              if (x >= 0 && w.d > 0u) v = x;
               else empty = true;
-              if (x >= 0) ev += w.d;
             }
           }
-          uint32_t u = NO_NODE;
+          uint32_t u0 = NO_NODE, u1 = NO_NODE;
           bool fin = false;
           if (v >= 0) {
-            bool more = true;
-            u = walk_step(w, J.g, v, J.rk, sc, dr, &more);
-            if (!more) {
+            uint32_t e0, e1;
+            if (!walk_step(w, v, J.rk, sc, dr, e0, e1)) {
               v = -1;
               fin = true;
             }
+            if (e0 != NO_NODE) u0 = __ldg(J.g.src + e0);
+            if (e1 != NO_NODE) u1 = __ldg(J.g.src + e1);
           }
-          if (visit(u, lt_mask)) break;
+          if (visit(u0, lt_mask)) break;
+          if (__any_sync(FULL_MASK, u1 != NO_NODE) && visit(u1, lt_mask)) break;
           const int nret = __popc(__ballot_sync(FULL_MASK, fin || empty));
           if (lane == 0 && nret) {
             __threadfence_block();  // the nodes they queued before they are retired
