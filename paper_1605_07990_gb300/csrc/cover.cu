@@ -103,6 +103,9 @@ constexpr int GCANDS = GREEDY_CANDS;  // candidates of one session: their gains,
 constexpr int GBITS = 14;          // a candidate's key: gain above, GCANDS - 1 - local id in the low GBITS
 constexpr int GMAX = 1 << (32 - GBITS);
 constexpr int GBINS = 1024;        // histogram bins
+constexpr int SCANDS = 4096;       // candidates and list entries of a session that fits shared memory whole:
+constexpr int SENTS = 24576;       // keys, ids, offsets, lengths (12 bytes a candidate), lists (6 an entry)
+constexpr int STHREADS = 256;      // threads that make its picks
 constexpr int GHISTS = 4;          // histograms in turn, so that one is cleared while another fills
 constexpr int GLONG = 256;         // members of a set beyond which its list is made by several warps
 
@@ -312,6 +315,12 @@ __device__ __forceinline__ void for_live_members(const GreedyJob& J, int64_t war
 // 6.0 -> 2.1 ms, 100 over 1,149,440 sets of the 2^25-node one 3.5 -> 2.0 ms,
 // each with its index (0.2, 0.3 and 1.6 ms) gone.
 //
+// With many picks to go and gains of some hundreds at most, the candidates and
+// all their lists fit shared memory (`small`: SCANDS candidates, SENTS entries):
+// eight warps then pick without a load from memory.  The 1000 picks above went
+// from 1.81 to 1.28 ms a round with it (a session of 1.5 us picks ends after 64
+// of them where 192 are left; one that served fewer than 96 is not tried again).
+//
 // Gains of 0 go by smallest id.  Barrier waits are bounded (sync[SYNC_ERR] on
 // timeout); a session makes at most GCANDS picks, milliseconds, between two
 // barriers.
@@ -332,7 +341,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
   const int64_t warp = gtid >> 5, nwarps = gthreads >> 5;
   const int64_t n4 = J.n_pad >> 2;
   int n_argmax = 0, n_hist = 0, i = 0;
-  bool first = true, bulk = J.bulk_first != 0, flat = false;
+  bool first = true, bulk = J.bulk_first != 0, flat = false, small_off = false;
   if (tid == 0) s_phase = 0u;  // the host zeroed the release word (sense 0)
   unsigned long long info = 0;
 
@@ -400,9 +409,10 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
     return true;
   };
   // The lowest bin b such that, with `have` nodes of `sum` list entries taken
-  // already, the nodes of bins >= b still fit (GCANDS nodes, ents_cap list
-  // entries; top(b): largest gain of bin b).  Returns b, adds what they take to
+  // already, the nodes of bins >= b still fit (cap_n nodes, cap_e list entries;
+  // top(b): largest gain of bin b).  Returns b, adds what they take to
   // have and sum; *total: nodes in all bins.
+  long long cap_n = GCANDS, cap_e = J.ents_cap;
   auto cut = [&](const unsigned int* hist, auto&& top, long long& have, long long& sum, long long* total) -> int {
     const int b = GBINS - 1 - tid;  // 1024 threads: one bin each, from the top
     const long long c = __ldcg(hist + b);
@@ -411,7 +421,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
     *total = s_scan_tot;
     __syncthreads();
     const long long is = block_exclusive_scan<long long>(e, s_scan, &s_scan_tot) + e;
-    const bool fits = have + ic <= GCANDS && sum + is <= (long long)J.ents_cap;
+    const bool fits = have + ic <= cap_n && sum + is <= cap_e;
     // bins fit from the top down to the first that does not
     const unsigned long long n_fit = GBINS - block_max(fits ? 0ull : (unsigned long long)(GBINS - tid), s_red);
     __shared__ long long s_have, s_sum;
@@ -469,7 +479,11 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
     }
     const bool session = !bulk || (first && !wide);  // else recount before the next session
     unsigned long long keystar = 0;
+    const bool small = session && !first && !small_off && J.k - i >= 64 && key_gain(best) <= SENTS / 64;
+    const int i0 = i;
     if (session) {
+      cap_n = small ? SCANDS : GCANDS;
+      cap_e = small ? SENTS : (long long)J.ents_cap;
       long long have = 0, sum = 0, total = 0;
       int b = cut(hist, [](int x) { return bin_gain(x + 1) - 1; }, have, sum, &total);
       b = max(b, 1);
@@ -684,7 +698,95 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
     if (session) {
       const int nc = (int)__ldcg(J.ncand);
       overflow = overflow || nc == 0;
-      if (blockIdx.x == 0 && !overflow) {
+      if (blockIdx.x == 0 && !overflow && small) {
+        // everything into shared memory: the lists of the sets one after the
+        // other (count, local ids; count 0: covered), the candidates' lists as
+        // places in them
+        s_id = s_key + SCANDS;
+        unsigned short* s_off16 = reinterpret_cast<unsigned short*>(s_id + SCANDS);
+        unsigned short* s_len16 = s_off16 + SCANDS;
+        unsigned short* s_ent16 = s_len16 + SCANDS;
+        unsigned short* s_mem = s_ent16 + SENTS;
+        __shared__ unsigned int s_nmem;
+        if (tid == 0) s_nmem = 0u;
+        const int E = (int)__ldcg(J.ncand + 4);
+        for (int t = tid; t < SCANDS; t += 1024) {
+          const unsigned int len = t < nc ? (unsigned int)__ldcg(J.cand_len + t) : 0u;
+          s_key[t] = t < nc ? (len << GBITS) | (unsigned int)(GCANDS - 1 - t) : 0u;
+          s_id[t] = t < nc ? (unsigned int)__ldcg(J.cand_id + t) : 0u;
+          s_off16[t] = t < nc ? (unsigned short)__ldcg(J.cand_off + t) : 0;
+          s_len16[t] = (unsigned short)len;
+        }
+        __syncthreads();
+        // the first list entry of a set to come (it sets the count's high bit) copies the set
+        for (int x0 = tid; x0 < E; x0 += 4096) {
+          unsigned int at[4], old[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t) at[t] = x0 + 1024 * t < E ? __ldcg(J.ents + x0 + 1024 * t) : 0u;
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+            old[t] = x0 + 1024 * t < E ? atomicOr(reinterpret_cast<unsigned int*>(J.chunks + at[t]), 0x80000000u)
+                                       : 0x80000000u;
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            if (old[t] >> 31) continue;
+            const unsigned int place = atomicAdd(&s_nmem, old[t] + 1u);
+            s_mem[place] = (unsigned short)old[t];
+            const unsigned short* ids = reinterpret_cast<const unsigned short*>(J.chunks + at[t]) + 4;
+            for (unsigned int y = 0; y < old[t]; ++y) s_mem[place + 1u + y] = __ldcg(ids + y);
+            *reinterpret_cast<unsigned int*>(J.chunks + at[t]) = 0x80000000u | place;
+          }
+        }
+        __syncthreads();
+        for (int x = tid; x < E; x += 1024)
+          s_ent16[x] =
+              (unsigned short)__ldcg(reinterpret_cast<const unsigned int*>(J.chunks + __ldcg(J.ents + x)));
+        __syncthreads();
+        if (tid < STHREADS) {
+          // as the picks below, by eight warps and without a load from memory
+          auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(STHREADS) : "memory"); };
+          unsigned int bk = 0xFFFFFFFFu;
+          int par = 0;
+          while (i < J.k) {
+            if (bk && s_key[(GCANDS - 1 - (bk & (GCANDS - 1))) & (SCANDS - 1)] != bk) {
+              bk = 0u;
+#pragma unroll
+              for (int r = 0; r < SCANDS / STHREADS; ++r) bk = max(bk, s_key[r * STHREADS + tid]);
+            }
+            const unsigned int wk = __reduce_max_sync(FULL_MASK, bk);
+            if (lane == 0) s_w[par][wid] = wk;
+            sync();
+            const unsigned int top = __reduce_max_sync(FULL_MASK, lane < STHREADS / 32 ? s_w[par][lane] : 0u);
+            par ^= 1;
+            const int l = GCANDS - 1 - (int)(top & (GCANDS - 1));
+            const int g = (int)(top >> GBITS);
+            if (top == 0u || gain_key(g, s_id[l]) < keystar) break;
+            if (tid == 0) {
+              J.seeds[i] = (int32_t)s_id[l];
+              J.gains[i] = g;
+              s_key[l] = 0u;  // never again; the loop below leaves it alone
+            }
+            const int off = s_off16[l], len = s_len16[l];
+            for (int x = tid; x < len; x += STHREADS) {
+              const int m = s_ent16[off + x];
+              const int c = s_mem[m];
+              if (c) s_mem[m] = 0;
+              for (int y = 1; y <= c; ++y) {
+                const int w = s_mem[m + y];
+                if (w != l) atomicSub(s_key + w, 1u << GBITS);
+              }
+            }
+            i += 1;
+            sync();
+          }
+        }
+        __syncthreads();
+        // the covered flags of the sets whose count is 0 now
+        for (int x = tid; x < E; x += 1024)
+          if (s_mem[s_ent16[x]] == 0)
+            J.covered[__ldcg(reinterpret_cast<const uint2*>(J.chunks + __ldcg(J.ents + x))).y] = 1;
+        s_id = s_key + GCANDS;
+      } else if (blockIdx.x == 0 && !overflow) {
         const int ncp = (nc + 1023) & ~1023;
         for (int t = tid; t < ncp; t += 1024) {
           s_key[t] = t < nc ? ((unsigned int)__ldcg(J.cand_len + t) << GBITS) | (unsigned int)(GCANDS - 1 - t) : 0u;
@@ -712,6 +814,8 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
           const int g = (int)(top >> GBITS);
           const unsigned int off = s_off[l], v = s_id[l];
           if (top == 0u || gain_key(g, v) < keystar) break;
+          // with many picks to go and gains this small, a session out of shared memory is quicker
+          if (!small_off && i - i0 >= 64 && J.k - i >= 192 && g <= SENTS / 96) break;
           const int len = __ldcg(J.cand_len + l);
           // lanes per set: eight chunks of each set at once while the sets are few, else two
           const unsigned int spec = __ldcg(J.ents + off + (tid >> 3));  // the buffer has spare entries past the last list
@@ -783,6 +887,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
       if (!greedy_barrier<CLUSTER>(J, &s_phase, [&] { return (unsigned long long)__ldcg(J.ncand + 2); }, info)) return;
       i = (int)info;
       if (i >= J.k) break;
+      if (small && i - i0 < 96) small_off = true;  // it did not pay for its lists
     }
     // ---- gains again over the sets left ----
     for (int64_t q = gtid; q < n4; q += gthreads) reinterpret_cast<int4*>(J.cnt)[q] = make_int4(0, 0, 0, 0);
