@@ -68,6 +68,49 @@ __device__ __forceinline__ T block_exclusive_scan(T x, T* s_warp, T* total) {
   return r;
 }
 
+// ---- WRIS prefix sums ----
+constexpr int PREFIX_TILE = 4096;  // 1024 threads x 4
+
+__device__ __forceinline__ void load_weights(const uint32_t* w, int64_t n, unsigned long long (&x)[4],
+                                             unsigned long long* sum) {
+  const int64_t base = (int64_t)blockIdx.x * PREFIX_TILE + (int64_t)threadIdx.x * 4;
+  *sum = 0;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    x[t] = base + t < n ? w[base + t] : 0u;
+    *sum += x[t];
+  }
+}
+
+__global__ void __launch_bounds__(1024) k_weight_tiles(const uint32_t* w, int64_t n, unsigned long long* part) {
+  __shared__ unsigned long long s_w[32], s_tot;
+  unsigned long long x[4], sum;
+  load_weights(w, n, x, &sum);
+  block_exclusive_scan<unsigned long long>(sum, s_w, &s_tot);
+  if (threadIdx.x == 0) part[blockIdx.x] = s_tot;
+}
+
+// out[v] = w[0] + ... + w[v - 1], out[n] the total; every block adds up the tiles before its own
+__global__ void __launch_bounds__(1024) k_weight_prefix(const uint32_t* w, int64_t n, const unsigned long long* part,
+                                                        uint64_t* out) {
+  __shared__ unsigned long long s_w[32], s_tot, s_before;
+  unsigned long long before = 0;
+  for (int64_t i = threadIdx.x; i < blockIdx.x; i += blockDim.x) before += part[i];
+  block_exclusive_scan<unsigned long long>(before, s_w, &s_tot);
+  if (threadIdx.x == 0) s_before = s_tot;
+  __syncthreads();
+  unsigned long long x[4], sum;
+  load_weights(w, n, x, &sum);
+  unsigned long long ex = s_before + block_exclusive_scan<unsigned long long>(sum, s_w, &s_tot);
+  const int64_t base = (int64_t)blockIdx.x * PREFIX_TILE + (int64_t)threadIdx.x * 4;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    if (base + t < n) out[base + t] = ex;
+    ex += x[t];
+    if (base + t == n - 1) out[n] = ex;
+  }
+}
+
 // ---- greedy ----
 
 // maximum over the block of x, in every thread
@@ -1059,6 +1102,16 @@ cudaError_t launch_count_nodes(const int32_t* nodes, const int32_t* samp, int64_
                                int64_t jhi, int32_t* cnt, cudaStream_t st, int num_sms) {
   if (e1 <= e0) return cudaSuccess;
   k_count_nodes<<<grid_stride_blocks(e1 - e0, num_sms), TPB, 0, st>>>(nodes, samp, e0, e1, jlo, jhi, cnt);
+  return cudaGetLastError();
+}
+
+size_t weight_tmp_words(int64_t n) { return (size_t)((n + PREFIX_TILE - 1) / PREFIX_TILE); }
+
+cudaError_t launch_weight_prefix(const uint32_t* w, int64_t n, uint64_t* out, unsigned long long* tmp,
+                                 cudaStream_t st) {
+  const unsigned tiles = (unsigned)((n + PREFIX_TILE - 1) / PREFIX_TILE);
+  k_weight_tiles<<<tiles, 1024, 0, st>>>(w, n, tmp);
+  k_weight_prefix<<<tiles, 1024, 0, st>>>(w, n, tmp, out);
   return cudaGetLastError();
 }
 

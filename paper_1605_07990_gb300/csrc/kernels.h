@@ -183,6 +183,10 @@ cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t st);
 // entries [e0, e1); with samp non-null only samples in [jlo, jhi) count
 cudaError_t launch_count_nodes(const int32_t* nodes, const int32_t* samp, int64_t e0, int64_t e1, int64_t jlo,
                                int64_t jhi, int32_t* cnt, cudaStream_t st, int num_sms);
+// WRIS: out[v] = w[0] + ... + w[v - 1] for v <= n (n >= 1); tmp: weight_tmp_words(n) 64-bit words
+size_t weight_tmp_words(int64_t n);
+cudaError_t launch_weight_prefix(const uint32_t* w, int64_t n, uint64_t* out, unsigned long long* tmp,
+                                 cudaStream_t st);
 
 struct GreedyJob {
   const int32_t* cnt0;          // n_pad counts over the sets [0, n_sets); padding 0
