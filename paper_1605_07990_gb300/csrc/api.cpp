@@ -115,7 +115,7 @@ struct ssa_graph {
   mutable int tuned_heavy = 0x7FFFFFFF;
   mutable int tuned_small_qcap = 0;  // queue of the small CTAs (0: min(n, 2^20))
   mutable int tuned_warp_global = 0;  // weighted-cascade IC: the global-bitmap warp tier takes every sample
-  mutable int tuned_lane_tier = 1;    // weighted-cascade IC: the lane tier runs first
+  mutable int tuned_lane_tier = 1;    // weighted-cascade IC: the lane tier (ssa_set_lane_tier)
   GraphView view() const {
     GraphView v;
     v.n = n;
@@ -299,7 +299,7 @@ struct Sampler {
   int lt_cumulative = 0;
   int wc_implicit = 0;
   int warp_global = 0;  // weighted-cascade IC: the global-bitmap warp tier takes every sample
-  int lane_tier = 0;    // weighted-cascade IC: the lane tier runs first
+  int lane_tier = 0;    // weighted-cascade IC: the lane tier runs first: 0 never, 1 where it pays, 2 always
   int64_t* lane_list = nullptr;
   int64_t lane_cap = 0;
   uint32_t* wg_bitmap = nullptr;
@@ -336,7 +336,7 @@ struct Sampler {
         heavy_groups = G->tuned_heavy;
       }
       warp_global = (G->tuned_warp_global && cfg.wg_blocks > 0) ? 1 : 0;
-      lane_tier = (G->tuned_lane_tier && cfg.lane_blocks > 0) ? 1 : 0;
+      lane_tier = cfg.lane_blocks > 0 ? G->tuned_lane_tier : 0;
     }
     X.num_sms = cfg.num_sms;
     edge_visits = node_visits = samples = hit_samples = 0;
@@ -453,7 +453,16 @@ struct Sampler {
     J.lt_cumulative = lt_cumulative;
     J.wc_implicit = wc_implicit;
     J.warp_global = warp_global;
-    J.lane_tier = (model == 0 && wc_implicit && lane_tier) ? 1 : 0;
+    // The lane tier pays where the warps' visited sets are in global memory and
+    // the batch is large: from 32,768 samples on (GB300, us off / on: 2^21 nodes
+    // 516 / 480, 2^23 696 / 636, 2^25 1164 / 1168; 262,144 samples 2133 / 1063,
+    // 2582 / 1304, 3726 / 2218; 8192 samples 335 / 401, 486 / 563, 887 / 967).
+    // Before warps with their hash in shared memory it only adds its own tail
+    // (2^14 to 2^20 nodes, 1024 to 262,144 samples: 70 / 156 to 447 / 526 us).
+    J.lane_tier = model == 0 && wc_implicit &&
+                          (lane_tier == 2 || (lane_tier == 1 && warp_global && count >= LANE_TIER_SAMPLES))
+                      ? 1
+                      : 0;
     J.lane_list = lane_list;
     J.wg_bitmap = wg_bitmap;
     J.wg_queue = wg_queue;
@@ -1680,7 +1689,7 @@ ssa_status ssa_set_warp_tier(const ssa_graph* g, int32_t global_bitmap) {
 ssa_status ssa_set_lane_tier(const ssa_graph* g, int32_t on) {
   if (!g) return fail(SSA_E_ARG, "null graph");
   std::lock_guard<std::mutex> lock(g->tune_mu);
-  g->tuned_lane_tier = on != 0 ? 1 : 0;
+  g->tuned_lane_tier = on == 0 ? 0 : on == 1 ? 1 : 2;
   return SSA_OK;
 }
 

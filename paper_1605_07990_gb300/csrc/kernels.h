@@ -130,6 +130,9 @@ struct SampleJob {
   Counters* ctr = nullptr;
 };
 
+// Samples of a batch from which the lane tier runs before the global-bitmap warp tier.
+constexpr int64_t LANE_TIER_SAMPLES = 32768;
+
 struct LaunchCfg {
   int num_sms = 152;
   int warp_blocks = 0;   // grid of the warp tier

@@ -28,7 +28,7 @@ def test_star_in_lists_match_oracle(d):
     b = np.zeros(el.n, np.uint32)
     b[0] = 1
     N = 20_000
-    for lane in (1, 0):
+    for lane in (2, 0):
         P.ssa_set_lane_tier(gg, lane)
         for seed, stream in ((9, 0), ((1 << 40) + 5, 255)):
             op = oracle.Pool(og, oracle.IC, seed, stream, b).grow(N)
@@ -39,3 +39,25 @@ def test_star_in_lists_match_oracle(d):
             gp.free()
     P.ssa_set_lane_tier(gg, 1)
     gg.free()
+
+
+@pytest.mark.parametrize("scale,wg", [(13, 0), (21, 0), (21, 1)])
+def test_lane_tier_every_batch(scale, wg):
+    # the lane tier before each warp tier (2: on every batch), sets of 1 to hundreds of nodes
+    g = P.ssa_gen_rmat(scale, 8 << scale, seed=3)
+    P.ssa_set_tuning(g, 0)
+    P.ssa_set_warp_tier(g, wg)
+    got = []
+    for lane in (0, 1, 2):
+        P.ssa_set_lane_tier(g, lane)
+        p = P.Pool(g, P.SSA_IC, 5, 3).grow(40_000)
+        sizes = p.set_sizes()
+        S = p.max_coverage(40_000, 20)
+        est = P.ssa_estimate_inf(g, P.SSA_IC, 5, 9, S[0], 900.5, 50_000)
+        got.append((p.counts(40_000), sizes, S[0], S[1], est))
+        p.free()
+    assert got[0][1].max() > 64
+    for other in got[1:]:
+        for x, y in zip(got[0], other):
+            assert np.array_equal(x, y)
+    g.free()
