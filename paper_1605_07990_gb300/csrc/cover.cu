@@ -351,12 +351,14 @@ __device__ __forceinline__ void for_live_members(const GreedyJob& J, int64_t war
 //
 // Bound: the chain of a pick (two L2 round trips of ~600 clocks, two block
 // barriers, the argmax over shared memory), 1.5 us while a pick covers tens of
-// sets; picks that cover thousands are bound by the shared-memory atomics of
-// one SM.  Measured on GB300 against the former design (an inverted index of
-// all entries, a grid barrier of ~6 us per pick): 1000 picks over 134,016 sets
-// of the 2^23-node R-MAT graph 8.7 -> 2.3 ms, 500 over 131,832 LT sets there
-// 6.0 -> 2.1 ms, 100 over 1,149,440 sets of the 2^25-node one 3.5 -> 2.0 ms,
-// each with its index (0.2, 0.3 and 1.6 ms) gone.
+// sets; picks that cover thousands are bound by the issue slots of one SM (a
+// member is three instructions: chunks hold byte offsets of keys).  Measured on
+// GB300 against the former design (an inverted index of all entries, a grid
+// barrier of ~6 us per pick): 1000 picks over 134,016 sets of the 2^23-node
+// R-MAT graph 8.7 -> 2.3 ms, 500 over 131,832 LT sets there 6.0 -> 2.1 ms, 100
+// over 1,149,440 sets of the 2^25-node one 3.5 -> 2.0 ms, each with its index
+// (0.2, 0.3 and 1.6 ms) gone.  Byte offsets and fewer candidates where few picks
+// are left: all rounds of the second 5.6 -> 5.1 ms, of the first 7.7 -> 7.3 ms.
 //
 // With many picks to go and gains of some hundreds at most, the candidates and
 // all their lists fit shared memory (`small`: SCANDS candidates, SENTS entries):
@@ -525,7 +527,10 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
     const bool small = session && !first && !small_off && J.k - i >= 64 && key_gain(best) <= SENTS / 64;
     const int i0 = i;
     if (session) {
-      cap_n = small ? SCANDS : GCANDS;
+      // exact counts: some dozens of candidates a pick serve, and the fewer there
+      // are, the cheaper an argmax (the counts before a bulk pick need them all)
+      const long long few = max(2048ll, 32ll * (J.k - i));
+      cap_n = small ? SCANDS : first && bulk ? GCANDS : min((long long)GCANDS, few);
       cap_e = small ? SENTS : (long long)J.ents_cap;
       long long have = 0, sum = 0, total = 0;
       int b = cut(hist, [](int x) { return bin_gain(x + 1) - 1; }, have, sum, &total);
@@ -630,9 +635,10 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
       if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
       // ---- candidate lists of the sets left ----
       // a member's local id (1 + id, 0: no candidate) goes to its place `r` in
-      // the set's chunks at cs, and the chunks to the candidate's list
+      // the set's chunks at cs, as the byte offset of its key in shared memory, and
+      // the chunks to the candidate's list
       auto put = [&](unsigned int l, unsigned int cs, unsigned int off, int pos, int r) {
-        reinterpret_cast<uint16_t*>(J.chunks + cs)[4 + r] = (uint16_t)(l - 1u);
+        reinterpret_cast<uint16_t*>(J.chunks + cs)[4 + r] = (uint16_t)((l - 1u) * 4u);
         J.ents[off + (unsigned int)pos] = cs;
       };
       unsigned int cs = 0;  // this lane's set: its first chunk
@@ -807,20 +813,18 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
             if (tid == 0) {
               J.seeds[i] = (int32_t)s_id[l];
               J.gains[i] = g;
-              s_key[l] = 0u;  // never again; the loop below leaves it alone
             }
             const int off = s_off16[l], len = s_len16[l];
             for (int x = tid; x < len; x += STHREADS) {
               const int m = s_ent16[off + x];
               const int c = s_mem[m];
               if (c) s_mem[m] = 0;
-              for (int y = 1; y <= c; ++y) {
-                const int w = s_mem[m + y];
-                if (w != l) atomicSub(s_key + w, 1u << GBITS);
-              }
+              for (int y = 1; y <= c; ++y)
+                atomicSub(reinterpret_cast<unsigned int*>(s_dyn + s_mem[m + y]), 1u << GBITS);
             }
             i += 1;
             sync();
+            if (tid == (l & (STHREADS - 1))) s_key[l] = 0u;  // never again
           }
         }
         __syncthreads();
@@ -868,12 +872,13 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
           if (tid == 0) {
             J.seeds[i] = (int32_t)v;
             J.gains[i] = g;
-            s_key[l] = 0u;  // never again; the loop below leaves it alone
           }
-          auto lower = [&](unsigned int pair, int slot, int cnt) {  // slots `slot` and `slot` + 1 of a list of cnt
-            const int x = (int)(pair & 0xFFFFu), y = (int)(pair >> 16);
-            if (slot < cnt && x != l) atomicSub(s_key + x, 1u << GBITS);
-            if (slot + 1 < cnt && y != l) atomicSub(s_key + y, 1u << GBITS);
+          // Slots `slot` and `slot` + 1 of a list of cnt.  Picks that cover thousands
+          // of sets are bound by this SM's issue slots: three instructions a member
+          // (the pick's own key goes down to gain 0 with the others).
+          auto lower = [&](unsigned int pair, int slot, int cnt) {
+            if (slot < cnt) atomicSub(reinterpret_cast<unsigned int*>(s_dyn + (pair & 0xFFFFu)), 1u << GBITS);
+            if (slot + 1 < cnt) atomicSub(reinterpret_cast<unsigned int*>(s_dyn + (pair >> 16)), 1u << GBITS);
           };
           for (int base = (tid & ~31) >> sh; base < len; base += 1024 >> sh) {
             const unsigned int c0 = cs;
@@ -920,6 +925,8 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
           }
           i += 1;
           __syncthreads();
+          // never again: its owner, the only thread that reads it, takes it out
+          if (tid == (l & 1023)) s_key[l] = 0u;
         }
       }
       // the local ids go back to 0 for the next session
