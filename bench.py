@@ -1,7 +1,7 @@
 """Benchmark: RR sets/s of whole SSA / D-SSA solves on a resident synthetic R-MAT graph.
 
 One step = one complete solve on the GPU: RR sampling of every doubling round,
-the node->set index, greedy Max-Coverage, the stare check and the host FP64
+the node counts, greedy Max-Coverage, the stare check and the host FP64
 stopping rule.  Default workload (the billion-edge configuration): plain SSA
 (Algorithm 1), IC with weighted-cascade weights w = 1/d_in, directed R-MAT on
 2^25 nodes from 1.3e9 draws (a,b,c,d = 0.57,0.19,0.19,0.05; duplicates and
@@ -66,7 +66,7 @@ PHILOX_MIN_INSTR = 40
 # (dram__bytes_read.sum + dram__bytes_write.sum), keyed by workload and kernel
 # class, valid only for the kernel sources they were taken on (hash of
 # csrc/sample.cu, csrc/device.cuh, csrc/kernels.h); any other build reports
-# traffic null.
+# traffic null.  Empty: no capture of the present sampler.
 TRAFFIC = {}
 
 
@@ -178,7 +178,9 @@ def roofline(kind, dom, ks, results, sm_count, clock_mhz, name, hbm_peak, hbm_ki
     16 per visited node (two CSR offsets), 8 per live edge taken (its record;
     one per visited node but the root), 8 per stored pool entry (node,
     sample), 12 per stored set (start, length), 1 per hit-tested set.  No
-    per-edge bytes: the gaps need only the in-degree.
+    per-edge bytes: the gaps need only the in-degree.  (The graph store reads 8
+    and 4 bytes where this model counts 16 and 8; the model stays, so that
+    figures compare over time.)
     Edge records (trivalency, explicit): bound "alu" in Philox draws/s against
     PHILOX_MIN_INSTR, with 8 per examined in-edge in the HBM side figure."""
     if dom not in ("sample_cta", "sample_warp") or kind == "lt" or ks[dom]["ms"] <= 0:
