@@ -366,6 +366,12 @@ __device__ __forceinline__ void for_live_members(const GreedyJob& J, int64_t war
 // from 1.81 to 1.28 ms a round with it (a session of 1.5 us picks ends after 64
 // of them where 192 are left; one that served fewer than 96 is not tried again).
 //
+// Where the lists of a session do not fit (2^25 chunks are room for every member
+// of 17M small sets), the next ones are `tight`: the members are looked at twice
+// and only sets that hold a candidate get room.  SSA over 33.7M sets (809M
+// entries) of the 2^23-node graph, k = 1000: 244 ms, 3,661 with the best node's
+// sets covered by a pass over the pool instead; room for 2^27 chunks: 268 ms.
+//
 // Gains of 0 go by smallest id.  Barrier waits are bounded (sync[SYNC_ERR] on
 // timeout); a session makes at most GCANDS picks, milliseconds, between two
 // barriers.
@@ -386,7 +392,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
   const int64_t warp = gtid >> 5, nwarps = gthreads >> 5;
   const int64_t n4 = J.n_pad >> 2;
   int n_argmax = 0, n_hist = 0, i = 0;
-  bool first = true, bulk = J.bulk_first != 0, flat = false, small_off = false;
+  bool first = true, bulk = J.bulk_first != 0, flat = false, small_off = false, tight = false;
   if (tid == 0) s_phase = 0u;  // the host zeroed the release word (sense 0)
   unsigned long long info = 0;
 
@@ -532,6 +538,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
       const long long few = max(2048ll, 32ll * (J.k - i));
       cap_n = small ? SCANDS : first && bulk ? GCANDS : min((long long)GCANDS, few);
       cap_e = small ? SENTS : (long long)J.ents_cap;
+      if (tight) cap_e = min(cap_e, (long long)(J.chunk_cap / 3));  // a set takes 2.5 chunks a candidate at most
       long long have = 0, sum = 0, total = 0;
       int b = cut(hist, [](int x) { return bin_gain(x + 1) - 1; }, have, sum, &total);
       b = max(b, 1);
@@ -646,9 +653,24 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
       bool over = false;
       for_live_members(
           J, warp, nwarps, lane,
-          [&](int64_t j, int64_t, int& len) {
+          [&](int64_t j, int64_t start, int& len) {
             // room for every member: chunks are cheap (2 bytes a member) and a counting pass is not
-            const int nch = len ? ((len + 19) >> 4) * 2 : 0;
+            int room = len;
+            if (tight) {  // that did not fit: room for the candidates only
+              room = 0;
+              if (len <= 32)
+                for (int x = 0; x < len; ++x) room += J.lid[__ldg(J.pool_nodes + start + x)] != 0;
+              for (unsigned int m = __ballot_sync(FULL_MASK, len > 32); m; m &= m - 1u) {
+                const int o = __ffs(m) - 1, end = __shfl_sync(FULL_MASK, len, o);
+                const int64_t at = __shfl_sync(FULL_MASK, start, o);
+                int c = 0;
+                for (int x = lane; x < end; x += 32) c += J.lid[__ldg(J.pool_nodes + at + x)] != 0;
+                c = __reduce_add_sync(FULL_MASK, c);
+                if (lane == o) room = c;
+              }
+              if (room == 0) len = 0;
+            }
+            const int nch = room ? ((room + 19) >> 4) * 2 : 0;
             const int incl = warp_inclusive_scan(nch, lane);
             unsigned long long at = 0;
             if (lane == 31) at = atomicAdd(J.nchunk, (unsigned long long)incl);
@@ -656,8 +678,9 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
             over = at + (unsigned long long)__shfl_sync(FULL_MASK, incl, 31) > J.chunk_cap;
             cs = (unsigned int)(at + (unsigned long long)(incl - nch));
             run = 0;
-            // a long set would keep its warp long after the others: its parts go to the queue
-            if (len > GLONG && !over) {
+            // a long set would keep its warp long after the others: its parts go to the
+            // queue (which has a place for every 16 chunks: not where room is tight)
+            if (len > GLONG && !over && !tight) {
               const unsigned int parts = (unsigned int)((len + GLONG - 1) / GLONG);
               const unsigned int t0 = atomicAdd(J.ncand + 3, parts);
               *reinterpret_cast<uint2*>(J.chunks + cs) = make_uint2(0u, (unsigned int)j);
@@ -742,6 +765,8 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
         info >>= 32;
       }
     }
+    // lists that did not fit: tight ones next, and if it is not that, the best node's sets first
+    const bool retry = session && info != 0ull && !tight;
     bool overflow = session && info != 0ull;
     // ---- the session's picks ----
     if (session) {
@@ -959,7 +984,8 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
         },
         [](int64_t, int) {});
     if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
-    bulk = overflow;  // lists that did not fit: cover the best node's sets first
+    bulk = overflow && !retry;
+    tight = tight || retry;
     first = false;
   }
   // every gain is 0: the smallest ids not picked yet
