@@ -937,7 +937,7 @@ ssa_status stare_issue(Sampler& S, Cover& C, uint64_t seed, uint32_t stream, int
                        const int32_t* d_seeds, int k, Exec& X) {
   const int64_t words = (S.g.n + 31) / 32;
   CU(cudaMemsetAsync(S.seed_bits, 0, sizeof(uint32_t) * (size_t)words, X.st));
-  CU(launch_set_bits(d_seeds, k, S.seed_bits, nullptr, X.st));
+  CU(launch_set_bits(d_seeds, k, S.g.n, S.seed_bits, nullptr, X.st));
   X.launches += 1;
   TRY(S.hits_issue(seed, stream, j0, count, X));
   int h = X.begin(SSA_K_STARE);
@@ -968,7 +968,7 @@ ssa_status estimate_inf_dev(Sampler& S, Cover& C, uint64_t seed, uint32_t stream
                             Exec& X) {
   const int64_t words = (S.g.n + 31) / 32;
   CU(cudaMemsetAsync(S.seed_bits, 0, sizeof(uint32_t) * (size_t)words, X.st));
-  CU(launch_set_bits(d_seeds, k, S.seed_bits, nullptr, X.st));
+  CU(launch_set_bits(d_seeds, k, S.g.n, S.seed_bits, nullptr, X.st));
   X.launches += 1;
   int64_t j = 0, before = 0, B = std::max<int64_t>(first_batch, 4096);
   *T_out = 0;
@@ -1253,6 +1253,7 @@ ssa_status solve_impl(ssa_solver* sv, const ssa_params* p, ssa_result* out) {
         TRY(C.greedy_issue(pool, N, k, X));
         return c ? stare_issue(S, C, p->seed, 0, N, N, C.d_seeds, k, X) : SSA_OK;
       }));
+      TRY(C.greedy_finish(k, seeds.data(), gains.data(), cov));
     } else {
       TRY(C.count_issue(pool, N, X));
       {
@@ -1260,12 +1261,12 @@ ssa_status solve_impl(ssa_solver* sv, const ssa_params* p, ssa_result* out) {
         TRY(C.greedy_issue(pool, N, k, X));
         CU(cudaStreamSynchronize(X.st));
       }
+      TRY(C.greedy_finish(k, seeds.data(), gains.data(), cov));  // no stare on seeds of a greedy that gave up
       if (c) {
         TRY(stare_issue(S, C, p->seed, 0, N, N, C.d_seeds, k, X));
         CU(cudaStreamSynchronize(X.st));
       }
     }
-    TRY(C.greedy_finish(k, seeds.data(), gains.data(), cov));
     return c ? stare_finish(S, C, N, c) : SSA_OK;
   };
   do {
@@ -1895,7 +1896,7 @@ ssa_status ssa_coverage(ssa_pool* p, int64_t first, int64_t count, const int32_t
   TRY(dev_alloc(&d, (size_t)std::max(k, 1), p->X.st));
   if (k > 0) CU(cudaMemcpyAsync(d, seeds, sizeof(int32_t) * (size_t)k, cudaMemcpyHostToDevice, p->X.st));
   CU(cudaMemsetAsync(p->C.in_seed, 0, (size_t)p->C.n_pad, p->X.st));
-  if (k > 0) CU(launch_set_bits(d, k, nullptr, p->C.in_seed, p->X.st));
+  if (k > 0) CU(launch_set_bits(d, k, p->C.n, nullptr, p->C.in_seed, p->X.st));
   ssa_status st = p->C.coverage_range(p->P, first, first + count, cov, p->X);
   dev_free(d, p->X.st);
   cudaStreamSynchronize(p->X.st);

@@ -1099,9 +1099,12 @@ __global__ void __launch_bounds__(1024) k_find_first(const uint8_t* f, int64_t c
   }
 }
 
-__global__ void k_set_bits(const int32_t* ids, int k, uint32_t* bits, uint8_t* bytes) {
+// ids outside [0, n) set nothing: a Max-Coverage that gave up at a barrier leaves
+// seeds unwritten, and a stare queued behind it reads them before the host knows
+__global__ void k_set_bits(const int32_t* ids, int k, int64_t n, uint32_t* bits, uint8_t* bytes) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < k; i += gridDim.x * blockDim.x) {
     const int32_t v = ids[i];
+    if (v < 0 || v >= n) continue;
     if (bits) atomicOr(bits + (v >> 5), 1u << (v & 31));
     if (bytes) bytes[v] = 1;
   }
@@ -1265,9 +1268,9 @@ cudaError_t launch_first_reach(const uint8_t* flags, int64_t count, long long ne
   return cudaGetLastError();
 }
 
-cudaError_t launch_set_bits(const int32_t* ids, int k, uint32_t* bits, uint8_t* bytes, cudaStream_t st) {
+cudaError_t launch_set_bits(const int32_t* ids, int k, int64_t n, uint32_t* bits, uint8_t* bytes, cudaStream_t st) {
   if (k <= 0) return cudaSuccess;
-  k_set_bits<<<(k + TPB - 1) / TPB, TPB, 0, st>>>(ids, k, bits, bytes);
+  k_set_bits<<<(k + TPB - 1) / TPB, TPB, 0, st>>>(ids, k, n, bits, bytes);
   return cudaGetLastError();
 }
 

@@ -264,7 +264,8 @@ cudaError_t launch_first_reach(const uint8_t* flags, int64_t count, long long ne
                                long long* out, void* tmp, cudaStream_t st, int* launches);
 size_t first_reach_tmp_bytes(int64_t count);
 
-cudaError_t launch_set_bits(const int32_t* ids, int k, uint32_t* bits, uint8_t* bytes, cudaStream_t st);
+// bit / byte of every id in [0, n); others are skipped
+cudaError_t launch_set_bits(const int32_t* ids, int k, int64_t n, uint32_t* bits, uint8_t* bytes, cudaStream_t st);
 cudaError_t launch_gather_sets(const int32_t* pool_nodes, const int64_t* set_start, const int32_t* set_len,
                                const int64_t* out_off, int64_t first, int64_t count, int32_t* out,
                                cudaStream_t st);
