@@ -171,6 +171,7 @@ template <class Visit>
 __device__ __forceinline__ bool drain(const Stage& st, bool all, int lane, Visit&& visit) {
   __syncwarp();
   int n = (int)*(volatile unsigned int*)st.cnt;
+  __syncwarp();  // every lane has read the count before a lane's next push raises it
   if (n < 32 && !(all && n > 0)) return false;
   const unsigned lt_mask = (1u << lane) - 1u;
   bool stop = false;
