@@ -552,12 +552,16 @@ struct Sampler {
     const double margin = P.count >= 65536 ? 1.15 : 1.5;
     int64_t want = P.entries + (int64_t)(mean * (double)count * margin) + 65536;
     // nothing is known about the first batch: room for large sets (the huge ones
-    // that coins can give: up to 256 MB of entries) spares their second sampling.
+    // that coins can give: up to 256 MB of entries) spares their second sampling,
+    // within a quarter of the pool's cap: the batches to come need the rest.
     // On GB300, sampling of a solve: SSA 2^25 nodes 13.5 -> 12.7 ms, D-SSA LT 2^23
     // 3.85 -> 3.47 ms, trivalency 2^20 (sets of 137,000 nodes) 204 -> 198 ms.
-    if (P.count == 0)
-      want = std::max(want, std::min<int64_t>(count * g.n, int64_t(1) << (model == 0 && !wc_implicit ? 25 : 21)));
-    TRY(grow_entries(P, want, X));
+    if (P.count == 0) {
+      int64_t room = std::min<int64_t>(count * g.n, int64_t(1) << (model == 0 && !wc_implicit ? 25 : 21));
+      if (P.byte_cap > 0) room = std::min(room, P.byte_cap / (4 * 12));
+      want = std::max(want, room);
+    }
+    TRY(grow_entries(P, P.entries + count, want, X));  // a set has its root at least
     int64_t todo = count;
     const int64_t* list = nullptr;
     unsigned long long cursor0 = (unsigned long long)P.entries;
@@ -589,7 +593,7 @@ struct Sampler {
       const int64_t need = (int64_t)h_ctr->cursor - ok_end;
       const int64_t failed = (int64_t)h_ctr->fail_count;
       P.entries = ok_end;
-      TRY(grow_entries(P, ok_end + need + need / 4 + 65536, X));
+      TRY(grow_entries(P, ok_end + need, ok_end + need + need / 4 + 65536, X));
       std::swap(fail_list, redo_list);
       std::swap(fail_cap, redo_cap);
       list = redo_list;
@@ -610,13 +614,17 @@ struct Sampler {
     return SSA_OK;
   }
 
-  ssa_status grow_entries(DevPool& P, int64_t want, Exec& X) {
+  // Room for `want` entries, an estimate, of which `need` are certain.  Only the
+  // need can pass the cap: an estimate that the cap does not allow gets what the
+  // cap leaves, or nothing more, and sets that then miss the pool say what they need.
+  ssa_status grow_entries(DevPool& P, int64_t need, int64_t want, Exec& X) {
     if (want <= P.cap_entries) return SSA_OK;
     want = std::max<int64_t>(want, P.cap_entries + P.cap_entries / 2);
     if (P.byte_cap > 0 && P.bytes_for(want, P.cap_sets) > P.byte_cap) {
       const int64_t most = (P.byte_cap - P.cap_sets * 14) / 12;
-      if (most <= P.cap_entries)
+      if (need > std::max(most, P.cap_entries))
         return fail(SSA_E_POOL_FULL, "RR pool needs more than its %lld-byte cap", (long long)P.byte_cap);
+      if (most <= P.cap_entries) return SSA_OK;
       want = most;
     }
     int64_t a = P.cap_entries, b = P.cap_entries;
