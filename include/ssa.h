@@ -192,9 +192,12 @@ ssa_status ssa_set_lane_tier(const ssa_graph* g, int32_t on);
 ssa_status ssa_set_greedy_mode(int32_t mode);
 
 /* Process-wide bound on the polls of each device-side wait: the grid barriers
- * of the greedy kernel (ssa_max_coverage and every solve).  A wait that reaches
- * it gives up, its kernel returns, and the call reports SSA_E_TIMEOUT.  polls
- * >= 1 sets the bound (each poll backs off up to 128 ns); 0 restores the
+ * of the greedy kernel (ssa_max_coverage and every solve).  A wait that makes
+ * this many polls without seeing progress gives up, its kernel returns, and the
+ * call reports SSA_E_TIMEOUT.  (One block makes up to thousands of picks in a
+ * row while the others wait; every pick, and every few hundred sets of a large
+ * one, counts as progress, so a bound has to span such a step or a pass over the
+ * pool, not the whole call.)  polls >= 1 sets the bound (each poll backs off up to 128 ns); 0 restores the
  * default of 2^22 polls, about a second.  Meant for failure handling and its
  * tests: a small bound makes ordinary barriers give up.  Applies to launches
  * after the call; SSA_E_ARG for polls < 0. */
@@ -324,8 +327,8 @@ ssa_status ssa_pool_counts(ssa_pool* p, int64_t N, int32_t* cnt);
  * gain, ties to the smallest id, seeds never re-picked.  seeds int32[k],
  * gains int64[k] (host); *cov = Cov_R(S).  1 <= k <= n; N <= 2^31 - 2
  * (SSA_E_ARG beyond).  All k picks run in one kernel; a wait at its grid
- * barriers gives up after a bounded number of polls (about a second
- * by default, see ssa_set_wait_polls): every block then returns and the call
+ * barriers gives up after a bounded number of polls without progress (about a
+ * second by default, see ssa_set_wait_polls): every block then returns and the call
  * reports SSA_E_TIMEOUT, leaving the CUDA context usable. */
 ssa_status ssa_max_coverage(ssa_pool* p, int64_t N, int32_t k, int32_t* seeds, int64_t* gains,
                             int64_t* cov);

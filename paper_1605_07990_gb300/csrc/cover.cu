@@ -138,9 +138,9 @@ __device__ __forceinline__ unsigned long long block_max(unsigned long long x, un
   return x;
 }
 
-// sync layout: arrival count, release word and error flag on separate
-// 128-byte lines so that polling does not contend with the arrivals.
-constexpr int SYNC_COUNT = 0, SYNC_GEN = 32, SYNC_ERR = 64;
+// sync layout: arrival count, release word, error flag and block 0's progress on
+// separate 128-byte lines so that polling does not contend with the arrivals.
+constexpr int SYNC_COUNT = 0, SYNC_GEN = 32, SYNC_ERR = 64, SYNC_PROGRESS = 96;
 constexpr int ARGMAX_STRIDE = 16;  // 64-bit words: argmax slots one 128-byte line apart
 constexpr int GCANDS = GREEDY_CANDS;  // candidates of one session: their gains, ids and list offsets fill 192 KB
 constexpr int GBITS = 14;          // a candidate's key: gain above, GCANDS - 1 - local id in the low GBITS
@@ -157,21 +157,25 @@ constexpr int GLONG = 256;         // members of a set beyond which its list is 
 // publishes the result (< 2^63) in the release word beside a sense bit (bit 0,
 // flipped by each release), so every waiter learns it from the poll that
 // releases it; all threads get it in `info`.  A wait gives up after `limit`
-// polls (about a second by default), sets sync[SYNC_ERR] and returns false;
-// that block then leaves the kernel, and the others give up at their next
-// barrier, which it never reaches.  Every block passes every barrier in the
-// same order, so each keeps the current sense in its shared `phase` (0 at
-// launch, when the release word is zero) instead of reading it back.
+// polls (about a second by default) without progress, sets sync[SYNC_ERR] and
+// returns false; that block then leaves the kernel, and the others give up at
+// their next barrier, which it never reaches.  Progress is the word that block 0
+// moves while it makes a session's picks alone (every few picks, and every 128 or
+// 512 sets of one): a session may take thousands of picks, and the bound has to
+// span one step of them, not the session.  Every block passes every barrier in
+// the same order, so each keeps the current sense in its shared wait[0] (0 at
+// launch, when the release word is zero) instead of reading it back, and in
+// wait[1] the progress it saw last.
 template <class F>
-__device__ __forceinline__ bool grid_barrier(unsigned int* sync, unsigned int* phase, long long limit, F&& f,
+__device__ __forceinline__ bool grid_barrier(unsigned int* sync, unsigned int* wait, long long limit, F&& f,
                                              unsigned long long& info) {
   __shared__ unsigned long long s_info;
   __shared__ unsigned int s_last, s_ok, s_sense;
   volatile unsigned long long* gw = reinterpret_cast<volatile unsigned long long*>(sync + SYNC_GEN);
   __syncthreads();
   if (threadIdx.x == 0) {
-    s_sense = *phase;
-    *phase = s_sense ^ 1u;
+    s_sense = wait[0];
+    wait[0] = s_sense ^ 1u;
     s_ok = 1;
     __threadfence();
     const bool last = atomicAdd(sync + SYNC_COUNT, 1u) + 1u == gridDim.x;
@@ -192,10 +196,15 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* sync, unsigned int* p
     unsigned long long w;
     unsigned int ns = 8;
     for (long long spins = 0; (unsigned int)((w = *gw) & 1ull) == s_sense; ++spins) {
-      if (spins > limit) {  // by default seconds: a barrier never takes that long
-        atomicExch(sync + SYNC_ERR, 1u);
-        s_ok = 0;
-        break;
+      if (spins > limit) {
+        const unsigned int p = *(volatile unsigned int*)(sync + SYNC_PROGRESS);
+        if (p == wait[1]) {
+          atomicExch(sync + SYNC_ERR, 1u);
+          s_ok = 0;
+          break;
+        }
+        wait[1] = p;
+        spins = 0;
       }
       __nanosleep(ns);
       if (ns < 128) ns <<= 1;
@@ -215,7 +224,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* sync, unsigned int* p
 // second cluster barrier.  A cluster barrier always completes (the cluster's
 // blocks are scheduled together), so it has no bound to reach.
 template <bool CLUSTER, class F>
-__device__ __forceinline__ bool greedy_barrier(const GreedyJob& J, unsigned int* phase, F&& f,
+__device__ __forceinline__ bool greedy_barrier(const GreedyJob& J, unsigned int* wait, F&& f,
                                                unsigned long long& info) {
   if constexpr (!CLUSTER) {
     if (gridDim.x == 1) {  // a single block needs no waits
@@ -224,7 +233,7 @@ __device__ __forceinline__ bool greedy_barrier(const GreedyJob& J, unsigned int*
       __syncthreads();
       return true;
     }
-    return grid_barrier(J.sync, phase, J.wait_polls, f, info);
+    return grid_barrier(J.sync, wait, J.wait_polls, f, info);
   } else {
     namespace cg = cooperative_groups;
     __shared__ unsigned long long s_res;
@@ -373,14 +382,15 @@ __device__ __forceinline__ void for_live_members(const GreedyJob& J, int64_t war
 // sets covered by a pass over the pool instead; room for 2^27 chunks: 268 ms.
 //
 // Gains of 0 go by smallest id.  Barrier waits are bounded (sync[SYNC_ERR] on
-// timeout); a session makes at most GCANDS picks, milliseconds, between two
-// barriers.
+// timeout).  Between two barriers block 0 may make up to GCANDS picks and lower
+// every member that the chunks hold (268M), hundreds of milliseconds; it shows
+// its progress, and the bound is on polls that see none.
 template <bool CLUSTER>
 __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ unsigned long long s_red[32];
   __shared__ long long s_scan[32], s_scan_tot;
-  __shared__ unsigned int s_phase;  // sense of the next grid barrier
+  __shared__ unsigned int s_wait[2];  // sense of the next grid barrier, block 0's progress at the last look
   __shared__ unsigned int s_w[2][32];
   unsigned int* s_key = reinterpret_cast<unsigned int*>(s_dyn);  // block 0 in a session: keys (gain, ~local id),
   unsigned int* s_id = s_key + GCANDS;                           // node ids
@@ -393,7 +403,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
   const int64_t n4 = J.n_pad >> 2;
   int n_argmax = 0, n_hist = 0, i = 0;
   bool first = true, bulk = J.bulk_first != 0, flat = false, small_off = false, tight = false;
-  if (tid == 0) s_phase = 0u;  // the host zeroed the release word (sense 0)
+  if (tid == 0) s_wait[0] = s_wait[1] = 0u;  // the host zeroed the release word (sense 0) and the progress
   unsigned long long info = 0;
 
   // One pass over the gains: histogram of bin(key) (-1: not counted) merged
@@ -446,7 +456,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
     best = block_max(best, s_red);
     unsigned long long* at = J.argmax + (n_argmax % 3) * ARGMAX_STRIDE;
     if (tid == 0 && best) atomicMax(at, best);
-    if (!greedy_barrier<CLUSTER>(J, &s_phase, [&] { return __ldcg(at); }, info)) return false;
+    if (!greedy_barrier<CLUSTER>(J, s_wait, [&] { return __ldcg(at); }, info)) return false;
     // clear the slot and the histogram of two scans on: nobody has touched
     // them since the barrier before this one
     if (blockIdx.x == 0) {
@@ -597,7 +607,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
       for (; q < n4; q += gthreads) select(q, c4[q]);
       __syncthreads();
       if (tid < (int)gridDim.x && s_blk[tid]) atomicAdd(J.blk + tid, s_blk[tid]);
-      if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
+      if (!greedy_barrier<CLUSTER>(J, s_wait, [] { return 0ull; }, info)) return;
       int nc;
       {
         const long long own_b = tid < (int)gridDim.x ? (long long)__ldcg(J.blk + tid) : 0ll;
@@ -623,7 +633,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
             J.mark[w] = 0u;
           }
       }
-      if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
+      if (!greedy_barrier<CLUSTER>(J, s_wait, [] { return 0ull; }, info)) return;
       // list space, as many entries as the count that chose the candidate
       for (int t0 = (int)blockIdx.x * 1024; t0 < nc; t0 += (int)gridDim.x * 1024) {
         const int t = t0 + tid;
@@ -639,7 +649,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
         __syncthreads();
       }
       if (blockIdx.x == 0 && tid == 0) J.ncand[0] = (unsigned int)nc;
-      if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
+      if (!greedy_barrier<CLUSTER>(J, s_wait, [] { return 0ull; }, info)) return;
       // ---- candidate lists of the sets left ----
       // a member's local id (1 + id, 0: no candidate) goes to its place `r` in
       // the set's chunks at cs, as the byte offset of its key in shared memory, and
@@ -729,7 +739,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
               *reinterpret_cast<uint2*>(J.chunks + cs) = make_uint2((unsigned int)run, (unsigned int)j);
             }
           });
-      if (!greedy_barrier<CLUSTER>(J, &s_phase, [&] {
+      if (!greedy_barrier<CLUSTER>(J, s_wait, [&] {
             return ((unsigned long long)__ldcg(J.ncand + 1) << 32) | (unsigned long long)__ldcg(J.ncand + 3);
           }, info)) return;
       const unsigned int ntasks = (unsigned int)info;
@@ -759,7 +769,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
           for (int u = 0; u < GLONG / 32; ++u)
             if (l[u]) put(l[u], t.x, J.cand_off[l[u] - 1u], atomicAdd(J.cand_len + (l[u] - 1u), 1), r++);
         }
-        if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
+        if (!greedy_barrier<CLUSTER>(J, s_wait, [] { return 0ull; }, info)) return;
         info = 0ull;
       } else {
         info >>= 32;
@@ -772,6 +782,10 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
     if (session) {
       const int nc = (int)__ldcg(J.ncand);
       overflow = overflow || nc == 0;
+      // thread 0, at every pick and at every further step of one
+      auto progress = [&](unsigned int step) {
+        if (!CLUSTER) __stcg(J.sync + SYNC_PROGRESS, (unsigned int)(i + 1) * 0x9E3779B1u + step);
+      };
       if (blockIdx.x == 0 && !overflow && small) {
         // everything into shared memory: the lists of the sets one after the
         // other (count, local ids; count 0: covered), the candidates' lists as
@@ -781,8 +795,8 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
         unsigned short* s_len16 = s_off16 + SCANDS;
         unsigned short* s_ent16 = s_len16 + SCANDS;
         unsigned short* s_mem = s_ent16 + SENTS;
-        __shared__ unsigned int s_nmem;
-        if (tid == 0) s_nmem = 0u;
+        __shared__ unsigned int s_nmem, s_over;
+        if (tid == 0) s_nmem = s_over = 0u;
         const int E = (int)__ldcg(J.ncand + 4);
         for (int t = tid; t < SCANDS; t += 1024) {
           const unsigned int len = t < nc ? (unsigned int)__ldcg(J.cand_len + t) : 0u;
@@ -851,6 +865,18 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
             sync();
             if (tid == (l & (STHREADS - 1))) s_key[l] = 0u;  // never again
           }
+          if (tid == 0) *(volatile unsigned int*)&s_over = 1u;
+        } else if (!CLUSTER && tid == STHREADS) {
+          // an idle warp shows the progress: every pick lowers the sum of the warps'
+          // best keys (a store by the picking warps cost 1% of 1000 picks)
+          for (int t = 0; t < (1 << 20) && *(volatile unsigned int*)&s_over == 0u; ++t) {
+            unsigned int sum = 0u;
+#pragma unroll
+            for (int w = 0; w < STHREADS / 32; ++w)
+              sum += *(volatile unsigned int*)&s_w[0][w] + *(volatile unsigned int*)&s_w[1][w];
+            __stcg(J.sync + SYNC_PROGRESS, sum);
+            __nanosleep(1000);
+          }
         }
         __syncthreads();
         // the covered flags of the sets whose count is 0 now
@@ -897,6 +923,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
           if (tid == 0) {
             J.seeds[i] = (int32_t)v;
             J.gains[i] = g;
+            progress(0u);
           }
           // Slots `slot` and `slot` + 1 of a list of cnt.  Picks that cover thousands
           // of sets are bound by this SM's issue slots: three instructions a member
@@ -906,6 +933,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
             if (slot + 1 < cnt) atomicSub(reinterpret_cast<unsigned int*>(s_dyn + (pair >> 16)), 1u << GBITS);
           };
           for (int base = (tid & ~31) >> sh; base < len; base += 1024 >> sh) {
+            if (base > 0 && tid == 0) progress((unsigned int)base);
             const unsigned int c0 = cs;
             if (base + (1024 >> sh) < len) cs = __ldcg(J.ents + off + base + (1024 >> sh) + (lane >> sh));
             uint4 a = make_uint4(0u, 0u, 0u, 0u);
@@ -959,14 +987,14 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
       if (b0 >= 0)
         for (int64_t t = b0 * 1024 + tid; t < nc; t += nb * 1024) J.lid[__ldcg(J.cand_id + t)] = 0;
       if (blockIdx.x == 0 && tid == 0) J.ncand[2] = (unsigned int)i;
-      if (!greedy_barrier<CLUSTER>(J, &s_phase, [&] { return (unsigned long long)__ldcg(J.ncand + 2); }, info)) return;
+      if (!greedy_barrier<CLUSTER>(J, s_wait, [&] { return (unsigned long long)__ldcg(J.ncand + 2); }, info)) return;
       i = (int)info;
       if (i >= J.k) break;
       if (small && i - i0 < 96) small_off = true;  // it did not pay for its lists
     }
     // ---- gains again over the sets left ----
     for (int64_t q = gtid; q < n4; q += gthreads) reinterpret_cast<int4*>(J.cnt)[q] = make_int4(0, 0, 0, 0);
-    if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
+    if (!greedy_barrier<CLUSTER>(J, s_wait, [] { return 0ull; }, info)) return;
     if (blockIdx.x == 0) {
       for (int t = tid; t < i; t += 1024) J.cnt[__ldcg(J.seeds + t)] = -1;  // in no set that is left
       if (tid < (int)gridDim.x) J.blk[tid] = 0u;
@@ -983,7 +1011,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
             if (node[t] >= 0) atomicAdd(J.cnt + node[t], 1);
         },
         [](int64_t, int) {});
-    if (!greedy_barrier<CLUSTER>(J, &s_phase, [] { return 0ull; }, info)) return;
+    if (!greedy_barrier<CLUSTER>(J, s_wait, [] { return 0ull; }, info)) return;
     bulk = overflow && !retry;
     tight = tight || retry;
     first = false;

@@ -207,7 +207,7 @@ struct GreedyJob {
   int32_t* gains;               // k (device)
   int k;
   // control block, zeroed: GREEDY_CTL_BYTES
-  unsigned int* sync;           // 128 words: count [0], release word (64-bit) [32], error flag [64]
+  unsigned int* sync;           // 128 words: count [0], release word (64-bit) [32], error flag [64], progress [96]
   unsigned long long* argmax;   // 3 slots 16 words apart
   unsigned long long* nchunk;   // chunks handed out
   unsigned int* ncand;          // candidates, chunk overflow, picks made, queued parts, list entries
@@ -224,7 +224,7 @@ struct GreedyJob {
   uint4* chunks;                // chunk_cap (+ GREEDY_CHUNKS_SPARE) chunks of the sets' candidates
   unsigned long long chunk_cap;
   uint4* tasks;                 // parts of long sets (first chunk, set, first member): chunk_cap / 16 + 1
-  long long wait_polls;         // polls after which a grid-barrier wait gives up
+  long long wait_polls;         // polls without progress after which a grid-barrier wait gives up
 };
 constexpr int GREEDY_CANDS = 16384;
 constexpr int GREEDY_ENTS_SPARE = 2048, GREEDY_CHUNKS_SPARE = 16;
