@@ -216,7 +216,9 @@ typedef struct {
   uint64_t seed;             /* Philox key */
   const uint32_t* benefit;   /* host uint32[n] WRIS benefits (Sec. 6.3.1), or NULL for
                                 uniform sources; copied during the call */
-  int64_t pool_bytes_cap;    /* RR-pool cap in bytes (0 = library default) */
+  int64_t pool_bytes_cap;    /* cap in bytes on the RR pool and Max-Coverage's candidate lists
+                                (0 = library default).  The pool asks 12 bytes an entry and 14 a
+                                set of it; the lists take what the pool leaves, at least 2 MB */
 } ssa_params;
 
 /* One stop-and-stare round. */
@@ -278,11 +280,12 @@ typedef struct {
  * SSA_E_NOMEM, SSA_E_POOL_FULL, SSA_E_CUDA, SSA_E_TIMEOUT. */
 ssa_status ssa_solve(const ssa_graph* g, const ssa_params* p, ssa_result* out);
 
-/* A solver keeps device workspaces (sampler scratch per model, index and
+/* A solver keeps device workspaces (sampler scratch per model, counts and
  * greedy buffers) and a CUDA stream across solves on one graph; each solve's
- * RR pool and index return to the device's memory pool when it ends.  stream: a cudaStream_t to run on, or NULL for a
- * library-created one.  pool_bytes_cap: cap for the RR pool (0 = 60% of the
- * device memory free at creation). */
+ * RR pool and Max-Coverage lists (beyond 32 MB of entries and 32 MB of chunks)
+ * return to the device's memory pool when it ends.  stream: a cudaStream_t to
+ * run on, or NULL for a library-created one.  pool_bytes_cap: cap for the RR
+ * pool and the lists (0 = 60% of the device memory free at creation). */
 ssa_status ssa_solver_create(const ssa_graph* g, void* stream, int64_t pool_bytes_cap, ssa_solver** out);
 ssa_status ssa_solver_solve(ssa_solver* s, const ssa_params* p, ssa_result* out);
 /* Run each round's device work after sampling -- the counts of the new sets,

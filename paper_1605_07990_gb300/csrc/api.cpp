@@ -62,6 +62,17 @@ void dev_free(T*& p, cudaStream_t st) {
   p = nullptr;
 }
 
+// Room for `want` elements where nothing is kept: the old array goes first.
+template <typename T>
+ssa_status dev_renew(T** p, int64_t* cap, int64_t want, cudaStream_t st) {
+  if (want <= *cap) return SSA_OK;
+  dev_free(*p, st);
+  *cap = 0;
+  TRY(dev_alloc(p, (size_t)want, st));
+  *cap = want;
+  return SSA_OK;
+}
+
 // Grow a device array to `want` elements keeping the first `keep`.
 template <typename T>
 ssa_status dev_grow(T** p, int64_t* cap, int64_t want, int64_t keep, cudaStream_t st) {
@@ -238,9 +249,11 @@ struct DevPool {
   int32_t* set_len = nullptr;
   int64_t count = 0, entries = 0;
   std::vector<std::pair<int64_t, int64_t>> bounds{{0, 0}};
-  int64_t byte_cap = 0;
+  int64_t byte_cap = 0;  // on the pool and the greedy's lists (0: none)
 
+  // what the cap asks of a pool: its 8 bytes an entry and 12 a set, and room for lists
   int64_t bytes_for(int64_t ents, int64_t sets) const { return ents * 12 + sets * 14; }
+  int64_t bytes_held() const { return cap_entries * 8 + cap_sets * 12; }
   // entries range covering samples [a, b); *whole: it holds no other samples
   void entry_range(int64_t a, int64_t b, int64_t* e0, int64_t* e1, bool* whole) const {
     *e0 = 0;
@@ -827,14 +840,22 @@ struct Cover {
     // Candidate lists: entries for every member while that is little, else for
     // the most frequent nodes (a candidate has at most N); 16-byte chunks for
     // every member of the sets left after the first pick, at most 512 MB (more
-    // than fits makes the kernel cover the best node's sets first).
+    // than fits makes the kernel list fewer candidates' sets, or cover the best
+    // node's sets first), and a 16-byte record per 16 chunks behind them (of 256
+    // members of a long set, which has more, so at least 16 chunks a record).
+    // Where the pool has a cap, both keep to what the pool leaves of it.
     ents_now = std::min<int64_t>(std::min<int64_t>(total_e, std::max<int64_t>(2 * N, int64_t(1) << 25)),
                                  INT32_MAX - 4096);
-    TRY(dev_grow(&ents, &ents_cap, ents_now + GREEDY_ENTS_SPARE, 0, X.st));
     chunks_now = std::min<int64_t>((total_e + 19 * N) / 8 + 1, int64_t(1) << 25);
-    // behind the chunks: a 16-byte record per 256 members of a long set (more
-    // than 256 members, so at least 16 chunks a record)
-    TRY(dev_grow(&chunks, &chunk_cap, chunks_now + GREEDY_CHUNKS_SPARE + chunks_now / 16 + 1, 0, X.st));
+    if (P.byte_cap > 0) {
+      const int64_t left = P.byte_cap - P.bytes_held();
+      if (ents_now * 4 + chunks_now * 17 > left) {
+        ents_now = std::min(ents_now, std::max<int64_t>(LISTS_ANY_ENTS, left / 16));
+        chunks_now = std::min(chunks_now, std::max<int64_t>(LISTS_ANY_CHUNKS, (left - ents_now * 4) / 17));
+      }
+    }
+    TRY(dev_renew(&ents, &ents_cap, ents_now + GREEDY_ENTS_SPARE, X.st));
+    TRY(dev_renew(&chunks, &chunk_cap, chunks_now + GREEDY_CHUNKS_SPARE + chunks_now / 16 + 1, X.st));
     if (lid_dirty) {
       CU(cudaMemsetAsync(lid, 0, sizeof(uint16_t) * lid_words(), X.st));
       lid_dirty = false;
@@ -842,6 +863,22 @@ struct Cover {
     return SSA_OK;
   }
   int64_t ents_now = 0, chunks_now = 0;  // what the next greedy may use of them
+  // 1 MB of list entries and 1 MB of chunks whatever the cap; a solver keeps up to
+  // 32 MB of each between solves and gives larger ones back to the device's memory
+  // pool (small solves, a few ms, then allocate nothing)
+  static constexpr int64_t LISTS_ANY_ENTS = int64_t(1) << 18, LISTS_ANY_CHUNKS = int64_t(1) << 16;
+  static constexpr int64_t LISTS_KEEP_BYTES = int64_t(32) << 20;
+  int64_t list_bytes() const { return ents_cap * 4 + chunk_cap * 16; }
+  void release_lists(cudaStream_t st) {
+    if (ents_cap * 4 > LISTS_KEEP_BYTES) {
+      dev_free(ents, st);
+      ents_cap = 0;
+    }
+    if (chunk_cap * 16 > LISTS_KEEP_BYTES) {
+      dev_free(chunks, st);
+      chunk_cap = 0;
+    }
+  }
   ssa_status greedy_issue(const DevPool& P, int64_t N, int k, Exec& X) {
     int h = X.begin(SSA_K_GREEDY);
     CU(cudaMemsetAsync(covered, 0, (size_t)std::max<int64_t>(N, 1), X.st));
@@ -1147,6 +1184,7 @@ struct ssa_solver {
   bool shared_gpu = false;  // concurrent solves share the GPU (serving): cluster-shaped greedy
   std::vector<cudaGraphExec_t> gexec;
   int64_t graph_launches = 0;
+  int64_t last_bytes = 0;  // RR pool and greedy lists that the last solve held at its end
 
   void release() {
     for (auto e : gexec)
@@ -1414,14 +1452,19 @@ ssa_status solve_impl(ssa_solver* sv, const ssa_params* p, ssa_result* out) {
   } else {
     X.collect(nullptr);
   }
-  // the RR pool goes back to the device's memory pool; the scratch stays with the solver
+  // the RR pool and large candidate lists go back to the device's memory pool; the
+  // scratch stays with the solver
+  sv->last_bytes = pool.bytes_held() + (sv->c_ready ? C.list_bytes() : 0);
   pool.release(X.st);
+  if (sv->c_ready) C.release_lists(X.st);
   if (sv->s_ready[p->model]) dev_free(S.bprefix, X.st);
   cudaStreamSynchronize(X.st);
   out->seconds = now_s() - t0;
   return st;
 }
 }  // namespace
+
+int64_t ssa::solver_bytes(const ssa_solver* s) { return s ? s->last_bytes : 0; }
 
 // ---------------------------------------------------------------------------
 // C ABI

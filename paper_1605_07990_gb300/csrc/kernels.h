@@ -4,7 +4,12 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+struct ssa_solver;
+
 namespace ssa {
+
+// Device bytes of the RR pool and the greedy lists at the end of the solver's last solve.
+int64_t solver_bytes(const ssa_solver* s);
 
 // Sets the calling thread's message returned by ssa_last_error().
 void set_last_error(const char* msg);

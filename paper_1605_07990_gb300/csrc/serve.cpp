@@ -152,7 +152,8 @@ struct ssa_server {
         if (s == SSA_OK) {
           completed += 1;
           latencies.push_back(r->t_done - r->t_submit);
-          learn(*r, r->res.pool_entries * 16 + r->res.n_rr * 16);
+          learn(*r, std::max(r->res.pool_entries * 16 + r->res.n_rr * 16,
+                             ssa::solver_bytes(solvers[(size_t)r->graph])));
         } else {
           failed += 1;
         }
