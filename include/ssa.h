@@ -175,10 +175,11 @@ ssa_status ssa_set_queue_tuning(const ssa_graph* g, int32_t small_queue);
 ssa_status ssa_set_warp_tier(const ssa_graph* g, int32_t global_bitmap);
 /* Weighted-cascade IC: a lane tier before the warp tiers, one sample per lane
  * with its queue of up to 32 nodes in thread-local memory; larger sets are redone
- * by the warp tiers.  on = 1 (the default) runs it where it is faster: on batches
- * of 32,768 samples or more whose warp tier is the global-bitmap one
- * (ssa_set_warp_tier); 2 on every batch; 0 sends every sample to the warp tiers.
- * Applies to sampling started after the call; results never depend on it. */
+ * by the warp tiers.  on > 0 runs it on every batch; 0 sends every sample to the
+ * warp tiers; on < 0, the state of a new graph, runs it where it is faster: on
+ * batches of 32,768 samples or more whose warp tier is the global-bitmap one
+ * (ssa_set_warp_tier).  Applies to sampling started after the call; results
+ * never depend on it. */
 ssa_status ssa_set_lane_tier(const ssa_graph* g, int32_t on);
 
 /* Process-wide choice of the greedy kernel's launch shape (results never

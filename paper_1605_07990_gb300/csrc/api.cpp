@@ -126,7 +126,7 @@ struct ssa_graph {
   mutable int tuned_heavy = 0x7FFFFFFF;
   mutable int tuned_small_qcap = 0;  // queue of the small CTAs (0: min(n, 2^20))
   mutable int tuned_warp_global = 0;  // weighted-cascade IC: the global-bitmap warp tier takes every sample
-  mutable int tuned_lane_tier = 1;    // weighted-cascade IC: the lane tier (ssa_set_lane_tier)
+  mutable int tuned_lane_tier = 1;    // weighted-cascade IC: the lane tier: 0 never, 1 where it pays, 2 always
   GraphView view() const {
     GraphView v;
     v.n = n;
@@ -1741,7 +1741,7 @@ ssa_status ssa_set_warp_tier(const ssa_graph* g, int32_t global_bitmap) {
 ssa_status ssa_set_lane_tier(const ssa_graph* g, int32_t on) {
   if (!g) return fail(SSA_E_ARG, "null graph");
   std::lock_guard<std::mutex> lock(g->tune_mu);
-  g->tuned_lane_tier = on == 0 ? 0 : on == 1 ? 1 : 2;
+  g->tuned_lane_tier = on == 0 ? 0 : on < 0 ? 1 : 2;
   return SSA_OK;
 }
 
