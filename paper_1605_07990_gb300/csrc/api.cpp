@@ -136,18 +136,23 @@ struct ssa_graph {
     v.thr = thr;
     v.wc_inv = wc_inv;
     v.wc_inv_k = wc_inv_k;
-    v.lt_cum = lt_cum;
-    return v;
+    return v;  // without lt_cum, which another thread may be making: see lt_sums
   }
   // Running sums for LT with explicit weights, made once per graph.
-  cudaError_t lt_sums(cudaStream_t st) const {
+  cudaError_t lt_sums(cudaStream_t st, const uint32_t** sums) const {
     std::lock_guard<std::mutex> lock(tune_mu);
-    if (lt_cum) return cudaSuccess;
-    uint32_t* c = nullptr;
-    cudaError_t e = build_lt_cum(off, thr, n, m, &c, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // other streams read them from here on
-    if (e == cudaSuccess) lt_cum = c;
-    return e;
+    if (!lt_cum) {
+      uint32_t* c = nullptr;
+      cudaError_t e = build_lt_cum(off, thr, n, m, &c, st);
+      if (e == cudaSuccess) {
+        e = cudaStreamSynchronize(st);  // other streams read them from here on
+        if (e != cudaSuccess) cudaFreeAsync(c, st);
+      }
+      if (e != cudaSuccess) return e;
+      lt_cum = c;
+    }
+    *sums = lt_cum;
+    return cudaSuccess;
   }
 };
 
@@ -390,8 +395,8 @@ struct Sampler {
   ssa_status init_scratch(const ssa_graph* G, int mdl, Exec& X) {
     model = mdl;
     lt_cumulative = (mdl == 1 && G->weighting == SSA_W_EXPLICIT) ? 1 : 0;
-    if (lt_cumulative) CU(G->lt_sums(X.st));
     g = G->view();
+    if (lt_cumulative) CU(G->lt_sums(X.st, &g.lt_cum));
     wc_implicit = G->weighting == SSA_W_WC ? 1 : 0;
     cfg = sampler_config(g, mdl, wc_implicit != 0);
     {
