@@ -178,11 +178,13 @@ def roofline(kind, dom, ks, results, sm_count, clock_mhz, name, hbm_peak, hbm_ki
     16 per visited node (two CSR offsets), 8 per live edge taken (its record;
     one per visited node but the root), 8 per stored pool entry (node,
     sample), 12 per stored set (start, length), 1 per hit-tested set.  No
-    per-edge bytes: the gaps need only the in-degree.  (The graph store reads 8
-    and 4 bytes where this model counts 16 and 8; the model stays, so that
-    figures compare over time.)
+    per-edge bytes: the gaps need only the in-degree.  The graph store reads 8
+    and 4 bytes where this model, which figures over time share, counts 16 and 8:
+    "store" gives what the present layout asks for, and its fraction.
     Edge records (trivalency, explicit): bound "alu" in Philox draws/s against
-    PHILOX_MIN_INSTR, with 8 per examined in-edge in the HBM side figure."""
+    PHILOX_MIN_INSTR, with 8 per examined in-edge in the HBM side figure (the
+    packed trivalency store reads 4).  Every 4-edge group of a visited node draws:
+    rates of builds that drew for fewer groups do not compare."""
     if dom not in ("sample_cta", "sample_warp") or kind == "lt" or ks[dom]["ms"] <= 0:
         return None
     cta = dom == "sample_cta"
@@ -207,7 +209,10 @@ def roofline(kind, dom, ks, results, sm_count, clock_mhz, name, hbm_peak, hbm_ki
     if kind == "ic_wc":
         abytes = 16 * nv + 8 * max(nv - sets, 0) + 8 * st_e + 12 * st_s + max(sets - st_s, 0)
         ach = abytes / sec / 1e9
-        return {**common, "bound": "hbm", "achieved": ach, "peak": hbm_peak, "unit": "GB/s",
+        sbytes = abytes - 8 * nv - 4 * max(nv - sets, 0)  # 32-bit offsets, tails without thresholds
+        return {**common, "store": {"bytes_per_launch": sbytes / launches, "gbs": sbytes / sec / 1e9,
+                                    "frac": sbytes / sec / 1e9 / hbm_peak},
+                "bound": "hbm", "achieved": ach, "peak": hbm_peak, "unit": "GB/s",
                 "frac": ach / hbm_peak, "peak_source": hbm_kind,
                 "algorithmic_bytes_per_launch": abytes / launches,
                 "implied_edge_visits_per_s": ev / sec}
@@ -477,7 +482,7 @@ def main():
     ap.add_argument("--sample-only", type=int, default=0,
                     help="profiling case: only sample this many RR sets of the workload into a pool")
     ap.add_argument("--then-greedy", type=int, default=0,
-                    help="with --sample-only: also index the pool and run greedy Max-Coverage for this k")
+                    help="with --sample-only: also count the pool and run greedy Max-Coverage for this k")
     ap.add_argument("--tune", default="",
                     help="with --sample-only: IC sampler hand-overs MID_CAP,HEAVY_GROUPS[,GLOBAL_BITMAP_TIER] "
                          "(ssa_set_tuning, ssa_set_warp_tier)")
@@ -605,7 +610,7 @@ def main():
     if args.e2e_steps > 0:
         line["e2e"] = {"value": rr_e2e / te, "unit": UNIT, "h2d_bytes_per_step": int(el.m * 8),
                        "d2h_bytes_per_step": int(k * 4 + 64), "steps": args.e2e_steps,
-                       "includes": "graph upload + device CSR build (and, under weighted cascade, the gap-power "
+                       "includes": "graph upload + device CSR build (and, under weighted cascade, the gap "
                                    "table) + solve (the first solve on a new graph handle picks the sampler tiers) "
                                    "+ seeds to host",
                        "load_s_per_step": t_load / args.e2e_steps, "solve_s_per_step": t_solve / args.e2e_steps,

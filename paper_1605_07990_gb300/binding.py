@@ -325,7 +325,7 @@ class Solver:
         return _unpack(r, seeds, tr)
 
     def set_graphs(self, on=True):
-        """Run each round's index, greedy and stare as one CUDA graph."""
+        """Run each round's counts, greedy and stare as one CUDA graph."""
         _check(lib().ssa_solver_set_graphs(self.h, int(bool(on))))
         return self
 

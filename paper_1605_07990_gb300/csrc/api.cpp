@@ -170,7 +170,7 @@ struct NvtxRange {
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
-const char* const kClassName[SSA_K_COUNT] = {"ssa sample (warp tiers)", "ssa sample (CTA tier)", "ssa index",
+const char* const kClassName[SSA_K_COUNT] = {"ssa sample (warp tiers)", "ssa sample (CTA tier)", "ssa counts",
                                               "ssa greedy", "ssa stare"};
 
 struct Exec {
@@ -327,7 +327,7 @@ struct Sampler {
   int64_t edge_visits = 0, node_visits = 0, samples = 0, hit_samples = 0;
   int64_t cta_edge_visits = 0, cta_node_visits = 0, cta_samples = 0;
   int64_t cta_store_nodes = 0, cta_store_sets = 0;  // the CTA tier's sets written to the pool
-  int64_t draws = 0;  // Philox draws of IC edge groups / LT picks
+  int64_t draws = 0;  // Philox draws of IC edge groups and gaps / LT picks
   int64_t cta_draws = 0;
 
   void tally(int64_t count) {
@@ -1178,12 +1178,12 @@ struct ssa_solver {
   bool own_stream = false;
   Exec X;
   int64_t byte_cap = 0;
-  // workspaces kept across solves: sampler scratch per model, index and greedy buffers
+  // workspaces kept across solves: sampler scratch per model, counts and greedy buffers
   Sampler S[2];
   bool s_ready[2] = {false, false};
   Cover C;
   bool c_ready = false;
-  // CUDA graphs of a round's device work (index, greedy, stare), one
+  // CUDA graphs of a round's device work (counts, greedy, stare), one
   // executable per (algorithm, round), patched in place by later solves
   bool use_graphs = false;
   bool shared_gpu = false;  // concurrent solves share the GPU (serving): cluster-shaped greedy

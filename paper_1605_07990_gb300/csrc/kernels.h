@@ -72,7 +72,7 @@ struct Counters {
   unsigned long long cta_edge_visits;  // the CTA tier's share of the two above
   unsigned long long cta_node_visits;
   unsigned long long cta_draws;    // the CTA tier's share of draws
-  unsigned long long draws;        // Philox draws (IC: one per 4-edge group that needed coins)
+  unsigned long long draws;        // Philox draws (IC: one per 4-edge group of a visited node, or per two gaps)
   unsigned long long ok_end;        // start of the first pool reservation that did not fit (the
                                     // host sets ~0 before a storing launch): the ones that fit end there
   unsigned long long fail_count;    // samples whose reservation did not fit (listed in fail_list)

@@ -13,11 +13,12 @@
 // unit of one Philox draw, one aligned 16-byte load of tails) dealt to lanes by
 // a warp prefix sum, every group draws its coins, and the live tails are
 // visited 32 at a time; the CTA tier shares long in-lists between its warps.
-// Bound: integer issue (ALU pipe 58%, multiplier 52%, 69% of issue slots), 102
-// instructions per 32 groups, 39 of them Philox.  On the 2^20-node trivalency
-// R-MAT graph (giant sets of 137,000 nodes) 350 -> 205 ms of sampling per
-// D-SSA solve, 5.1e10 -> 1.5e11 draws/s over the solve, against the form that
-// asked for each tail first and visited slab by slab.
+// Bound: integer issue (67% of all issue slots and 60% of the ALU pipe over a
+// whole launch of 24,576 trivalency sets; the level barriers are 4% of its
+// stalls): 171 instructions per 32 draws, 39 of them Philox.  On the 2^20-node
+// R-MAT graph (giant sets of 137,000 nodes) a D-SSA solve went from 366 to 205 ms
+// against the form that asked for each tail first, drew for fewer groups (so the
+// two forms' draws a second say nothing) and visited slab by slab.
 // IC with weighted-cascade weights: every in-edge of a node has the same
 // probability, so each lane walks one frontier node's in-list by geometric
 // gaps between live edges (the gap form below); the work per node is a
@@ -147,7 +148,7 @@ __device__ __forceinline__ bool hash_insert(uint32_t* H, uint32_t u, uint32_t* s
     if (prev == key) return false;
     h = (h + 1u) & ((1u << HBITS) - 1u);
   }
-  return false;  // not reached: the table is never more than half full
+  return false;  // not reached: the cap and one round's 64 at most, 576 of 1,024 and 16,448 of 32,768 slots
 }
 
 // Threshold of a packed trivalency edge (its class in the two high bits).

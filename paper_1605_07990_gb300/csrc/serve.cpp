@@ -6,7 +6,7 @@
 // admitted as soon as a slot is free and its estimated RR-pool footprint fits
 // the server's byte budget (footprints are learned per (graph, model, k) from
 // finished requests).  Admitted requests run concurrently on their slots'
-// streams, so their sampling, index, greedy and stare kernels overlap on the
+// streams, so their sampling, counts, greedy and stare kernels overlap on the
 // GPU while later arrivals wait for a slot or for memory.  Every request's
 // randomness is keyed by its own seed, so its answer does not depend on what
 // else is in flight.
@@ -127,7 +127,7 @@ struct ssa_server {
       ssa_status s = SSA_OK;
       if (!solvers[(size_t)r->graph]) {
         s = ssa_solver_create(graphs[(size_t)r->graph], st, 0, &solvers[(size_t)r->graph]);
-        // each round's index, greedy and stare as one CUDA graph, reused by later requests;
+        // each round's counts, greedy and stare as one CUDA graph, reused by later requests;
         // the greedy in one thread-block cluster, so concurrent requests keep the other SMs
         if (s == SSA_OK) s = ssa_solver_set_graphs(solvers[(size_t)r->graph], 1);
         if (s == SSA_OK) s = ssa_solver_set_shared(solvers[(size_t)r->graph], 1);
