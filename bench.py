@@ -623,7 +623,7 @@ def main():
         res3, ms3 = run_solves(P, solver3, EXTRA, args.extra_steps, 2, seed_of, stream, torch)
         ex = summarise(P, EXTRA, res3, ms3, sm_count, clock_mhz)
         ex["config"] = {"n": el2.n, "m": el2.m, "algo": "D-SSA", "model": "IC", "weights": "trivalency", "k": 100,
-                        "eps": 0.1, "delta": "1/n", "l2": "CSR 137 MB: mostly L2-resident"}
+                        "eps": 0.1, "delta": "1/n", "l2": "CSR 68 MB: mostly L2-resident"}
         ex["steps"] = args.extra_steps
         line["extra"] = {EXTRA: ex}
         solver3.free()
