@@ -178,7 +178,8 @@ ssa_status ssa_set_warp_tier(const ssa_graph* g, int32_t global_bitmap);
  * by the warp tiers.  on > 0 runs it on every batch; 0 sends every sample to the
  * warp tiers; on < 0, the state of a new graph, runs it where it is faster: on
  * batches of 32,768 samples or more whose warp tier is the global-bitmap one
- * (ssa_set_warp_tier).  Applies to sampling started after the call; results
+ * (ssa_set_warp_tier), and elsewhere on those of 262,144 or more whose sets have
+ * a few nodes.  Applies to sampling started after the call; results
  * never depend on it. */
 ssa_status ssa_set_lane_tier(const ssa_graph* g, int32_t on);
 

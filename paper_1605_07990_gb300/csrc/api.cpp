@@ -475,12 +475,16 @@ struct Sampler {
     // the batch is large: from 32,768 samples on (GB300, us off / on: 2^21 nodes
     // 516 / 480, 2^23 696 / 636, 2^25 1164 / 1168; 262,144 samples 2133 / 1063,
     // 2582 / 1304, 3726 / 2218; 8192 samples 335 / 401, 486 / 563, 887 / 967).
-    // Before warps with their hash in shared memory it only adds its own tail
-    // (2^14 to 2^20 nodes, 1024 to 262,144 samples: 70 / 156 to 447 / 526 us).
-    J.lane_tier = model == 0 && wc_implicit &&
-                          (lane_tier == 2 || (lane_tier == 1 && warp_global && count >= LANE_TIER_SAMPLES))
-                      ? 1
-                      : 0;
+    // Before warps with their hash in shared memory it mostly adds its own tail
+    // (2^14 to 2^20 nodes, 1024 to 262,144 samples: 70 / 156 to 447 / 526 us),
+    // but not where the sets are a few nodes and the batch is large, as on sparse
+    // graphs (2^14 nodes, us off / on: mean 2.7 nodes, 65,536 samples 161 / 175,
+    // 300,000 455 / 350, 4M 5032 / 3054; mean 4.2, 300,000 458 / 401; mean 8.8,
+    // 300,000 488 / 542, 4M 5168 / 4811; 2^20 nodes, mean 5.0, 300,000 677 / 667,
+    // 4M 6522 / 5131): the sets of the solve so far say which.
+    const bool small_sets = samples >= 1024 && node_visits <= LANE_TIER_MEAN * samples;
+    const bool pays = warp_global ? count >= LANE_TIER_SAMPLES : small_sets && count >= LANE_TIER_SMALL_SETS;
+    J.lane_tier = model == 0 && wc_implicit && (lane_tier == 2 || (lane_tier == 1 && pays)) ? 1 : 0;
     J.lane_list = lane_list;
     J.wg_bitmap = wg_bitmap;
     J.wg_queue = wg_queue;

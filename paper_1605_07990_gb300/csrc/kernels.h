@@ -135,8 +135,9 @@ struct SampleJob {
   Counters* ctr = nullptr;
 };
 
-// Samples of a batch from which the lane tier runs before the global-bitmap warp tier.
-constexpr int64_t LANE_TIER_SAMPLES = 32768;
+// Samples of a batch from which the lane tier runs before the global-bitmap warp
+// tier, and before the shared-memory one where sets have at most LANE_TIER_MEAN nodes.
+constexpr int64_t LANE_TIER_SAMPLES = 32768, LANE_TIER_SMALL_SETS = 1 << 18, LANE_TIER_MEAN = 6;
 
 struct LaunchCfg {
   int num_sms = 152;
