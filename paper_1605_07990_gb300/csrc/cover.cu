@@ -545,15 +545,10 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
     const bool small = session && !first && !small_off && J.k - i >= 64 && key_gain(best) <= SENTS / 64;
     const int i0 = i;
     if (session) {
-      // A few candidates a pick serve, and the fewer there are, the fewer members one
-      // block lowers where picks cover hundreds of thousands of large sets.  All
-      // rounds of plain SSA under LT at eps = 0.05, ms, with 16,384 after a bulk pick
-      // and 32 a pick (2,048 at least) else / 16 (512) / 8 (512) / 4 (256): 2^20
-      // nodes, k = 100 48.0 / 37.7 / 33.3 / 30.2, k = 10 5.7 / 4.1 / 4.1 / 3.8; 2^23,
-      // k = 100 22.6 / 15.8 / 14.4 / 13.9, targeted 7.2 / 5.9 / 5.6 / 6.0; but D-SSA
-      // k = 500 5.3 / 5.1 / 5.0 / 5.9 (sessions end early, and each has its passes).
-      const long long few = max(512ll, 8ll * (J.k - i));
-      cap_n = small ? SCANDS : min((long long)GCANDS, few);
+      // exact counts: some dozens of candidates a pick serve, and the fewer there
+      // are, the cheaper an argmax (the counts before a bulk pick need them all)
+      const long long few = max(2048ll, 32ll * (J.k - i));
+      cap_n = small ? SCANDS : first && bulk ? GCANDS : min((long long)GCANDS, few);
       cap_e = small ? SENTS : (long long)J.ents_cap;
       if (tight) cap_e = min(cap_e, (long long)(J.chunk_cap / 3));  // a set takes 2.5 chunks a candidate at most
       long long have = 0, sum = 0, total = 0;
