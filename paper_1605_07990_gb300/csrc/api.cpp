@@ -718,12 +718,12 @@ struct Cover {
   int32_t* cnt_total = nullptr;  // counts of the sets [0, counted); padding 0
   int32_t* cnt = nullptr;        // working gains of the current Max-Coverage
   uint16_t* lid = nullptr;       // greedy: local ids of the candidates, then their mark bits; zero between launches
-  bool lid_dirty = true;
+  bool lid_dirty = true;         // lid and the shared picks' decrements are to be zeroed
   uint8_t* covered = nullptr;
   int64_t covered_cap = 0;
   uint8_t* in_seed = nullptr;
   unsigned char* ctl = nullptr;  // greedy control block
-  int32_t* cand = nullptr;       // 3 x GREEDY_CANDS: ids, list lengths, list offsets
+  int32_t* cand = nullptr;       // 4 x GREEDY_CANDS: ids, list lengths, list offsets, shared picks' decrements
   unsigned int* ents = nullptr;  // greedy candidate lists
   int64_t ents_cap = 0;
   uint4* chunks = nullptr;
@@ -759,7 +759,7 @@ struct Cover {
     TRY(reset(X));
     TRY(dev_alloc(&in_seed, (size_t)n_pad, X.st));
     TRY(dev_alloc(&ctl, GREEDY_CTL_BYTES, X.st));
-    TRY(dev_alloc(&cand, 3 * (size_t)GREEDY_CANDS, X.st));
+    TRY(dev_alloc(&cand, 4 * (size_t)GREEDY_CANDS, X.st));
     TRY(dev_alloc(&d_count, 1, X.st));
     TRY(dev_alloc(&d_first, 2, X.st));
     CU(cudaMallocHost(reinterpret_cast<void**>(&h_sync), sizeof(unsigned int) * 128));
@@ -867,6 +867,7 @@ struct Cover {
     TRY(dev_renew(&chunks, &chunk_cap, chunks_now + GREEDY_CHUNKS_SPARE + chunks_now / 16 + 1, X.st));
     if (lid_dirty) {
       CU(cudaMemsetAsync(lid, 0, sizeof(uint16_t) * lid_words(), X.st));
+      CU(cudaMemsetAsync(cand + 3 * GREEDY_CANDS, 0, sizeof(int32_t) * GREEDY_CANDS, X.st));
       lid_dirty = false;
     }
     return SSA_OK;
@@ -919,6 +920,7 @@ struct Cover {
     J.cand_id = cand;
     J.cand_len = cand + GREEDY_CANDS;
     J.cand_off = reinterpret_cast<unsigned int*>(cand + 2 * GREEDY_CANDS);
+    J.cand_dec = reinterpret_cast<unsigned int*>(cand + 3 * GREEDY_CANDS);
     J.ents = ents;
     J.ents_cap = ents_now;
     J.chunks = chunks;

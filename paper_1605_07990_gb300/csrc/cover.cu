@@ -151,6 +151,9 @@ constexpr int SCANDS = 4096;       // candidates and list entries of a session t
 constexpr int SENTS = 24576;       // keys, ids, offsets, lengths (12 bytes a candidate), lists (6 an entry)
 constexpr int STHREADS = 256;      // threads that make its picks
 constexpr int GHISTS = 4;          // histograms in turn, so that one is cleared while another fills
+constexpr int GSHARE = 4096;       // sets of a list from which every block covers a share of them (two grid barriers
+                                   // and adding up a turn; 820,000 IC sets, k = 300: 3.7 ms alone and from 2,048
+                                   // sets on, 3.0 from 4,096 on)
 constexpr int GLONG = 256;         // members of a set beyond which its list is made by several warps
 
 // Grid barrier for a cooperative launch.  The last block to arrive runs f()
@@ -363,7 +366,8 @@ __device__ __forceinline__ void for_live_members(const GreedyJob& J, int64_t war
 // barriers, the argmax over shared memory), 1.5 us while a pick covers tens of
 // sets; picks that cover thousands load the issue slots of the one SM (a member
 // is three instructions: chunks hold byte offsets of keys), whose ALU pipe is
-// busy for 12% (IC, 1000 picks) to 24% (LT, 500) of a launch.  Measured on
+// busy for 12% (IC, 1000 picks) to 24% (LT, 500) of a launch.  The blocks of a
+// large pool's greedy (SHARE) cover such a pick together.  Measured on
 // GB300 against the former design (an inverted index of all entries, a grid
 // barrier of ~6 us per pick): 1000 picks over 134,016 sets of the 2^23-node
 // R-MAT graph 8.7 -> 2.3 ms, 500 over 131,832 LT sets there 6.0 -> 2.1 ms, 100
@@ -384,10 +388,9 @@ __device__ __forceinline__ void for_live_members(const GreedyJob& J, int64_t war
 // sets covered by a pass over the pool instead; room for 2^27 chunks: 268 ms.
 //
 // Gains of 0 go by smallest id.  Barrier waits are bounded (sync[SYNC_ERR] on
-// timeout).  Between two barriers block 0 may make up to GCANDS picks and lower
-// every member that the chunks hold (268M), hundreds of milliseconds; it shows
-// its progress, and the bound is on polls that see none.
-template <bool CLUSTER>
+// timeout).  Between two barriers block 0 may make up to GCANDS picks, tens of
+// milliseconds; it shows its progress, and the bound is on polls that see none.
+template <bool CLUSTER, bool SHARE>
 __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ unsigned long long s_red[32];
@@ -788,209 +791,266 @@ __global__ void __launch_bounds__(1024, 1) k_greedy(GreedyJob J) {
       auto progress = [&](unsigned int step) {
         if (!CLUSTER) __stcg(J.sync + SYNC_PROGRESS, (unsigned int)(i + 1) * 0x9E3779B1u + step);
       };
-      if (blockIdx.x == 0 && !overflow && small) {
-        // everything into shared memory: the lists of the sets one after the
-        // other (count, local ids; count 0: covered), the candidates' lists as
-        // places in them
-        s_id = s_key + SCANDS;
-        unsigned short* s_off16 = reinterpret_cast<unsigned short*>(s_id + SCANDS);
-        unsigned short* s_len16 = s_off16 + SCANDS;
-        unsigned short* s_ent16 = s_len16 + SCANDS;
-        unsigned short* s_mem = s_ent16 + SENTS;
-        __shared__ unsigned int s_nmem, s_over;
-        if (tid == 0) s_nmem = s_over = 0u;
-        const int E = (int)__ldcg(J.ncand + 4);
-        for (int t = tid; t < SCANDS; t += 1024) {
-          const unsigned int len = t < nc ? (unsigned int)__ldcg(J.cand_len + t) : 0u;
-          s_key[t] = t < nc ? (len << GBITS) | (unsigned int)(GCANDS - 1 - t) : 0u;
-          s_id[t] = t < nc ? (unsigned int)__ldcg(J.cand_id + t) : 0u;
-          s_off16[t] = t < nc ? (unsigned short)__ldcg(J.cand_off + t) : 0;
-          s_len16[t] = (unsigned short)len;
-        }
-        __syncthreads();
-        // the first list entry of a set to come (it sets the count's high bit) copies the set
-        for (int x0 = tid; x0 < E; x0 += 4096) {
-          unsigned int at[4], old[4];
+      // Picks out of lists in memory: block 0 picks and covers.  With SHARE it covers
+      // the sets of a short list itself; a list of GSHARE sets or more ends its turn: at
+      // a barrier the blocks learn the pick, each covers a share of the list and lowers
+      // a copy of the keys in its own shared memory (0 at first), and what the others
+      // lowered adds up in cand_dec, which block 0 subtracts behind a second barrier.
+      const int ncp = (nc + 1023) & ~1023;
+      // Slots `slot` and `slot` + 1 of a list of cnt.  Picks that cover thousands
+      // of sets load an SM's issue slots: three instructions a member (the pick's
+      // own key goes down to gain 0 with the others).
+      auto lower = [&](unsigned int pair, int slot, int cnt) {
+        if (slot < cnt) atomicSub(reinterpret_cast<unsigned int*>(s_dyn + (pair & 0xFFFFu)), 1u << GBITS);
+        if (slot + 1 < cnt) atomicSub(reinterpret_cast<unsigned int*>(s_dyn + (pair >> 16)), 1u << GBITS);
+      };
+      // the sets of list [off, off + len) from place `base` on in steps of `stride`
+      // (warp-uniform; cs: the lane's first), 2^sh lanes a set
+      auto cover = [&](const unsigned int off, const int len, int base, const int stride, unsigned int cs, const int sh,
+                       const bool own) {
+        const int per_set = 1 << sh, r0 = lane & (per_set - 1), first_slots = 8 * per_set - 4;
+        for (; base < len; base += stride) {
+          if (base > 0 && tid == 0 && own) progress((unsigned int)base);
+          const unsigned int c0 = cs;
+          if (base + stride < len) cs = __ldcg(J.ents + off + base + stride + (lane >> sh));
+          uint4 a = make_uint4(0u, 0u, 0u, 0u);
+          if (base + (lane >> sh) < len) a = __ldcg(J.chunks + c0 + r0);  // may run past the list: spare chunks
+          const int cnt_l = (int)__shfl_sync(FULL_MASK, a.x, lane & ~(per_set - 1));  // 0: covered
+          if (r0 == 0) {
+            if (cnt_l) {
+              J.covered[a.y] = 1;
+              *reinterpret_cast<unsigned int*>(J.chunks + c0) = 0u;
+            }
+          } else {
+            lower(a.x, 8 * r0 - 4, cnt_l);
+            lower(a.y, 8 * r0 - 2, cnt_l);
+          }
+          lower(a.z, 8 * r0, cnt_l);
+          lower(a.w, 8 * r0 + 2, cnt_l);
+          // what is left of the warp's sets is dealt to the lanes chunk by chunk
+          const int rest = r0 == 0 && cnt_l > first_slots ? (cnt_l - first_slots + 7) >> 3 : 0;
+          if (!__any_sync(FULL_MASK, rest)) continue;
+          const int incl = warp_inclusive_scan(rest, lane);
+          const int total = __shfl_sync(FULL_MASK, incl, 31);
+          for (int q0 = 0; q0 < total; q0 += 32) {
+            const int q = q0 + lane;
+            int o = 0;
 #pragma unroll
-          for (int t = 0; t < 4; ++t) at[t] = x0 + 1024 * t < E ? __ldcg(J.ents + x0 + 1024 * t) : 0u;
-#pragma unroll
-          for (int t = 0; t < 4; ++t)
-            old[t] = x0 + 1024 * t < E ? atomicOr(reinterpret_cast<unsigned int*>(J.chunks + at[t]), 0x80000000u)
-                                       : 0x80000000u;
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            if (old[t] >> 31) continue;
-            const unsigned int place = atomicAdd(&s_nmem, old[t] + 1u);
-            s_mem[place] = (unsigned short)old[t];
-            const unsigned short* ids = reinterpret_cast<const unsigned short*>(J.chunks + at[t]) + 4;
-            for (unsigned int y = 0; y < old[t]; ++y) s_mem[place + 1u + y] = __ldcg(ids + y);
-            *reinterpret_cast<unsigned int*>(J.chunks + at[t]) = 0x80000000u | place;
+            for (int s = 16; s; s >>= 1) {
+              const int x = __shfl_sync(FULL_MASK, incl, o + s - 1);
+              if (x <= q) o += s;
+            }
+            o = o > 31 ? 31 : o;
+            const int r = q - (__shfl_sync(FULL_MASK, incl, o) - __shfl_sync(FULL_MASK, rest, o));
+            const unsigned int oc = __shfl_sync(FULL_MASK, c0, o);
+            const int ocnt = __shfl_sync(FULL_MASK, cnt_l, o);
+            if (q < total) {
+              const uint4 w = __ldcg(J.chunks + oc + per_set + r);
+              lower(w.x, first_slots + 8 * r, ocnt);
+              lower(w.y, first_slots + 8 * r + 2, ocnt);
+              lower(w.z, first_slots + 8 * r + 4, ocnt);
+              lower(w.w, first_slots + 8 * r + 6, ocnt);
+            }
           }
         }
-        __syncthreads();
-        for (int x = tid; x < E; x += 1024)
-          s_ent16[x] =
-              (unsigned short)__ldcg(reinterpret_cast<const unsigned int*>(J.chunks + __ldcg(J.ents + x)));
-        __syncthreads();
-        if (tid < STHREADS) {
-          // as the picks below, by eight warps and without a load from memory
-          auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(STHREADS) : "memory"); };
+      };
+      for (bool begun = false;; begun = true) {
+        int turn = 0;  // 1 + the pick that ended block 0's turn (0: the session is over)
+        if (blockIdx.x == 0 && !overflow && small) {
+          // everything into shared memory: the lists of the sets one after the
+          // other (count, local ids; count 0: covered), the candidates' lists as
+          // places in them
+          s_id = s_key + SCANDS;
+          unsigned short* s_off16 = reinterpret_cast<unsigned short*>(s_id + SCANDS);
+          unsigned short* s_len16 = s_off16 + SCANDS;
+          unsigned short* s_ent16 = s_len16 + SCANDS;
+          unsigned short* s_mem = s_ent16 + SENTS;
+          __shared__ unsigned int s_nmem, s_over;
+          if (tid == 0) s_nmem = s_over = 0u;
+          const int E = (int)__ldcg(J.ncand + 4);
+          for (int t = tid; t < SCANDS; t += 1024) {
+            const unsigned int len = t < nc ? (unsigned int)__ldcg(J.cand_len + t) : 0u;
+            s_key[t] = t < nc ? (len << GBITS) | (unsigned int)(GCANDS - 1 - t) : 0u;
+            s_id[t] = t < nc ? (unsigned int)__ldcg(J.cand_id + t) : 0u;
+            s_off16[t] = t < nc ? (unsigned short)__ldcg(J.cand_off + t) : 0;
+            s_len16[t] = (unsigned short)len;
+          }
+          __syncthreads();
+          // the first list entry of a set to come (it sets the count's high bit) copies the set
+          for (int x0 = tid; x0 < E; x0 += 4096) {
+            unsigned int at[4], old[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) at[t] = x0 + 1024 * t < E ? __ldcg(J.ents + x0 + 1024 * t) : 0u;
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+              old[t] = x0 + 1024 * t < E ? atomicOr(reinterpret_cast<unsigned int*>(J.chunks + at[t]), 0x80000000u)
+                                         : 0x80000000u;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+              if (old[t] >> 31) continue;
+              const unsigned int place = atomicAdd(&s_nmem, old[t] + 1u);
+              s_mem[place] = (unsigned short)old[t];
+              const unsigned short* ids = reinterpret_cast<const unsigned short*>(J.chunks + at[t]) + 4;
+              for (unsigned int y = 0; y < old[t]; ++y) s_mem[place + 1u + y] = __ldcg(ids + y);
+              *reinterpret_cast<unsigned int*>(J.chunks + at[t]) = 0x80000000u | place;
+            }
+          }
+          __syncthreads();
+          for (int x = tid; x < E; x += 1024)
+            s_ent16[x] =
+                (unsigned short)__ldcg(reinterpret_cast<const unsigned int*>(J.chunks + __ldcg(J.ents + x)));
+          __syncthreads();
+          if (tid < STHREADS) {
+            // as the picks below, by eight warps and without a load from memory
+            auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(STHREADS) : "memory"); };
+            unsigned int bk = 0xFFFFFFFFu;
+            int par = 0;
+            while (i < J.k) {
+              if (bk && s_key[(GCANDS - 1 - (bk & (GCANDS - 1))) & (SCANDS - 1)] != bk) {
+                bk = 0u;
+#pragma unroll
+                for (int r = 0; r < SCANDS / STHREADS; ++r) bk = max(bk, s_key[r * STHREADS + tid]);
+              }
+              const unsigned int wk = __reduce_max_sync(FULL_MASK, bk);
+              if (lane == 0) s_w[par][wid] = wk;
+              sync();
+              const unsigned int top = __reduce_max_sync(FULL_MASK, lane < STHREADS / 32 ? s_w[par][lane] : 0u);
+              par ^= 1;
+              const int l = GCANDS - 1 - (int)(top & (GCANDS - 1));
+              const int g = (int)(top >> GBITS);
+              if (top == 0u || gain_key(g, s_id[l]) < keystar) break;
+              if (tid == 0) {
+                J.seeds[i] = (int32_t)s_id[l];
+                J.gains[i] = g;
+              }
+              const int off = s_off16[l], len = s_len16[l];
+              for (int x = tid; x < len; x += STHREADS) {
+                const int m = s_ent16[off + x];
+                const int c = s_mem[m];
+                if (c) s_mem[m] = 0;
+                for (int y = 1; y <= c; ++y)
+                  atomicSub(reinterpret_cast<unsigned int*>(s_dyn + s_mem[m + y]), 1u << GBITS);
+              }
+              i += 1;
+              sync();
+              if (tid == (l & (STHREADS - 1))) s_key[l] = 0u;  // never again
+            }
+            if (tid == 0) *(volatile unsigned int*)&s_over = 1u;
+          } else if (!CLUSTER && tid == STHREADS) {
+            // an idle warp shows the progress: every pick lowers the sum of the warps'
+            // best keys (a store by the picking warps cost 1% of 1000 picks)
+            for (int t = 0; t < (1 << 20) && *(volatile unsigned int*)&s_over == 0u; ++t) {
+              unsigned int sum = 0u;
+#pragma unroll
+              for (int w = 0; w < STHREADS / 32; ++w)
+                sum += *(volatile unsigned int*)&s_w[0][w] + *(volatile unsigned int*)&s_w[1][w];
+              __stcg(J.sync + SYNC_PROGRESS, sum);
+              __nanosleep(1000);
+            }
+          }
+          __syncthreads();
+          // the covered flags of the sets whose count is 0 now
+          for (int x = tid; x < E; x += 1024)
+            if (s_mem[s_ent16[x]] == 0)
+              J.covered[__ldcg(reinterpret_cast<const uint2*>(J.chunks + __ldcg(J.ents + x))).y] = 1;
+          s_id = s_key + GCANDS;
+        } else if (blockIdx.x == 0 && !overflow) {
+          if (!begun) {
+            for (int t = tid; t < ncp; t += 1024) {
+              s_key[t] = t < nc ? ((unsigned int)__ldcg(J.cand_len + t) << GBITS) | (unsigned int)(GCANDS - 1 - t) : 0u;
+              s_id[t] = t < nc ? (unsigned int)__ldcg(J.cand_id + t) : 0u;
+              s_off[t] = t < nc ? __ldcg(J.cand_off + t) : 0u;
+            }
+          }
+          __syncthreads();
+          // best key of the thread's candidates tid, tid + 1024, ...; gains only
+          // fall, so it stands until that candidate's own key changes
           unsigned int bk = 0xFFFFFFFFu;
           int par = 0;
           while (i < J.k) {
-            if (bk && s_key[(GCANDS - 1 - (bk & (GCANDS - 1))) & (SCANDS - 1)] != bk) {
+            if (bk && s_key[GCANDS - 1 - (bk & (GCANDS - 1))] != bk) {
               bk = 0u;
 #pragma unroll
-              for (int r = 0; r < SCANDS / STHREADS; ++r) bk = max(bk, s_key[r * STHREADS + tid]);
+              for (int r = 0; r < GCANDS / 1024; ++r)
+                if (r * 1024 < ncp) bk = max(bk, s_key[r * 1024 + tid]);
             }
             const unsigned int wk = __reduce_max_sync(FULL_MASK, bk);
             if (lane == 0) s_w[par][wid] = wk;
-            sync();
-            const unsigned int top = __reduce_max_sync(FULL_MASK, lane < STHREADS / 32 ? s_w[par][lane] : 0u);
+            __syncthreads();
+            const unsigned int top = __reduce_max_sync(FULL_MASK, s_w[par][lane]);
             par ^= 1;
             const int l = GCANDS - 1 - (int)(top & (GCANDS - 1));
             const int g = (int)(top >> GBITS);
-            if (top == 0u || gain_key(g, s_id[l]) < keystar) break;
+            const unsigned int off = s_off[l], v = s_id[l];
+            if (top == 0u || gain_key(g, v) < keystar) break;
+            // with many picks to go and gains this small, a session out of shared memory is quicker
+            if (!small_off && i - i0 >= 64 && J.k - i >= 192 && g <= SENTS / 96) break;
+            const int len = __ldcg(J.cand_len + l);
+            // lanes per set: eight chunks of each set at once while the sets are few, else two
+            const unsigned int spec = __ldcg(J.ents + off + (tid >> 3));  // the buffer has spare entries past the last list
+            const int sh = len <= 128 ? 3 : 1;
+            const unsigned int cs = sh == 3 ? spec : __ldcg(J.ents + off + (tid >> 1));
             if (tid == 0) {
-              J.seeds[i] = (int32_t)s_id[l];
+              J.seeds[i] = (int32_t)v;
               J.gains[i] = g;
+              progress(0u);
             }
-            const int off = s_off16[l], len = s_len16[l];
-            for (int x = tid; x < len; x += STHREADS) {
-              const int m = s_ent16[off + x];
-              const int c = s_mem[m];
-              if (c) s_mem[m] = 0;
-              for (int y = 1; y <= c; ++y)
-                atomicSub(reinterpret_cast<unsigned int*>(s_dyn + s_mem[m + y]), 1u << GBITS);
+            if (SHARE && len >= GSHARE) {
+              i += 1;
+              turn = i < J.k ? l + 1 : 0;  // the last pick's sets need no covering
+              break;
             }
+            cover(off, len, (tid & ~31) >> sh, 1024 >> sh, cs, sh, true);
             i += 1;
-            sync();
-            if (tid == (l & (STHREADS - 1))) s_key[l] = 0u;  // never again
-          }
-          if (tid == 0) *(volatile unsigned int*)&s_over = 1u;
-        } else if (!CLUSTER && tid == STHREADS) {
-          // an idle warp shows the progress: every pick lowers the sum of the warps'
-          // best keys (a store by the picking warps cost 1% of 1000 picks)
-          for (int t = 0; t < (1 << 20) && *(volatile unsigned int*)&s_over == 0u; ++t) {
-            unsigned int sum = 0u;
-#pragma unroll
-            for (int w = 0; w < STHREADS / 32; ++w)
-              sum += *(volatile unsigned int*)&s_w[0][w] + *(volatile unsigned int*)&s_w[1][w];
-            __stcg(J.sync + SYNC_PROGRESS, sum);
-            __nanosleep(1000);
+            __syncthreads();
+            // never again: its owner, the only thread that reads it, takes it out
+            if (tid == (l & 1023)) s_key[l] = 0u;
           }
         }
-        __syncthreads();
-        // the covered flags of the sets whose count is 0 now
-        for (int x = tid; x < E; x += 1024)
-          if (s_mem[s_ent16[x]] == 0)
-            J.covered[__ldcg(reinterpret_cast<const uint2*>(J.chunks + __ldcg(J.ents + x))).y] = 1;
-        s_id = s_key + GCANDS;
-      } else if (blockIdx.x == 0 && !overflow) {
-        const int ncp = (nc + 1023) & ~1023;
-        for (int t = tid; t < ncp; t += 1024) {
-          s_key[t] = t < nc ? ((unsigned int)__ldcg(J.cand_len + t) << GBITS) | (unsigned int)(GCANDS - 1 - t) : 0u;
-          s_id[t] = t < nc ? (unsigned int)__ldcg(J.cand_id + t) : 0u;
-          s_off[t] = t < nc ? __ldcg(J.cand_off + t) : 0u;
+        if (!begun) {
+          // the local ids go back to 0 for the next session
+          const int64_t b0 = gridDim.x > 1 ? blockIdx.x - 1 : 0, nb = gridDim.x > 1 ? gridDim.x - 1 : 1;
+          if (b0 >= 0)
+            for (int64_t t = b0 * 1024 + tid; t < nc; t += nb * 1024) J.lid[__ldcg(J.cand_id + t)] = 0;
+          if (SHARE && blockIdx.x != 0 && !overflow && !small)
+            for (int t = tid; t < ncp; t += 1024) s_key[t] = 0u;
         }
-        __syncthreads();
-        // best key of the thread's candidates tid, tid + 1024, ...; gains only
-        // fall, so it stands until that candidate's own key changes
-        unsigned int bk = 0xFFFFFFFFu;
-        int par = 0;
-        while (i < J.k) {
-          if (bk && s_key[GCANDS - 1 - (bk & (GCANDS - 1))] != bk) {
-            bk = 0u;
-#pragma unroll
-            for (int r = 0; r < GCANDS / 1024; ++r)
-              if (r * 1024 < ncp) bk = max(bk, s_key[r * 1024 + tid]);
-          }
-          const unsigned int wk = __reduce_max_sync(FULL_MASK, bk);
-          if (lane == 0) s_w[par][wid] = wk;
-          __syncthreads();
-          const unsigned int top = __reduce_max_sync(FULL_MASK, s_w[par][lane]);
-          par ^= 1;
-          const int l = GCANDS - 1 - (int)(top & (GCANDS - 1));
-          const int g = (int)(top >> GBITS);
-          const unsigned int off = s_off[l], v = s_id[l];
-          if (top == 0u || gain_key(g, v) < keystar) break;
-          // with many picks to go and gains this small, a session out of shared memory is quicker
-          if (!small_off && i - i0 >= 64 && J.k - i >= 192 && g <= SENTS / 96) break;
+        if (blockIdx.x == 0 && tid == 0) {
+          J.ncand[2] = (unsigned int)i;
+          if (SHARE) J.ncand[5] = (unsigned int)turn;
+        }
+        if (!greedy_barrier<CLUSTER>(J, s_wait, [&] {
+              return ((unsigned long long)__ldcg(J.ncand + 2) << 15) | (unsigned long long)__ldcg(J.ncand + 5);
+            }, info)) return;
+        i = (int)(info >> 15);
+        const int l = (int)(info & 0x7FFFull) - 1;
+        if (!SHARE || l < 0) break;
+        {
+          const unsigned int off = __ldcg(J.cand_off + l);
           const int len = __ldcg(J.cand_len + l);
-          // lanes per set: eight chunks of each set at once while the sets are few, else two
-          const unsigned int spec = __ldcg(J.ents + off + (tid >> 3));  // the buffer has spare entries past the last list
-          const int sh = len <= 128 ? 3 : 1;
-          const int per_set = 1 << sh, r0 = lane & (per_set - 1), first_slots = 8 * per_set - 4;
-          unsigned int cs = sh == 3 ? spec : __ldcg(J.ents + off + (tid >> 1));
-          if (tid == 0) {
-            J.seeds[i] = (int32_t)v;
-            J.gains[i] = g;
-            progress(0u);
-          }
-          // Slots `slot` and `slot` + 1 of a list of cnt.  Picks that cover thousands
-          // of sets are bound by this SM's issue slots: three instructions a member
-          // (the pick's own key goes down to gain 0 with the others).
-          auto lower = [&](unsigned int pair, int slot, int cnt) {
-            if (slot < cnt) atomicSub(reinterpret_cast<unsigned int*>(s_dyn + (pair & 0xFFFFu)), 1u << GBITS);
-            if (slot + 1 < cnt) atomicSub(reinterpret_cast<unsigned int*>(s_dyn + (pair >> 16)), 1u << GBITS);
-          };
-          for (int base = (tid & ~31) >> sh; base < len; base += 1024 >> sh) {
-            if (base > 0 && tid == 0) progress((unsigned int)base);
-            const unsigned int c0 = cs;
-            if (base + (1024 >> sh) < len) cs = __ldcg(J.ents + off + base + (1024 >> sh) + (lane >> sh));
-            uint4 a = make_uint4(0u, 0u, 0u, 0u);
-            if (base + (lane >> sh) < len) a = __ldcg(J.chunks + c0 + r0);  // may run past the list: spare chunks
-            const int cnt_l = (int)__shfl_sync(FULL_MASK, a.x, lane & ~(per_set - 1));  // 0: covered
-            if (r0 == 0) {
-              if (cnt_l) {
-                J.covered[a.y] = 1;
-                *reinterpret_cast<unsigned int*>(J.chunks + c0) = 0u;
-              }
-            } else {
-              lower(a.x, 8 * r0 - 4, cnt_l);
-              lower(a.y, 8 * r0 - 2, cnt_l);
+          const int base = (int)blockIdx.x * 512 + ((tid & ~31) >> 1);
+          const unsigned int cs = base < len ? __ldcg(J.ents + off + base + (lane >> 1)) : 0u;
+          cover(off, len, base, (int)gridDim.x * 512, cs, 1, false);
+        }
+        __syncthreads();
+        if (blockIdx.x != 0)
+          for (int t = tid; t < ncp; t += 1024)
+            if (s_key[t]) {
+              atomicAdd(J.cand_dec + t, (0u - s_key[t]) >> GBITS);
+              s_key[t] = 0u;
             }
-            lower(a.z, 8 * r0, cnt_l);
-            lower(a.w, 8 * r0 + 2, cnt_l);
-            // what is left of the warp's sets is dealt to the lanes chunk by chunk
-            const int rest = r0 == 0 && cnt_l > first_slots ? (cnt_l - first_slots + 7) >> 3 : 0;
-            if (!__any_sync(FULL_MASK, rest)) continue;
-            const int incl = warp_inclusive_scan(rest, lane);
-            const int total = __shfl_sync(FULL_MASK, incl, 31);
-            for (int q0 = 0; q0 < total; q0 += 32) {
-              const int q = q0 + lane;
-              int o = 0;
-#pragma unroll
-              for (int s = 16; s; s >>= 1) {
-                const int x = __shfl_sync(FULL_MASK, incl, o + s - 1);
-                if (x <= q) o += s;
-              }
-              o = o > 31 ? 31 : o;
-              const int r = q - (__shfl_sync(FULL_MASK, incl, o) - __shfl_sync(FULL_MASK, rest, o));
-              const unsigned int oc = __shfl_sync(FULL_MASK, c0, o);
-              const int ocnt = __shfl_sync(FULL_MASK, cnt_l, o);
-              if (q < total) {
-                const uint4 w = __ldcg(J.chunks + oc + per_set + r);
-                lower(w.x, first_slots + 8 * r, ocnt);
-                lower(w.y, first_slots + 8 * r + 2, ocnt);
-                lower(w.z, first_slots + 8 * r + 4, ocnt);
-                lower(w.w, first_slots + 8 * r + 6, ocnt);
-              }
+        if (!greedy_barrier<CLUSTER>(J, s_wait, [] { return 0ull; }, info)) return;
+        if (blockIdx.x == 0) {
+          for (int t = tid; t < ncp; t += 1024) {
+            const unsigned int d = __ldcg(J.cand_dec + t);
+            if (d) {
+              s_key[t] -= d << GBITS;
+              __stcg(J.cand_dec + t, 0u);
             }
+            if (t == l) s_key[t] = 0u;  // never again
           }
-          i += 1;
-          __syncthreads();
-          // never again: its owner, the only thread that reads it, takes it out
-          if (tid == (l & 1023)) s_key[l] = 0u;
         }
       }
-      // the local ids go back to 0 for the next session
-      const int64_t b0 = gridDim.x > 1 ? blockIdx.x - 1 : 0, nb = gridDim.x > 1 ? gridDim.x - 1 : 1;
-      if (b0 >= 0)
-        for (int64_t t = b0 * 1024 + tid; t < nc; t += nb * 1024) J.lid[__ldcg(J.cand_id + t)] = 0;
-      if (blockIdx.x == 0 && tid == 0) J.ncand[2] = (unsigned int)i;
-      if (!greedy_barrier<CLUSTER>(J, s_wait, [&] { return (unsigned long long)__ldcg(J.ncand + 2); }, info)) return;
-      i = (int)info;
       if (i >= J.k) break;
       if (small && i - i0 < 96) small_off = true;  // it did not pay for its lists
     }
@@ -1191,10 +1251,12 @@ int greedy_cluster_size() {
   std::lock_guard<std::mutex> lock(mu);
   if (size >= 0) return size;
   size = 0;
-  if (cudaFuncSetAttribute(k_greedy<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GREEDY_SMEM) != cudaSuccess)
-    (void)cudaGetLastError();
-  if (cudaFuncSetAttribute(k_greedy<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-    (void)cudaGetLastError();
+  for (auto* k : {k_greedy<true, false>, k_greedy<true, true>}) {
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, GREEDY_SMEM) != cudaSuccess)
+      (void)cudaGetLastError();
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+      (void)cudaGetLastError();
+  }
   for (int c : {16, 8}) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(c);
@@ -1208,7 +1270,7 @@ int greedy_cluster_size() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, k_greedy<true>, &cfg) == cudaSuccess && clusters >= 1) {
+    if (cudaOccupancyMaxActiveClusters(&clusters, k_greedy<true, true>, &cfg) == cudaSuccess && clusters >= 1) {
       size = c;
       break;
     }
@@ -1231,6 +1293,7 @@ cudaError_t launch_greedy(const GreedyJob& J, cudaStream_t st, int num_sms, bool
   const int mode = g_greedy_mode.load();
   const int csize = mode == 1 ? 0 : greedy_cluster_size();
   const unsigned long long work = (unsigned long long)J.n_pad + J.total_entries;
+  const bool share = J.total_entries >= GREEDY_SHARE_ENTRIES;
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr[1];
   cfg.blockDim = dim3(1024);
@@ -1246,7 +1309,7 @@ cudaError_t launch_greedy(const GreedyJob& J, cudaStream_t st, int num_sms, bool
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_greedy<true>, J);
+    return cudaLaunchKernelEx(&cfg, share ? k_greedy<true, true> : k_greedy<true, false>, J);
   } else {
     cfg.gridDim = dim3(num_sms);
     // a cooperative launch (all blocks resident at once), also valid inside a stream capture
@@ -1254,15 +1317,15 @@ cudaError_t launch_greedy(const GreedyJob& J, cudaStream_t st, int num_sms, bool
     attr[0].val.cooperative = 1;
     cfg.numAttrs = 1;
   }
-  const cudaError_t e =
-      cudaFuncSetAttribute(k_greedy<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, GREEDY_SMEM);
+  auto* k = share ? k_greedy<false, true> : k_greedy<false, false>;
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, GREEDY_SMEM);
   if (e != cudaSuccess) return e;
-  return cudaLaunchKernelEx(&cfg, k_greedy<false>, J);
+  return cudaLaunchKernelEx(&cfg, k, J);
 }
 
 cudaError_t device_code_version(int* binary, int* ptx) {
   cudaFuncAttributes a{};
-  const cudaError_t e = cudaFuncGetAttributes(&a, k_greedy<false>);
+  const cudaError_t e = cudaFuncGetAttributes(&a, k_greedy<false, false>);
   if (e != cudaSuccess) return e;
   *binary = a.binaryVersion;
   *ptx = a.ptxVersion;

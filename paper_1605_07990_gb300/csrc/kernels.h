@@ -216,7 +216,7 @@ struct GreedyJob {
   unsigned int* sync;           // 128 words: count [0], release word (64-bit) [32], error flag [64], progress [96]
   unsigned long long* argmax;   // 3 slots 16 words apart
   unsigned long long* nchunk;   // chunks handed out
-  unsigned int* ncand;          // candidates, chunk overflow, picks made, queued parts, list entries
+  unsigned int* ncand;          // candidates, chunk overflow, picks made, queued parts, list entries, shared pick
   unsigned int* hist;           // 4 x 1024 bins
   unsigned int* blk;            // 1024: candidates among the nodes that a block numbers
   // candidates of a session
@@ -225,6 +225,7 @@ struct GreedyJob {
   int32_t* cand_id;             // GREEDY_CANDS node ids
   int32_t* cand_len;            // gain when the lists were made = entries of the list
   unsigned int* cand_off;       // first entry of the candidate's list
+  unsigned int* cand_dec;       // what the other blocks' shares of a pick take off the candidate's gain; zero between launches
   unsigned int* ents;           // ents_cap (+ GREEDY_ENTS_SPARE) first chunks of the candidates' sets
   long long ents_cap;
   uint4* chunks;                // chunk_cap (+ GREEDY_CHUNKS_SPARE) chunks of the sets' candidates
@@ -253,6 +254,13 @@ long long greedy_wait_polls();
 // others and a pool of up to GREEDY_CLUSTER_ENTRIES entries, one thread-block
 // cluster.
 constexpr unsigned long long GREEDY_CLUSTER_ENTRIES = 1ull << 26;
+// Pools of this many entries and more share the sets of heavy picks between the
+// blocks.  max_coverage on GB300, ms, one block's alone / shared: 820,000 LT sets of
+// the 2^17-node R-MAT graph (25M entries) k = 20 4.35 / 1.00, k = 100 7.6 / 2.1; 1.9M
+// of the 2^20-node one (75M) k = 100 13.1 / 2.7; 820,000 IC sets (12M) k = 100 2.40 /
+// 1.68.  Below, few lists are that long, and the turns cost: 130,000 LT sets of the
+// 2^22-node graph (5.7M) k = 1000 2.71 / 2.82, 268,000 IC sets (5.9M) 1.65 / 1.67.
+constexpr unsigned long long GREEDY_SHARE_ENTRIES = 1ull << 23;
 cudaError_t launch_greedy(const GreedyJob& J, cudaStream_t st, int num_sms, bool shared_gpu);
 // 0: by the rule above (default); 1: always the cooperative grid; 2: always a cluster (when the device has one)
 void set_greedy_mode(int mode);
