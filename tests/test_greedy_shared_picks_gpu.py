@@ -1,7 +1,8 @@
 """Max-Coverage picks whose lists are so long that every block covers a share of
 them (4,096 sets and more of pools of 2^23 entries and more), against the oracle
 (exact): sets that overlap under many heavy picks, sets that one pick covers
-whole, lists of just under and over that length, under each launch shape."""
+whole, lists of just under and over that length, picks of more sets than a
+session's keys hold, under each launch shape."""
 import numpy as np
 import pytest
 
@@ -29,6 +30,9 @@ CASES = {
     "ic_overlap": (inputs.rmat(13, 1 << 17, seed=6), oracle.W_WC, oracle.IC, 1_200_000, (30, 300)),
     "whole": (_teeth(24, 50), oracle.W_EXPLICIT, oracle.IC, 500_000, (23, 24, 25, 1200)),
     "threshold": (_teeth(147, 40), oracle.W_EXPLICIT, oracle.IC, 602_000, (60, 147)),  # about 4,095 sets a tooth
+    # several picks of more sets (2^18) than a session's keys hold
+    "wide": (_teeth(6, 8), oracle.W_EXPLICIT, oracle.IC, 2_900_003, (5, 6, 48)),
+    "wide_overlap": (inputs.rmat(9, 1 << 12, seed=5), oracle.W_WC, oracle.LT, 2_500_001, (2, 3, 30)),
 }
 
 
